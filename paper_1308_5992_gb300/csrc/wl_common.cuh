@@ -249,6 +249,7 @@ struct LevelOps {
   DBuf A;    // stencil [n][9][2][2]
   DBuf den;  // Kaczmarz denominators ||A e_i||^2, [n][2] (real, T)
   DBuf P;    // interpolation weights to the next level [n][2][4]
+  DBuf rows; // packed tile rows of the row-block sweep (wl_rows.cu), made on first use
 };
 
 // launch form of a Kaczmarz sweep on one level, chosen by the autotuner
@@ -268,6 +269,7 @@ struct Level {
   // cycle work vectors, [n][2][nrhs_cap] in the cycle precision
   DBuf x, r, f, t;
   std::vector<KTune> tune;    // autotuned sweep forms per (nrhs, precision)
+  std::vector<KTune> rowtune; // where the row-block sweep measured faster: form 4, param = R | RPT << 8
 };
 
 struct wl_amg {
@@ -298,6 +300,7 @@ struct wl_amg {
   // second solve lane (amg_params.overlap): a hierarchy that views this one's
   // operators and has its own stream, workspace and graphs; created on demand
   wl_amg *twin = nullptr;
+  bool is_twin = false;  // this object is such a second lane
 };
 
 // --------------------------------------------------------- internal C++ API
@@ -329,6 +332,13 @@ int kaczmarz_colour(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int 
 int kaczmarz_tile(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int tc, cudaStream_t s, int R = 0);
 int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s);  // every level but the coarsest
 int tile_timeout_take(cudaStream_t s);  // 1 if a tile launch's bounded wait ran out (flag cleared)
+int *tile_timeout_flag();               // device address of that flag on the current device
+// row-block form of the tile-coloured sweep (wl_rows.cu): FP32 and BF16 cycles
+bool rows_ok(const wl_amg *a, int l, int prec, int nrhs);
+bool rows_form_exists(const wl_amg *a, int l, int prec, int param);
+int rows_candidates(int nrhs, int *out);  // launch parameters worth timing (at most 8)
+int rows_prepare(wl_amg *a, int l, int prec, cudaStream_t s);
+int rows_sweeps(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int sweeps, int param, cudaStream_t s);
 KTune sweep_form_of(wl_amg *a, int l, int prec, int nrhs);
 int restrict_op(wl_amg *a, int l, int prec, const void *r, void *fc, int nrhs, cudaStream_t s);
 int prolong_op(wl_amg *a, int l, int prec, const void *e, void *x, int nrhs, cudaStream_t s);
@@ -356,9 +366,10 @@ __device__ __forceinline__ unsigned long long gtimer() {
 }
 
 // wait for the completion of the mbarrier phase of the given parity, at most
-// `ns` nanoseconds (the timer is read once per 32 polls); false on timeout
+// `ns` nanoseconds (the timer is read once per 32 polls, first after the
+// first 32); false on timeout
 __device__ __forceinline__ bool mbar_wait(uint32_t mb, uint32_t parity, unsigned long long ns) {
-  unsigned long long t0 = gtimer();
+  unsigned long long t0 = 0;
   for (;;) {
     for (int i = 0; i < 32; ++i) {
       uint32_t done;
@@ -369,7 +380,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mb, uint32_t parity, unsigned
           : "memory");
       if (done) return true;
     }
-    if (gtimer() - t0 > ns) return false;
+    unsigned long long t = gtimer();
+    if (!t0) t0 = t;
+    else if (t - t0 > ns) return false;
   }
 }
 

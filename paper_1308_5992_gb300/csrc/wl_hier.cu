@@ -368,6 +368,7 @@ wl_amg *make_twin(wl_amg *a) {
   t->cap = 0;
   t->cap_prec = a->cap_prec;
   t->h_small = nullptr;
+  t->is_twin = true;
   return t;
 }
 
@@ -386,6 +387,7 @@ void amg_free(wl_amg *a) {
       o->A.release();
       o->den.release();
       o->P.release();
+      o->rows.release();
     }
     L.x.release();
     L.r.release();

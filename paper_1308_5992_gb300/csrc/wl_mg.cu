@@ -1326,6 +1326,19 @@ int tile_timeout_take(cudaStream_t s) {
   return v;
 }
 
+// device address of g_tile_timeout (looked up once per device)
+int *tile_timeout_flag() {
+  static std::atomic<int *> cached[WL_MAX_DEVICES];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= WL_MAX_DEVICES) return nullptr;
+  int *p = cached[dev].load(std::memory_order_acquire);
+  if (!p) {
+    if (cudaGetSymbolAddress((void **)&p, g_tile_timeout) != cudaSuccess) return nullptr;
+    cached[dev].store(p, std::memory_order_release);
+  }
+  return p;
+}
+
 // shared memory of the persistent form: two r buffers, step scales, the
 // stencil-row ring, the site-index table and two mbarriers
 template <typename T, typename S>
@@ -1525,6 +1538,22 @@ int kaczmarz_sweeps(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int 
   return run_sweeps(a, l, prec, x, r, nrhs, sweeps, sweep_form_of(a, l, prec, nrhs), s);
 }
 
+// the sweeps of a cycle: the row-block form where it measured faster, unless
+// the launch form is explicit (sweep_kernel) or pinned; per-step calls
+// (amg_kaczmarz) keep kaczmarz_sweeps, whose forms agree bit for bit
+static int cycle_sweeps(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int sweeps, cudaStream_t s) {
+  const Level &L = a->lev[l];
+  if (sweeps <= 0) return WL_OK;
+  if (a->prm.sweep_kernel == 0 && rows_ok(a, l, prec, nrhs)) {
+    bool pinned = false;
+    for (const KTune &k : L.tune) pinned |= k.nrhs == nrhs && k.prec == prec && k.us == 0.f;
+    if (!pinned)
+      for (const KTune &k : L.rowtune)
+        if (k.nrhs == nrhs && k.prec == prec) return rows_sweeps(a, l, prec, x, r, nrhs, sweeps, k.param, s);
+  }
+  return kaczmarz_sweeps(a, l, prec, x, r, nrhs, sweeps, s);
+}
+
 // Autotuner: time every launch form of one sweep on each level (the level's
 // own cycle buffers, whose contents the next cycle overwrites) and keep the
 // fastest.  Candidates: per-colour launches and the cooperative launch at
@@ -1577,13 +1606,22 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
           if (!dup) cand.push_back(KTune{nrhs, prec, 1, b, 0.f});
         }
     }
-    KTune best = cand[0];
+    if (rows_ok(a, l, prec, nrhs)) {
+      if ((rc = rows_prepare(a, l, prec, s))) break;
+      int prm[8], n = rows_candidates(nrhs, prm);
+      for (int i = 0; i < n; ++i) cand.push_back(KTune{nrhs, prec, 4, prm[i], 0.f});
+    }
+    KTune best = cand[0], rows{nrhs, prec, 4, 0, 1e30f};
     float best_us = 1e30f;
+    auto sweep = [&](const KTune &c) -> int {
+      return c.form == 4 ? rows_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c.param, s)
+                         : run_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c, s);
+    };
     for (KTune &c : cand) {
-      rc = run_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c, s);  // warm-up
+      rc = sweep(c);  // warm-up
       if (rc) break;
       if ((rc = (cudaEventRecord(e0, s) == cudaSuccess) ? WL_OK : WL_ECUDA)) break;
-      for (int rep = 0; rep < 3 && rc == WL_OK; ++rep) rc = run_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c, s);
+      for (int rep = 0; rep < 3 && rc == WL_OK; ++rep) rc = sweep(c);
       if (rc) break;
       float ms = 0;
       if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
@@ -1592,12 +1630,17 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
         break;
       }
       c.us = ms * 1e3f / 3;
-      if (c.us < best_us) {
+      if (c.form == 4) {
+        if (c.us < rows.us) rows = c;
+      } else if (c.us < best_us) {
         best_us = c.us;
         best = c;
       }
     }
-    if (rc == WL_OK) L.tune.push_back(best);
+    if (rc == WL_OK) {
+      L.tune.push_back(best);
+      if (rows.us < best_us) L.rowtune.push_back(rows);
+    }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1681,7 +1724,7 @@ static int cycle_level(wl_amg *a, int l, int nrhs, int prec, cudaStream_t s) {
   if (l == a->L - 1) return coarsest_apply(a, prec, L.f.p, L.x.p, nrhs, s);
   WL_CUDA(cudaMemsetAsync(L.x.p, 0, vb, s));
   WL_CUDA(cudaMemcpyAsync(L.r.p, L.f.p, vb, cudaMemcpyDeviceToDevice, s));
-  WL_TRY(kaczmarz_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, a->prm.nu_pre, s));
+  WL_TRY(cycle_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, a->prm.nu_pre, s));
   Level &C = a->lev[l + 1];
   WL_TRY(restrict_op(a, l, prec, L.r.p, C.f.p, nrhs, s));
   int gamma = (a->prm.cycle == WL_CYCLE_W) ? 2 : 1;
@@ -1703,7 +1746,7 @@ static int cycle_level(wl_amg *a, int l, int nrhs, int prec, cudaStream_t s) {
   }
   WL_TRY(prolong_op(a, l, prec, C.x.p, L.x.p, nrhs, s));
   WL_TRY(stencil_apply(a, l, prec, L.x.p, L.r.p, L.f.p, nrhs, s));
-  WL_TRY(kaczmarz_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, a->prm.nu_post, s));
+  WL_TRY(cycle_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, a->prm.nu_post, s));
   return WL_OK;
 }
 
@@ -1816,7 +1859,8 @@ static int kaczmarz_entry(wl_amg *a, int level, void *x, void *r, int nrhs, int 
     wl_set_error("%s: invalid argument (the coarsest level is not relaxed)", who);
     return WL_EINVAL;
   }
-  if (form >= 0 && !form_exists(a, level, nrhs, prec, form, param)) {
+  const bool rows = form == 4 && level < a->L - 1 && wl::rows_form_exists(a, level, prec, param);
+  if (form >= 0 && !rows && !form_exists(a, level, nrhs, prec, form, param)) {
     wl_set_error("%s: launch form %d / %d does not exist for this level and ordering", who, form, param);
     return WL_EINVAL;
   }
@@ -1831,6 +1875,9 @@ static int kaczmarz_entry(wl_amg *a, int level, void *x, void *r, int nrhs, int 
   WL_TRY(wl::to_internal((const zd *)r, sb.b[1].p, n2, nrhs, pin, s));
   if (form < 0) {
     WL_TRY(wl::kaczmarz_sweeps(a, level, prec, sb.b[0].p, sb.b[1].p, nrhs, sweeps, s));
+  } else if (rows) {
+    WL_TRY(wl::rows_prepare(a, level, prec, s));
+    WL_TRY(wl::rows_sweeps(a, level, prec, sb.b[0].p, sb.b[1].p, nrhs, sweeps, param, s));
   } else if (sweeps > 0) {
     KTune t{nrhs, prec, form, param, 0.f};
     WL_TRY(wl::run_sweeps(a, level, prec, sb.b[0].p, sb.b[1].p, nrhs, sweeps, t, s));
@@ -1849,7 +1896,7 @@ extern "C" int amg_kaczmarz(wl_amg *a, int level, void *x, void *r, int nrhs, in
 extern "C" int amg_kaczmarz_form(wl_amg *a, int level, void *x, void *r, int nrhs, int sweeps, int prec, int form,
                                  int param) {
   if (form < 0) {
-    wl_set_error("amg_kaczmarz_form: form must be 0, 1 or 2");
+    wl_set_error("amg_kaczmarz_form: form must be 0 to 4");
     return WL_EINVAL;
   }
   return kaczmarz_entry(a, level, x, r, nrhs, sweeps, prec, form, param, "amg_kaczmarz_form");

@@ -1,0 +1,458 @@
+// wl_rows.cu -- row-block form of the tile-coloured Kaczmarz sweep (Sec. 3.1)
+// for the FP32 and BF16-stored cycles.
+//
+// A sweep relaxes one unknown after the other: s_i = omega <r, A e_i> / den_i,
+// x_i += s_i, r -= s_i A e_i.  For a block of unknowns taken in order this is
+// the same as forming every <r, A e_i> from the r the block starts with and
+// then solving a small triangular system, since
+//   <r - sum_{j<i} s_j A e_j, A e_i> = <r, A e_i> - sum_{j<i} K_ij s_j,
+//   K_ij = <A e_j, A e_i>,
+// so s = T (<r, A e_i>)_i with T = (den / omega on the diagonal, K below)^-1,
+// a constant of the level.  Here a block is one row of a tile (8 sites, 16
+// unknowns): the 16 dependent colour steps of a tile become 4 row steps (rows
+// i and i + 4 at once, which share no cell of r), at the cost of the product
+// with T, 12 of 48 complex multiply-adds per unknown.  T is formed in FP64
+// from the stored stencil and rounded once.
+//
+// Within a row the order is that of wl_tile_order.h: even rows 0 1 2 3, odd
+// rows 3 2 1 0 in each 4-site cell, both cells at once.  Two sites couple when
+// at most two columns apart, so a cell needs its own 8 inner products and, for
+// the left cell of an even row (the right cell of an odd one), 4 of the other
+// cell: T has 12 columns.
+#include <algorithm>
+#include <atomic>
+
+#include "wl_common.cuh"
+#include "wl_tile_order.h"
+
+#define RB_KT 8
+#define RB_W 10    // window side: tile and halo
+#define RB_RS 209  // complex floats between the r windows of two right-hand sides in shared memory:
+                   // 200 used; 2 * 209 = 2 (mod 32) puts consecutive right-hand sides in
+                   // consecutive bank pairs for the transposing copies
+
+// bytes of one row step of a packed tile: per lane the stencil entries of its
+// site for its spin (9 offsets x 2 rows) and its row of T (12 entries)
+template <typename S>
+__host__ __device__ constexpr int rb_step_bytes() {
+  return 32 * (9 * 2 * (int)sizeof(S) + 12 * (int)sizeof(zf));
+}
+
+__device__ __forceinline__ int rb_site(const Geo &g, int A0, int B0, int i, int j) {
+  int a = A0 + i, b = B0 + j;
+  return g.idx(a + b, a - b);
+}
+
+// tile `t` of tile colour tc: its origin
+__device__ __forceinline__ void rb_origin(const Geo &g, int tc, int t, int &A0, int &B0) {
+  int nb4 = g.N / (4 * RB_KT);
+  A0 = ((tc & 1) + 2 * (t / nb4)) * RB_KT;
+  B0 = ((tc >> 1) + 2 * (t % nb4)) * RB_KT;
+}
+
+// K = <A e_(h2,t2), A e_(h,t)> for sites h, h2 of one row, h2 = h + delta
+// columns (|delta| <= 2): column (h, t) has the entries g_s g_t conj(A[h][d][t][s])
+template <typename S>
+__device__ zd rb_gram(const S *__restrict__ A, int h, int t, int h2, int t2, int delta) {
+  zd k = mk(0.0, 0.0);
+  for (int da = 0; da < 3; ++da)
+    for (int db = 0; db < 3; ++db) {
+      int eb = db - delta;  // the same cell seen from h2
+      if (eb < 0 || eb > 2) continue;
+      const S *p = A + ((long)h * 9 + da * 3 + db) * 4 + t * 2;
+      const S *q = A + ((long)h2 * 9 + da * 3 + eb) * 4 + t2 * 2;
+      for (int s = 0; s < 2; ++s) k = k + widen<double>(ld<float>(p + s)) * cconj(widen<double>(ld<float>(q + s)));
+    }
+  double f = (t ^ t2) ? -1.0 : 1.0;
+  return mk(f * k.re, f * k.im);
+}
+
+// 16 threads per cell of 4 sites: its stencil entries and rows of T, packed in
+// the lane order of k_kacz_rows ([tile colour][tile][step][9 + 6][32 lanes]).
+// Thread i < 12 forms row i of the block's matrix (in the order of
+// relaxation), then column i of its inverse by forward substitution.
+#define RBP_CELLS 8
+template <typename S>
+__global__ void __launch_bounds__(16 * RBP_CELLS) k_rows_pack(Geo g, const S *__restrict__ A, double omega,
+                                                              unsigned char *__restrict__ out) {
+  __shared__ zd Ms[RBP_CELLS][12][13];
+  const int ntile = (g.N / (2 * RB_KT)) * (g.N / (4 * RB_KT));
+  const int lc = threadIdx.x >> 4, i = threadIdx.x & 15;
+  const int id = blockIdx.x * RBP_CELLS + lc;  // 16 cells a tile: the grid is exact
+  const int cell = id & 1, grp = (id >> 1) & 1, step = (id >> 2) & 3, tile = id >> 4;  // tile counts through the colours
+  int A0, B0;
+  rb_origin(g, tile / ntile, tile % ntile, A0, B0);
+  const int row = step + 4 * grp;
+  const bool rev = step & 1;
+  const bool dep = cell == (rev ? 1 : 0);  // needs the other cell's first two sites
+  // site v = 0..5 of the order of relaxation: own sites, and the other cell's
+  // first two after the own ones of the same colour (in a cell that needs no
+  // other site v = 4, 5 are unused: unit rows)
+  auto column = [&](int v) -> int {
+    if (!dep) return v < 4 ? cell * 4 + (rev ? 3 - v : v) : -1;
+    const int u = v < 4 ? v >> 1 : v - 2, j = rev ? 3 - u : u;  // own, other, own, other, own, own
+    return ((v < 4 && (v & 1)) ? 1 - cell : cell) * 4 + j;
+  };
+  if (i < 12) {
+    const int p = i >> 1, t = i & 1, cp = column(p);
+    for (int q = 0; q < 6; ++q) {
+      const int cq = column(q), dl = cq - cp;
+      for (int t2 = 0; t2 < 2; ++t2) {
+        zd k = mk(0.0, 0.0);
+        if (2 * q + t2 <= i) {
+          if (cp < 0 || cq < 0) {
+            if (2 * q + t2 == i) k = mk(1.0, 0.0);
+          } else if (dl >= -2 && dl <= 2) {
+            k = rb_gram(A, rb_site(g, A0, B0, row, cp), t, rb_site(g, A0, B0, row, cq), t2, dl);
+            if (2 * q + t2 == i) k = mk(k.re / omega, 0.0);
+          }
+        }
+        Ms[lc][i][2 * q + t2] = k;
+      }
+    }
+  }
+  __syncthreads();
+  unsigned char *so = out + ((long)tile * 4 + step) * rb_step_bytes<S>();
+  S *oa = (S *)so;
+  zf *ot = (zf *)(so + 32 * 18 * sizeof(S));
+  if (i < 12) {
+    const int cq = column(i >> 1), kq = cq < 0 ? 0 : cq / 4 == cell ? 2 * (cq & 3) + (i & 1)
+                                       : 8 + 2 * (rev ? (cq & 3) - 2 : (cq & 3)) + (i & 1);  // this column of T
+    zd X[12];
+#pragma unroll
+    for (int r = 0; r < 12; ++r) {
+      zd v = mk(r == i ? 1.0 : 0.0, 0.0);
+#pragma unroll
+      for (int q = 0; q < r; ++q) v = v - Ms[lc][r][q] * X[q];
+      double d = Ms[lc][r][r].re;
+      X[r] = mk(v.re / d, v.im / d);
+      const int cr = column(r >> 1);
+      if (cq >= 0 && cr >= 0 && cr / 4 == cell)
+        ot[((kq >> 1) * 32 + grp * 16 + cr * 2 + (r & 1)) * 2 + (kq & 1)] = ccast<float>(X[r]);
+    }
+  }
+  if (!dep)  // the columns of the other cell's sites
+    for (int e = i; e < 32; e += 16) {
+      int u = e >> 2, k = 8 + (e & 3);
+      ot[((k >> 1) * 32 + grp * 16 + cell * 8 + u) * 2 + (k & 1)] = mk(0.f, 0.f);
+    }
+  for (int e = i; e < 4 * 36; e += 16) {
+    int b = cell * 4 + e / 36, c = e % 36, d = c >> 2, t = (c >> 1) & 1, p = c & 1;
+    oa[(d * 32 + grp * 16 + b * 2 + p) * 2 + t] = A[(long)rb_site(g, A0, B0, row, b) * 36 + c];
+  }
+}
+
+// stencil entries (rows t = 0 and 1) of one offset, or two entries of T
+__device__ __forceinline__ void rb_ld(const zf *p, float2 &a0, float2 &a1) {
+  float4 v = *(const float4 *)p;
+  a0 = make_float2(v.x, v.y);
+  a1 = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void rb_ld(const zb *p, float2 &a0, float2 &a1) {
+  uint2 u = *(const uint2 *)p;
+  a0 = __bfloat1622float2(*(const __nv_bfloat162 *)&u.x);
+  a1 = __bfloat1622float2(*(const __nv_bfloat162 *)&u.y);
+}
+__device__ __forceinline__ float2 rb_swap(float2 v) { return make_float2(v.y, v.x); }
+__device__ __forceinline__ float2 rb_shfl_xor1(float2 v) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, 1), __shfl_xor_sync(0xffffffffu, v.y, 1));
+}
+
+// One tile colour (a quarter of a sweep): a block per tile and chunk of R
+// right-hand sides, a warp per RPT of them.  Lane (row group, column b, spin
+// p) = (lane / 16, (lane / 2) % 8, lane % 2) forms the partial products of its
+// site's two unknowns over the nine cells of spin p, the pair of lanes of a
+// site swaps halves, the 12 inner products a row of T needs go through shared
+// memory, and the update of r is summed per column with the neighbours' parts
+// taken by shuffles.  A warp never waits for another one between the first
+// and the last barrier; its RPT right-hand sides go through each phase
+// together, so that their latencies overlap.  Complex products are paired
+// FMAs on (re, im) pairs as they lie in memory: sum (a.re x.re, a.im x.im) and
+// sum (a.re x.im, a.im x.re), combined once per sum.  The tile's packed rows
+// arrive as one bulk copy per row step, all four issued at the start (bounded
+// waits; on a timeout *timeout gets 1 and nothing is written).
+template <typename S, int R, int RPT>
+__global__ void __launch_bounds__(32 * R / RPT, RPT == 1 ? 16 / R : 0) k_kacz_rows(Geo g, int tc, const unsigned char *__restrict__ pk,
+                                                            zf *__restrict__ x, zf *__restrict__ r, int nrhs,
+                                                            int *timeout) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  constexpr int NT = 32 * R / RPT, NW = R / RPT, SB = rb_step_bytes<S>();
+  unsigned char *cs = sm_raw;                           // [4][SB] packed rows
+  float2 *rs = (float2 *)(sm_raw + 4 * SB);             // [R][RB_RS] r of tile + halo, [site][spin]
+  float2 *nums = rs + ((R * RB_RS + 1) & ~1);           // [NW][RPT][2][20] inner products
+  int *hs = (int *)(nums + R * 40);                     // [100] site index of tile + halo
+  uint64_t *mbar = (uint64_t *)(hs + RB_W * RB_W);      // [4], 8-byte aligned: every part above is a multiple of 8
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int ntile = (g.N / (2 * RB_KT)) * (g.N / (4 * RB_KT));
+  const int r0 = blockIdx.y * R, Rc = min(R, nrhs - r0);
+  int A0, B0;
+  rb_origin(g, tc, blockIdx.x, A0, B0);
+  if (tid == 0) {
+    for (int i = 0; i < 4; ++i) mbar_init(smem_u32(&mbar[i]), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    const unsigned char *src = pk + ((long)tc * ntile + blockIdx.x) * 4 * SB;
+    for (int i = 0; i < 4; ++i) {
+      mbar_arrive_expect_tx(smem_u32(&mbar[i]), SB);
+      bulk_g2s(smem_u32(cs + i * SB), src + i * SB, SB, smem_u32(&mbar[i]));
+    }
+  }
+  for (int ls = tid; ls < RB_W * RB_W; ls += NT) hs[ls] = rb_site(g, A0, B0, ls / RB_W - 1, ls % RB_W - 1);
+  __syncthreads();
+  // this thread's elements of the window, in global and in shared memory
+  constexpr int NE = (RB_W * RB_W * 2 * R + NT - 1) / NT;
+  float2 *ga[NE];
+#pragma unroll
+  for (int i = 0; i < NE; ++i) {
+    int e = tid + i * NT, q = e % R, row = e / R;
+    bool in = e < RB_W * RB_W * 2 * R && q < Rc;
+    ga[i] = in ? (float2 *)r + ((long)hs[row >> 1] * 2 + (row & 1)) * nrhs + r0 + q : nullptr;
+  }
+  const int grp = lane >> 4, b = (lane >> 1) & 7, p = lane & 1;
+  const int q0 = w * RPT;
+  bool act[RPT];
+#pragma unroll
+  for (int m = 0; m < RPT; ++m) act[m] = q0 + m < Rc;
+  float2 *xa[4];  // x of this lane's unknown in the four row steps
+#pragma unroll
+  for (int st = 0; st < 4; ++st)
+    xa[st] = (float2 *)x + ((long)hs[(st + 4 * grp + 1) * RB_W + b + 1] * 2 + p) * nrhs + r0 + q0;
+  // r and x are the previous launch's
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+#pragma unroll
+  for (int i = 0; i < NE; ++i) {
+    int e = tid + i * NT;
+    if (ga[i])
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_u32(rs + (e % R) * RB_RS + e / R)),
+                   "l"(ga[i]));
+  }
+  float2 xp[4][RPT];
+#pragma unroll
+  for (int st = 0; st < 4; ++st)
+#pragma unroll
+    for (int m = 0; m < RPT; ++m)
+      if (act[m]) xp[st][m] = xa[st][m];
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  __syncthreads();
+  const bool edge = b == 0 || b == 7;
+  const int eo = b == 0 ? 0 : 4;  // the halo column an edge lane also updates, from its own column - 1
+  const float ml = b == 0 ? 0.f : 1.f, mr = b == 7 ? 0.f : 1.f;
+  float2 *nw = nums + w * RPT * 40 + grp * 20;
+  const int own = (b >> 2) * 8;
+  bool ok = true;
+#pragma unroll
+  for (int st = 0; st < 4; ++st) {
+    ok = ok && mbar_wait(smem_u32(&mbar[st]), 0, 1000000000ull);
+    if (!__all_sync(0xffffffffu, ok)) {
+      ok = false;
+      break;
+    }
+    float2 a0[9], a1[9], T[12];
+    const S *ca = (const S *)(cs + st * SB);
+    const zf *ct = (const zf *)(cs + st * SB + 32 * 18 * sizeof(S));
+#pragma unroll
+    for (int d = 0; d < 9; ++d) rb_ld(ca + (d * 32 + lane) * 2, a0[d], a1[d]);
+    float2 *rq = rs + q0 * RB_RS + ((st + 4 * grp) * RB_W + b) * 2 + p;
+    float2 rc[RPT][3], re[RPT][3];  // own column and, on edge lanes, the halo column beside it
+#pragma unroll
+    for (int m = 0; m < RPT; ++m) {
+      float2 d0 = make_float2(0.f, 0.f), d1 = d0, e0 = d0, e1 = d0;
+#pragma unroll
+      for (int d = 0; d < 9; ++d) {
+        float2 v = rq[m * RB_RS + ((d / 3) * RB_W + d % 3) * 2], vs = rb_swap(v);
+        d0 = __ffma2_rn(a0[d], v, d0);
+        e0 = __ffma2_rn(a0[d], vs, e0);
+        d1 = __ffma2_rn(a1[d], v, d1);
+        e1 = __ffma2_rn(a1[d], vs, e1);
+        if (d % 3 == 1) rc[m][d / 3] = v;
+        if (d % 3 == 0) re[m][d / 3] = v;
+        if (d % 3 == 2 && b == 7) re[m][d / 3] = v;
+      }
+      float2 P0 = make_float2(d0.x - d0.y, e0.x + e0.y), P1 = make_float2(d1.x - d1.y, e1.x + e1.y);
+      float2 mine = p ? P1 : P0, recv = rb_shfl_xor1(p ? P0 : P1);
+      nw[m * 40 + b * 2 + p] = make_float2(mine.x - recv.x, mine.y - recv.y);
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) rb_ld(ct + (k * 32 + lane) * 2, T[2 * k], T[2 * k + 1]);
+    __syncwarp();
+    const int oth = (st & 1) ? 4 : 8;  // the 4 inner products beside the own cell's 8
+    float2 m0[RPT], m1[RPT];
+#pragma unroll
+    for (int m = 0; m < RPT; ++m) {
+      float2 d0 = make_float2(0.f, 0.f), e0 = d0, d1 = d0, e1 = d0;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        float4 v = *(const float4 *)(nw + m * 40 + (k < 4 ? own + 2 * k : oth + 2 * (k - 4)));
+        d0 = __ffma2_rn(T[2 * k], make_float2(v.x, v.y), d0);
+        e0 = __ffma2_rn(T[2 * k], make_float2(v.y, v.x), e0);
+        d1 = __ffma2_rn(T[2 * k + 1], make_float2(v.z, v.w), d1);
+        e1 = __ffma2_rn(T[2 * k + 1], make_float2(v.w, v.z), e1);
+      }
+      float2 s = make_float2((d0.x - d0.y) + (d1.x - d1.y), (e0.x + e0.y) + (e1.x + e1.y));
+      if (act[m]) xa[st][m] = make_float2(xp[st][m].x + s.x, xp[st][m].y + s.y);
+      float2 so = rb_shfl_xor1(s);
+      // r_(d,p) -= g_p sum_t g_t s_t conj(a[d][t][p])
+      m0[m] = p ? make_float2(-so.x, -so.y) : s;
+      m1[m] = p ? s : make_float2(-so.x, -so.y);
+    }
+#pragma unroll
+    for (int m = 0; m < RPT; ++m) {
+      float2 dl[9], n0 = rb_swap(m0[m]), n1 = rb_swap(m1[m]);
+#pragma unroll
+      for (int d = 0; d < 9; ++d) {  // m0 conj(a0) + m1 conj(a1)
+        float2 u = __ffma2_rn(a1[d], m1[m], __fmul2_rn(a0[d], m0[m]));
+        float2 v = __ffma2_rn(a1[d], n1, __fmul2_rn(a0[d], n0));
+        dl[d] = make_float2(u.x + u.y, v.x - v.y);
+      }
+      float2 up[3], dn[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        up[i] = make_float2(__shfl_up_sync(0xffffffffu, dl[i * 3 + 2].x, 2, 16),
+                            __shfl_up_sync(0xffffffffu, dl[i * 3 + 2].y, 2, 16));
+        dn[i] = make_float2(__shfl_down_sync(0xffffffffu, dl[i * 3].x, 2, 16),
+                            __shfl_down_sync(0xffffffffu, dl[i * 3].y, 2, 16));
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        float2 v = dl[i * 3 + 1];
+        v = __ffma2_rn(up[i], make_float2(ml, ml), v);
+        v = __ffma2_rn(dn[i], make_float2(mr, mr), v);
+        rq[m * RB_RS + (i * RB_W + 1) * 2] = make_float2(rc[m][i].x - v.x, rc[m][i].y - v.y);
+      }
+      if (edge) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          float2 v = b == 0 ? dl[i * 3] : dl[i * 3 + 2];
+          rq[m * RB_RS + i * RB_W * 2 + eo] = make_float2(re[m][i].x - v.x, re[m][i].y - v.y);
+        }
+      }
+    }
+    __syncwarp();
+  }
+  if (!__syncthreads_and(ok)) {
+    if (tid == 0) atomicExch(timeout, 1);
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < NE; ++i) {
+    int e = tid + i * NT;
+    if (ga[i]) *ga[i] = rs[(e % R) * RB_RS + e / R];
+  }
+}
+
+namespace wl {
+
+int *tile_timeout_flag();
+
+template <typename S, int R, int RPT>
+static int launch_rows(const Level &L, const LevelOps &o, int tc, void *x, void *r, int nrhs, int pdl, cudaStream_t s) {
+  constexpr int NW = R / RPT;
+  size_t smem = (size_t)4 * rb_step_bytes<S>() + sizeof(zf) * ((R * RB_RS + 1) & ~1) + sizeof(zf) * R * 40 +
+                sizeof(int) * RB_W * RB_W + 4 * sizeof(uint64_t);
+  static std::atomic<unsigned long long> done{0};
+  int dev = 0;
+  WL_CUDA(cudaGetDevice(&dev));
+  unsigned long long bit = 1ull << (dev & 63);
+  if (!(done.load(std::memory_order_acquire) & bit)) {
+    WL_CUDA(cudaFuncSetAttribute(k_kacz_rows<S, R, RPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    done.fetch_or(bit, std::memory_order_acq_rel);
+  }
+  int *flag = tile_timeout_flag();
+  if (!flag) return WL_ECUDA;
+  dim3 grid((L.N / (2 * RB_KT)) * (L.N / (4 * RB_KT)), (nrhs + R - 1) / R);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(32 * NW);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = pdl;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  WL_CUDA(cudaLaunchKernelEx(&cfg, k_kacz_rows<S, R, RPT>, L.geo, tc, (const unsigned char *)o.rows.p, (zf *)x, (zf *)r,
+                             nrhs, flag));
+  return WL_OK;
+}
+
+template <typename S>
+static int rows_tile(const Level &L, const LevelOps &o, int tc, void *x, void *r, int nrhs, int param, int pdl,
+                     cudaStream_t s) {
+  switch (param) {
+#define RB_CASE(R, RPT) \
+  case R | RPT << 8: return launch_rows<S, R, RPT>(L, o, tc, x, r, nrhs, pdl, s);
+    RB_CASE(1, 1) RB_CASE(2, 1) RB_CASE(4, 1) RB_CASE(8, 1) RB_CASE(8, 2)
+#undef RB_CASE
+    default: wl_set_error("internal: no row-block form %d", param); return WL_EINVAL;
+  }
+}
+
+// the launch parameters (R | RPT << 8) worth timing for nrhs right-hand sides
+int rows_candidates(int nrhs, int *out) {
+  int n = 0;
+  if (nrhs <= 2) out[n++] = 1 | 1 << 8;
+  if (nrhs >= 2) out[n++] = 2 | 1 << 8;
+  if (nrhs >= 3) out[n++] = 4 | 1 << 8;
+  if (nrhs >= 5) {
+    out[n++] = 8 | 1 << 8;
+    out[n++] = 8 | 2 << 8;
+  }
+  return n;
+}
+
+// Which sweeps may take the row-block form.  Two concurrent lanes fill the GPU
+// between them, so there the work of a sweep counts and not its latency: with
+// the row form (about twice the instructions of k_kacz_tile, a third of its
+// dependent steps) on level 1 the 512x512 step of 64 right-hand sides took
+// 145.0 ms instead of 143.7, although that level's sweep alone takes 21
+// instead of 41.7 us.
+bool rows_ok(const wl_amg *a, int l, int prec, int nrhs) {
+  // A launch relaxes a quarter of the level's tiles for every right-hand side.
+  // Measured per sweep, row form against the best other one: 512x512 (512 tiles
+  // a launch) 16 against 58 us for 1 right-hand side, 34 against 46 us for 4,
+  // 52 against 54 us for 5; 256x256 (128 tiles) 57 against 70 us for 16;
+  // 128x128 (32 tiles) 11 against 41.7 us for 1, 20 against 41.7 us for 32.
+  const Level &L = a->lev[l];
+  if ((long)L.n / 256 * nrhs > 2048) return false;
+  return !a->is_twin && !(a->prm.overlap && nrhs >= 16) && prec != WL_FP64 && a->prm.kacz_order == 1 && l < a->L - 1 && L.N >= 64 && L.N % (4 * RB_KT) == 0 &&
+         a->prm.omega > 0.0;
+}
+
+bool rows_form_exists(const wl_amg *a, int l, int prec, int param) {
+  bool known = false;
+  for (int nrhs : {1, 8}) {  // the parameters rows_candidates hands out
+    int c[8], n = rows_candidates(nrhs, c);
+    for (int i = 0; i < n; ++i) known |= c[i] == param;
+  }
+  return known && rows_ok(a, l, prec, 1);
+}
+
+// the level's packed rows in precision prec, made on first use (stream s)
+int rows_prepare(wl_amg *a, int l, int prec, cudaStream_t s) {
+  Level &L = a->lev[l];
+  LevelOps &o = prec == WL_FP32 ? L.op32 : L.opbf;
+  if (o.rows.p) return WL_OK;
+  int nt = L.n / 64;
+  int sb = prec == WL_FP32 ? rb_step_bytes<zf>() : rb_step_bytes<zb>();
+  WL_TRY(o.rows.alloc((size_t)nt * 4 * sb));
+  unsigned grid = nt * 16 / RBP_CELLS;
+  if (prec == WL_FP32) k_rows_pack<zf><<<grid, 16 * RBP_CELLS, 0, s>>>(L.geo, o.A.as<zf>(), a->prm.omega, o.rows.as<unsigned char>());
+  else k_rows_pack<zb><<<grid, 16 * RBP_CELLS, 0, s>>>(L.geo, o.A.as<zb>(), a->prm.omega, o.rows.as<unsigned char>());
+  wl_count_launches(1);
+  WL_CUDA(cudaGetLastError());
+  return WL_OK;
+}
+
+int rows_sweeps(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int sweeps, int param, cudaStream_t s) {
+  const Level &L = a->lev[l];
+  for (int sw = 0; sw < sweeps; ++sw)
+    for (int tc = 0; tc < 4; ++tc) {
+      wl_count_launches(1);
+      if (prec == WL_FP32) WL_TRY(rows_tile<zf>(L, L.op32, tc, x, r, nrhs, param, sw + tc > 0, s));
+      else WL_TRY(rows_tile<zb>(L, L.opbf, tc, x, r, nrhs, param, sw + tc > 0, s));
+    }
+  WL_CUDA(cudaGetLastError());
+  return WL_OK;
+}
+
+}  // namespace wl

@@ -1,0 +1,87 @@
+"""Row-block form of the tile-coloured Kaczmarz sweep (launch form 4 of amg_kaczmarz_form) on the GPU."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1308_5992_gb300 import wilson_amg as W
+from oracle import oracle as O
+from wl_inputs import workload, cgauss
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+PARAMS = [1 | 1 << 8, 2 | 1 << 8, 4 | 1 << 8, 8 | 1 << 8, 8 | 2 << 8]
+
+
+def T(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+
+
+def rel(a, b):
+    return np.abs(a - b).max() / np.abs(b).max()
+
+
+def f32(a):
+    return a.astype(np.complex64).astype(np.complex128)
+
+
+@pytest.fixture(scope="module")
+def hier(tmp_path_factory):
+    from oracle.hierfile import write
+    out = {}
+    for name in ("T64", "T128"):  # fine grids 64 and 128, a coarse level of side 64
+        w = workload(name)
+        h = O.Hierarchy.setup(w["N"], w["U"], w["m"], O.setup_params(w["blocks"], k_r=w["k"], k_e=w["k"],
+                                                                     seed=w["seed"]))
+        path = str(tmp_path_factory.mktemp("rows") / (name + ".wlh"))
+        write(path, h.U, h.m, h.Nl, h.Bl, *h.export())
+        out[name] = (h, W.wilson_create(T(w["U"]), w["N"], w["m"]), path)
+    return out
+
+
+@pytest.mark.parametrize("name", ["T64", "T128"])
+@pytest.mark.parametrize("nrhs", [1, 2, 3, 5, 17])
+def test_row_block_sweep(hier, name, nrhs):
+    """Two sweeps against the oracle's tile order, every chunk of right-hand sides (ragged ones
+    too), to the bound of the other FP32 forms (1e-6 from the FP32 values of the inputs)."""
+    h, op, path = hier[name]
+    amg = W.amg_import(op, path, W.amg_params_default(zero_guess=1, kacz_order=1, precision=W.WL_FP32))
+    for l in range(h.L - 1):
+        if h.Nl[l] < 64:
+            continue
+        n = h.n(l)
+        x0 = f32(0.1 * np.stack([cgauss(410 + l, r, n) for r in range(nrhs)]))
+        r0 = f32(np.stack([cgauss(420 + l, r, n) for r in range(nrhs)]))
+        ref = [h.kaczmarz(l, x0[r], r0[r], order=O.ORDER_TILE, sweeps=2) for r in range(nrhs)]
+        xr, rr = np.stack([a for a, _ in ref]), np.stack([b for _, b in ref])
+        for param in PARAMS:
+            xg, rg = T(x0), T(r0)
+            W.amg_kaczmarz_form(amg, l, xg, rg, nrhs, 2, W.WL_FP32, 4, param)
+            assert rel(xg.cpu().numpy(), xr) <= 1e-6 and rel(rg.cpu().numpy(), rr) <= 1e-6, (l, param)
+    amg.close()
+
+
+@pytest.mark.parametrize("prec", [W.WL_FP32, W.WL_FP32_BF16])
+def test_row_block_sweep_relaxed(hier, prec):
+    """omega = 0.8 and BF16-stored stencils, against the tile kernel on the same stored numbers
+    (each within 1e-6 of the exact sweep, so 2e-6 of each other)."""
+    h, op, path = hier["T64"]
+    amg = W.amg_import(op, path, W.amg_params_default(zero_guess=1, kacz_order=1, precision=prec, omega=0.8))
+    n, nrhs = h.n(0), 3
+    x0 = f32(0.1 * np.stack([cgauss(430, r, n) for r in range(nrhs)]))
+    r0 = f32(np.stack([cgauss(440, r, n) for r in range(nrhs)]))
+    xa, ra, xb, rb = T(x0), T(r0), T(x0), T(r0)
+    W.amg_kaczmarz(amg, 0, xa, ra, nrhs, 2, prec)
+    W.amg_kaczmarz_form(amg, 0, xb, rb, nrhs, 2, prec, 4, 4 | 1 << 8)
+    assert rel(xb.cpu().numpy(), xa.cpu().numpy()) <= 2e-6 and rel(rb.cpu().numpy(), ra.cpu().numpy()) <= 2e-6
+    amg.close()
+
+
+def test_row_block_form_refused(hier):
+    """FP64 sweeps, the 16-colour ordering and unknown chunks have no row-block form."""
+    h, op, path = hier["T64"]
+    z = T(np.zeros((1, h.n(0)), dtype=complex))
+    for order, prec, param in ((1, W.WL_FP64, 1 | 1 << 8), (0, W.WL_FP32, 1 | 1 << 8), (1, W.WL_FP32, 3 | 1 << 8)):
+        amg = W.amg_import(op, path, W.amg_params_default(zero_guess=1, kacz_order=order))
+        with pytest.raises(W.WilsonAMGError):
+            W.amg_kaczmarz_form(amg, 0, z, z.clone(), 1, 1, prec, 4, param)
+        amg.close()
