@@ -339,6 +339,12 @@ bool rows_form_exists(const wl_amg *a, int l, int prec, int param);
 int rows_candidates(int nrhs, int *out);  // launch parameters worth timing (at most 8)
 int rows_prepare(wl_amg *a, int l, int prec, cudaStream_t s);
 int rows_sweeps(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int sweeps, int param, cudaStream_t s);
+// the same blocks on 32 x 32 and 16 x 16 levels (16-colour ordering), all sweeps in one launch;
+// rin: r or the right-hand side, xin: x or NULL (zero)
+bool rings_ok(const wl_amg *a, int l, int prec);
+int rings_prepare(wl_amg *a, int l, int prec, cudaStream_t s);
+int rings_sweeps(wl_amg *a, int l, int prec, const void *rin, const void *xin, void *x, void *r, int nrhs, int sweeps,
+                 cudaStream_t s);
 KTune sweep_form_of(wl_amg *a, int l, int prec, int nrhs);
 int restrict_op(wl_amg *a, int l, int prec, const void *r, void *fc, int nrhs, cudaStream_t s);
 int prolong_op(wl_amg *a, int l, int prec, const void *e, void *x, int nrhs, cudaStream_t s);

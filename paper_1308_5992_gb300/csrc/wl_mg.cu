@@ -1538,20 +1538,34 @@ int kaczmarz_sweeps(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int 
   return run_sweeps(a, l, prec, x, r, nrhs, sweeps, sweep_form_of(a, l, prec, nrhs), s);
 }
 
-// the sweeps of a cycle: the row-block form where it measured faster, unless
-// the launch form is explicit (sweep_kernel) or pinned; per-step calls
-// (amg_kaczmarz) keep kaczmarz_sweeps, whose forms agree bit for bit
-static int cycle_sweeps(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int sweeps, cudaStream_t s) {
-  const Level &L = a->lev[l];
-  if (sweeps <= 0) return WL_OK;
-  if (a->prm.sweep_kernel == 0 && rows_ok(a, l, prec, nrhs)) {
-    bool pinned = false;
-    for (const KTune &k : L.tune) pinned |= k.nrhs == nrhs && k.prec == prec && k.us == 0.f;
-    if (!pinned)
-      for (const KTune &k : L.rowtune)
-        if (k.nrhs == nrhs && k.prec == prec) return rows_sweeps(a, l, prec, x, r, nrhs, sweeps, k.param, s);
+// The sweeps of a cycle: the row-block forms (wl_rows.cu) on 32 x 32 and
+// 16 x 16 levels, and on larger tile-ordered levels where the autotuner
+// measured them faster, unless the launch form is explicit (sweep_kernel) or
+// pinned; per-step calls (amg_kaczmarz) keep kaczmarz_sweeps, whose forms
+// agree bit for bit.  zero: start from x = 0 and r = f (both written).
+static bool form_pinned(const wl_amg *a, int l, int prec, int nrhs) {
+  for (const KTune &k : a->lev[l].tune)
+    if (k.nrhs == nrhs && k.prec == prec && k.us == 0.f) return true;
+  return false;
+}
+static bool use_rings(const wl_amg *a, int l, int prec, int nrhs) {
+  const LevelOps &o = ops_of(a->lev[l], prec);
+  return a->prm.sweep_kernel == 0 && rings_ok(a, l, prec) && o.rows.p && !form_pinned(a, l, prec, nrhs);
+}
+static int cycle_sweeps(wl_amg *a, int l, int prec, int nrhs, int sweeps, bool zero, cudaStream_t s) {
+  Level &L = a->lev[l];
+  if (sweeps > 0 && use_rings(a, l, prec, nrhs))
+    return rings_sweeps(a, l, prec, zero ? L.f.p : L.r.p, zero ? nullptr : L.x.p, L.x.p, L.r.p, nrhs, sweeps, s);
+  if (zero) {
+    size_t vb = prec_bytes(prec) * (size_t)L.n * 2 * nrhs;
+    WL_CUDA(cudaMemsetAsync(L.x.p, 0, vb, s));
+    WL_CUDA(cudaMemcpyAsync(L.r.p, L.f.p, vb, cudaMemcpyDeviceToDevice, s));
   }
-  return kaczmarz_sweeps(a, l, prec, x, r, nrhs, sweeps, s);
+  if (sweeps <= 0) return WL_OK;
+  if (a->prm.sweep_kernel == 0 && rows_ok(a, l, prec, nrhs) && !form_pinned(a, l, prec, nrhs))
+    for (const KTune &k : L.rowtune)
+      if (k.nrhs == nrhs && k.prec == prec) return rows_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, sweeps, k.param, s);
+  return kaczmarz_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, sweeps, s);
 }
 
 // Autotuner: time every launch form of one sweep on each level (the level's
@@ -1720,11 +1734,8 @@ int coarsest_apply(wl_amg *a, int prec, const void *f, void *x, int nrhs, cudaSt
 static int cycle_level(wl_amg *a, int l, int nrhs, int prec, cudaStream_t s) {
   Level &L = a->lev[l];
   size_t eb = prec_bytes(prec);
-  size_t vb = eb * (size_t)L.n * 2 * nrhs;
   if (l == a->L - 1) return coarsest_apply(a, prec, L.f.p, L.x.p, nrhs, s);
-  WL_CUDA(cudaMemsetAsync(L.x.p, 0, vb, s));
-  WL_CUDA(cudaMemcpyAsync(L.r.p, L.f.p, vb, cudaMemcpyDeviceToDevice, s));
-  WL_TRY(cycle_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, a->prm.nu_pre, s));
+  WL_TRY(cycle_sweeps(a, l, prec, nrhs, a->prm.nu_pre, true, s));
   Level &C = a->lev[l + 1];
   WL_TRY(restrict_op(a, l, prec, L.r.p, C.f.p, nrhs, s));
   int gamma = (a->prm.cycle == WL_CYCLE_W) ? 2 : 1;
@@ -1746,7 +1757,7 @@ static int cycle_level(wl_amg *a, int l, int nrhs, int prec, cudaStream_t s) {
   }
   WL_TRY(prolong_op(a, l, prec, C.x.p, L.x.p, nrhs, s));
   WL_TRY(stencil_apply(a, l, prec, L.x.p, L.r.p, L.f.p, nrhs, s));
-  WL_TRY(cycle_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, a->prm.nu_post, s));
+  WL_TRY(cycle_sweeps(a, l, prec, nrhs, a->prm.nu_post, false, s));
   return WL_OK;
 }
 
@@ -1765,6 +1776,8 @@ int cycle_prepare(wl_amg *a, int nrhs, int prec, cudaStream_t s, const wl_amg::G
       return WL_OK;
     }
   WL_TRY(autotune_sweeps(a, nrhs, prec, s));  // measured launch forms, before the capture
+  for (int l = 0; l < a->L - 1; ++l)
+    if (a->prm.sweep_kernel == 0 && rings_ok(a, l, prec)) WL_TRY(rings_prepare(a, l, prec, s));
   cudaGraph_t graph;
   long long before = wl_launch_count();
   WL_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
@@ -1859,8 +1872,9 @@ static int kaczmarz_entry(wl_amg *a, int level, void *x, void *r, int nrhs, int 
     wl_set_error("%s: invalid argument (the coarsest level is not relaxed)", who);
     return WL_EINVAL;
   }
+  const bool rings = form == 5 && param == 0 && wl::rings_ok(a, level, prec);
   const bool rows = form == 4 && level < a->L - 1 && wl::rows_form_exists(a, level, prec, param);
-  if (form >= 0 && !rows && !form_exists(a, level, nrhs, prec, form, param)) {
+  if (form >= 0 && !rows && !rings && !form_exists(a, level, nrhs, prec, form, param)) {
     wl_set_error("%s: launch form %d / %d does not exist for this level and ordering", who, form, param);
     return WL_EINVAL;
   }
@@ -1878,6 +1892,10 @@ static int kaczmarz_entry(wl_amg *a, int level, void *x, void *r, int nrhs, int 
   } else if (rows) {
     WL_TRY(wl::rows_prepare(a, level, prec, s));
     WL_TRY(wl::rows_sweeps(a, level, prec, sb.b[0].p, sb.b[1].p, nrhs, sweeps, param, s));
+  } else if (rings) {
+    WL_TRY(wl::rings_prepare(a, level, prec, s));
+    if (sweeps > 0)
+      WL_TRY(wl::rings_sweeps(a, level, prec, sb.b[1].p, sb.b[0].p, sb.b[0].p, sb.b[1].p, nrhs, sweeps, s));
   } else if (sweeps > 0) {
     KTune t{nrhs, prec, form, param, 0.f};
     WL_TRY(wl::run_sweeps(a, level, prec, sb.b[0].p, sb.b[1].p, nrhs, sweeps, t, s));
@@ -1896,7 +1914,7 @@ extern "C" int amg_kaczmarz(wl_amg *a, int level, void *x, void *r, int nrhs, in
 extern "C" int amg_kaczmarz_form(wl_amg *a, int level, void *x, void *r, int nrhs, int sweeps, int prec, int form,
                                  int param) {
   if (form < 0) {
-    wl_set_error("amg_kaczmarz_form: form must be 0 to 4");
+    wl_set_error("amg_kaczmarz_form: form must be 0 to 5");
     return WL_EINVAL;
   }
   return kaczmarz_entry(a, level, x, r, nrhs, sweeps, prec, form, param, "amg_kaczmarz_form");

@@ -340,9 +340,282 @@ __global__ void __launch_bounds__(32 * R / RPT, RPT == 1 ? 16 / R : 0) k_kacz_ro
   }
 }
 
+// ------------------------------------------------------------- small levels
+// The 16-colour sweep of a 32 x 32 or 16 x 16 level with the same blocks: the
+// sites of a row a = const form a ring of N sites (position u; crossing u = N/2
+// continues in row a + N/2), and the colours 4 (a mod 4) + (b mod 4) take the
+// rings a mod 4 = 0, 1, 2, 3 in turn, in each ring the sites u mod 4 = 0, 1, 2,
+// 3.  So a sweep is 4 passes over N / 8 rings each, and in a pass a cell of 4
+// sites needs its own 8 inner products and the next cell's first 4.  One block
+// per right-hand side, a lane per site of a pass, r and the packed rings in
+// shared memory for all sweeps of a level visit, x in registers.
+//
+// Row of T of unknown (u, t) packed by what its colour j = u mod 4 can need: the
+// columns of the cell's colours 0, 1 (all sites), 2, 3 and the next cell's 0
+// (j >= 2), the next cell's 1 (j = 3): 15 complex floats a site on average.
+template <typename S, int N>
+__host__ __device__ constexpr int ring_bytes() {
+  return N * (36 * (int)sizeof(S) + 15 * (int)sizeof(zf));
+}
+// first float4 of the row (t) of T, part q = 0..3, for position u
+template <int N>
+__host__ __device__ constexpr int ring_t_at(int q, int t, int h, int u) {
+  // part 0: 2 float4 a row for all sites; 1: 2 for j >= 2; 2: 1 for j >= 2; 3: 1 for j = 3
+  return q == 0   ? (t * 2 + h) * N + u
+         : q == 1 ? 4 * N + (t * 2 + h) * (N / 2) + (u >> 2) * 2 + (u & 1)
+         : q == 2 ? 6 * N + t * (N / 2) + (u >> 2) * 2 + (u & 1)
+                  : 7 * N + t * (N / 4) + (u >> 2);
+}
+
+template <typename S, int N>
+__global__ void __launch_bounds__(16 * RBP_CELLS) k_rings_pack(Geo g, const S *__restrict__ A, double omega,
+                                                               unsigned char *__restrict__ out) {
+  __shared__ zd Ms[RBP_CELLS][12][13];
+  const int lc = threadIdx.x >> 4, i = threadIdx.x & 15;
+  const int id = blockIdx.x * RBP_CELLS + lc;  // N / 4 cells a ring, N / 2 rings: the grid is exact
+  const int cell = id % (N / 4), rg = id / (N / 4), pass = rg / (N / 8), row = pass + 4 * (rg % (N / 8));
+  auto site = [&](int u) { return g.idx(row + u, row - u); };
+  // position of site v = 0..5 of the order of relaxation: own 0, next 0, own 1, next 1, own 2, own 3
+  auto column = [&](int v) { return cell * 4 + (v < 4 ? (v >> 1) + 4 * (v & 1) : v - 2); };
+  if (i < 12)
+    for (int q = 0; q < 6; ++q)
+      for (int t2 = 0; t2 < 2; ++t2) {
+        const int cp = column(i >> 1), cq = column(q), dl = cq - cp;
+        zd k = mk(0.0, 0.0);
+        if (2 * q + t2 <= i && dl >= -2 && dl <= 2) k = rb_gram(A, site(cp), i & 1, site(cq), t2, dl);
+        if (2 * q + t2 == i) k = mk(k.re / omega, 0.0);
+        Ms[lc][i][2 * q + t2] = k;
+      }
+  __syncthreads();
+  unsigned char *so = out + (long)rg * ring_bytes<S, N>();
+  S *oa = (S *)so;
+  zf *ot = (zf *)(so + N * 36 * sizeof(S));
+  if (i < 12) {
+    const int v = i >> 1, t2 = i & 1;
+    const int k = (v < 4 ? ((v & 1) ? 8 : 0) + 2 * (v >> 1) : 2 * (v - 2)) + t2;  // column of T: own 0..7, next 8..11
+    const int q = k < 4 ? 0 : k < 8 ? 1 : k < 10 ? 2 : 3, h = q < 2 ? (k >> 1) & 1 : 0;
+    zd X[12];
+#pragma unroll
+    for (int r = 0; r < 12; ++r) {
+      zd w = mk(r == i ? 1.0 : 0.0, 0.0);
+#pragma unroll
+      for (int c = 0; c < r; ++c) w = w - Ms[lc][r][c] * X[c];
+      double d = Ms[lc][r][r].re;
+      X[r] = mk(w.re / d, w.im / d);
+      const int u = column(r >> 1), j = u & 3;
+      if (u < cell * 4 + 4 && (q == 0 || j == 3 || (j == 2 && q < 3)))
+        ot[2 * ring_t_at<N>(q, r & 1, h, u) + (k & 1)] = ccast<float>(X[r]);
+    }
+  }
+  for (int e = i; e < 4 * 36; e += 16) {
+    int u = cell * 4 + e / 36, c = e % 36;
+    oa[((c >> 1) * N + u) * 2 + (c & 1)] = A[(long)site(u) * 36 + c];
+  }
+}
+
+__device__ __forceinline__ float4 rb_cat(float2 a, float2 b) { return make_float4(a.x, a.y, b.x, b.y); }
+
+// `sweeps` sweeps for one right-hand side per block; rin (r or the level's
+// right-hand side) and xin (x, or NULL for a zero start) are read, x and r
+// written.  Bounded waits as in k_kacz_rows.
+//
+// Bound by shared-memory bandwidth (a pass reads 61 KB) and the chain of a pass.
+// Four sweeps of the 32 x 32 level: 5 right-hand sides with BF16-stored stencil
+// 17.9 us (k_kacz_block 61.7), one FP32 right-hand side 17 us (k_kacz_coop 160).
+template <typename S, int N>
+__global__ void __launch_bounds__(N *N / 8) k_kacz_rings(Geo g, int sweeps, const unsigned char *__restrict__ pk,
+                                                         const zf *rin, const zf *xin, zf *x, zf *r, int nrhs,
+                                                         int *timeout) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  constexpr int NT = N * N / 8, RB = ring_bytes<S, N>(), PB = RB * (N / 8);
+  unsigned char *cs = sm_raw;                                // [4][N / 8][RB]
+  float4 *rs = (float4 *)(sm_raw + 4 * PB);                  // [N / 2][N] both spins
+  float4 *nums = rs + N * N / 2;                             // [N / 8][N] both rows
+  uint64_t *mbar = (uint64_t *)(nums + NT);                  // [4]
+  const int tid = threadIdx.x, u = tid % N, ig = tid / N, rh = blockIdx.x;
+  if (tid == 0) {
+    for (int i = 0; i < 4; ++i) mbar_init(smem_u32(&mbar[i]), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int i = 0; i < 4; ++i) {
+      mbar_arrive_expect_tx(smem_u32(&mbar[i]), PB);
+      bulk_g2s(smem_u32(cs + i * PB), pk + (long)i * PB, PB, smem_u32(&mbar[i]));
+    }
+  }
+  const float2 *ri = (const float2 *)rin, *xi = (const float2 *)xin;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    int row = k + 4 * ig;
+    long o = (long)g.idx(row + u, row - u) * 2 * nrhs + rh;
+    rs[row * N + u] = rb_cat(ri[o], ri[o + nrhs]);
+  }
+  float2 xr[4][2];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    int row = k + 4 * ig;
+    long o = (long)g.idx(row + u, row - u) * 2 * nrhs + rh;
+    xr[k][0] = xi ? xi[o] : make_float2(0.f, 0.f);
+    xr[k][1] = xi ? xi[o + nrhs] : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  bool ok = true;
+  for (int sw = 0; sw < sweeps && ok; ++sw) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (sw == 0) {
+        ok = ok && mbar_wait(smem_u32(&mbar[k]), 0, 1000000000ull);
+        ok = __syncthreads_and(ok);
+        if (!ok) break;
+      }
+      const int row = k + 4 * ig;
+      const S *ca = (const S *)(cs + k * PB + ig * RB);
+      const zf *ct = (const zf *)(cs + k * PB + ig * RB + N * 36 * sizeof(S));
+      // the window: rows row - 1, row, row + 1 (past the last ring the ring 0
+      // half a turn on, before the first one the last ring likewise)
+      float4 *wr[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        int ro = row + i - 1, sh = 0;
+        if (ro < 0) ro += N / 2, sh = N / 2;
+        if (ro >= N / 2) ro -= N / 2, sh = N / 2;
+        wr[i] = rs + ro * N + ((u + sh) & (N - 1));
+      }
+      const int ul[3] = {-1, 0, 1};
+      float2 a[9][2][2];  // [d][row t][spin]
+#pragma unroll
+      for (int d = 0; d < 9; ++d)
+#pragma unroll
+        for (int t = 0; t < 2; ++t) rb_ld(ca + ((d * 2 + t) * N + u) * 2, a[d][t][0], a[d][t][1]);
+      float2 d0[2][2], e0[2][2];  // [t][spin]
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int sp = 0; sp < 2; ++sp) d0[t][sp] = e0[t][sp] = make_float2(0.f, 0.f);
+      float4 rc[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        float4 *row0 = rs + ((wr[i] - rs) & ~(N - 1));
+        const int uu = (int)((wr[i] - rs) & (N - 1));
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          float4 v = row0[(uu + ul[q]) & (N - 1)];
+          if (q == 1) rc[i] = v;
+          float2 v0 = make_float2(v.x, v.y), v1 = make_float2(v.z, v.w);
+          float2 w0 = rb_swap(v0), w1 = rb_swap(v1);
+          const int d = i * 3 + q;
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            d0[t][0] = __ffma2_rn(a[d][t][0], v0, d0[t][0]);
+            e0[t][0] = __ffma2_rn(a[d][t][0], w0, e0[t][0]);
+            d0[t][1] = __ffma2_rn(a[d][t][1], v1, d0[t][1]);
+            e0[t][1] = __ffma2_rn(a[d][t][1], w1, e0[t][1]);
+          }
+        }
+      }
+      float2 nm[2];
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        float re = (d0[t][0].x - d0[t][0].y) - (d0[t][1].x - d0[t][1].y);
+        float im = (e0[t][0].x + e0[t][0].y) - (e0[t][1].x + e0[t][1].y);
+        nm[t] = t ? make_float2(-re, -im) : make_float2(re, im);
+      }
+      float4 *nr = nums + ig * N;
+      nr[u] = rb_cat(nm[0], nm[1]);
+      const int j = u & 3;
+      float2 T[2][12];
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+#pragma unroll
+        for (int c = 4; c < 12; ++c) T[t][c] = make_float2(0.f, 0.f);
+        rb_ld(ct + 2 * ring_t_at<N>(0, t, 0, u), T[t][0], T[t][1]);
+        rb_ld(ct + 2 * ring_t_at<N>(0, t, 1, u), T[t][2], T[t][3]);
+        if (j >= 2) {
+          rb_ld(ct + 2 * ring_t_at<N>(1, t, 0, u), T[t][4], T[t][5]);
+          rb_ld(ct + 2 * ring_t_at<N>(1, t, 1, u), T[t][6], T[t][7]);
+          rb_ld(ct + 2 * ring_t_at<N>(2, t, 0, u), T[t][8], T[t][9]);
+        }
+        if (j == 3) rb_ld(ct + 2 * ring_t_at<N>(3, t, 0, u), T[t][10], T[t][11]);
+      }
+      __syncwarp();
+      float2 sd[2][2], se[2][2];
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) sd[t][c] = se[t][c] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        float4 v = nr[((u & ~3) + c) & (N - 1)];  // the cell's four sites, then the next cell's first two
+        float2 v0 = make_float2(v.x, v.y), v1 = make_float2(v.z, v.w), w0 = rb_swap(v0), w1 = rb_swap(v1);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          sd[t][0] = __ffma2_rn(T[t][2 * c], v0, sd[t][0]);
+          se[t][0] = __ffma2_rn(T[t][2 * c], w0, se[t][0]);
+          sd[t][1] = __ffma2_rn(T[t][2 * c + 1], v1, sd[t][1]);
+          se[t][1] = __ffma2_rn(T[t][2 * c + 1], w1, se[t][1]);
+        }
+      }
+      float2 s0 = make_float2((sd[0][0].x - sd[0][0].y) + (sd[0][1].x - sd[0][1].y),
+                              (se[0][0].x + se[0][0].y) + (se[0][1].x + se[0][1].y));
+      float2 s1 = make_float2((sd[1][0].x - sd[1][0].y) + (sd[1][1].x - sd[1][1].y),
+                              (se[1][0].x + se[1][0].y) + (se[1][1].x + se[1][1].y));
+      xr[k][0] = make_float2(xr[k][0].x + s0.x, xr[k][0].y + s0.y);
+      xr[k][1] = make_float2(xr[k][1].x + s1.x, xr[k][1].y + s1.y);
+      // r_(d,sp) -= g_sp (s_0 conj(a[d][0][sp]) - s_1 conj(a[d][1][sp]))
+      float2 m1 = make_float2(-s1.x, -s1.y), n0 = rb_swap(s0), n1 = rb_swap(m1);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        float2 dl[3][2];
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+          for (int sp = 0; sp < 2; ++sp) {
+            float2 v = __ffma2_rn(a[i * 3 + q][1][sp], m1, __fmul2_rn(a[i * 3 + q][0][sp], s0));
+            float2 w = __ffma2_rn(a[i * 3 + q][1][sp], n1, __fmul2_rn(a[i * 3 + q][0][sp], n0));
+            dl[q][sp] = make_float2(v.x + v.y, w.x - w.y);
+          }
+        float2 tot[2];
+#pragma unroll
+        for (int sp = 0; sp < 2; ++sp) {
+          float2 up = make_float2(__shfl_sync(0xffffffffu, dl[2][sp].x, (u - 1) & (N - 1), N),
+                                  __shfl_sync(0xffffffffu, dl[2][sp].y, (u - 1) & (N - 1), N));
+          float2 dn = make_float2(__shfl_sync(0xffffffffu, dl[0][sp].x, (u + 1) & (N - 1), N),
+                                  __shfl_sync(0xffffffffu, dl[0][sp].y, (u + 1) & (N - 1), N));
+          tot[sp] = make_float2(dl[1][sp].x + up.x + dn.x, dl[1][sp].y + up.y + dn.y);
+        }
+        *wr[i] = make_float4(rc[i].x - tot[0].x, rc[i].y - tot[0].y, rc[i].z + tot[1].x, rc[i].w + tot[1].y);
+      }
+      __syncthreads();
+    }
+  }
+  if (!__syncthreads_and(ok)) {
+    if (tid == 0) atomicExch(timeout, 1);
+    return;
+  }
+  float2 *ro = (float2 *)r, *xo = (float2 *)x;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    int row = k + 4 * ig;
+    long o = (long)g.idx(row + u, row - u) * 2 * nrhs + rh;
+    float4 v = rs[row * N + u];
+    ro[o] = make_float2(v.x, v.y);
+    ro[o + nrhs] = make_float2(v.z, v.w);
+    xo[o] = xr[k][0];
+    xo[o + nrhs] = xr[k][1];
+  }
+}
+
 namespace wl {
 
-int *tile_timeout_flag();
+// raise a kernel's dynamic shared-memory limit once per device
+static int rb_smem_limit(const void *fn, size_t bytes, std::atomic<unsigned long long> &done) {
+  int dev = 0;
+  WL_CUDA(cudaGetDevice(&dev));
+  unsigned long long bit = 1ull << (dev & 63);
+  if (!(done.load(std::memory_order_acquire) & bit)) {
+    WL_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    done.fetch_or(bit, std::memory_order_acq_rel);
+  }
+  return WL_OK;
+}
 
 template <typename S, int R, int RPT>
 static int launch_rows(const Level &L, const LevelOps &o, int tc, void *x, void *r, int nrhs, int pdl, cudaStream_t s) {
@@ -350,13 +623,7 @@ static int launch_rows(const Level &L, const LevelOps &o, int tc, void *x, void 
   size_t smem = (size_t)4 * rb_step_bytes<S>() + sizeof(zf) * ((R * RB_RS + 1) & ~1) + sizeof(zf) * R * 40 +
                 sizeof(int) * RB_W * RB_W + 4 * sizeof(uint64_t);
   static std::atomic<unsigned long long> done{0};
-  int dev = 0;
-  WL_CUDA(cudaGetDevice(&dev));
-  unsigned long long bit = 1ull << (dev & 63);
-  if (!(done.load(std::memory_order_acquire) & bit)) {
-    WL_CUDA(cudaFuncSetAttribute(k_kacz_rows<S, R, RPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    done.fetch_or(bit, std::memory_order_acq_rel);
-  }
+  WL_TRY(rb_smem_limit((const void *)k_kacz_rows<S, R, RPT>, smem, done));
   int *flag = tile_timeout_flag();
   if (!flag) return WL_ECUDA;
   dim3 grid((L.N / (2 * RB_KT)) * (L.N / (4 * RB_KT)), (nrhs + R - 1) / R);
@@ -453,6 +720,57 @@ int rows_sweeps(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int swee
     }
   WL_CUDA(cudaGetLastError());
   return WL_OK;
+}
+
+// ---- small levels
+bool rings_ok(const wl_amg *a, int l, int prec) {
+  const Level &L = a->lev[l];
+  return prec != WL_FP64 && l < a->L - 1 && (L.N == 32 || L.N == 16) && a->prm.omega > 0.0;
+}
+
+template <typename S, int N>
+static int rings_pack(const Level &L, LevelOps &o, double omega, cudaStream_t s) {
+  WL_TRY(o.rows.alloc((size_t)(N / 2) * ring_bytes<S, N>()));
+  k_rings_pack<S, N><<<N * N / 8 / RBP_CELLS, 16 * RBP_CELLS, 0, s>>>(L.geo, o.A.as<S>(), omega,
+                                                                     o.rows.as<unsigned char>());
+  wl_count_launches(1);
+  WL_CUDA(cudaGetLastError());
+  return WL_OK;
+}
+
+int rings_prepare(wl_amg *a, int l, int prec, cudaStream_t s) {
+  Level &L = a->lev[l];
+  LevelOps &o = prec == WL_FP32 ? L.op32 : L.opbf;
+  if (o.rows.p) return WL_OK;
+  if (prec == WL_FP32) return L.N == 32 ? rings_pack<zf, 32>(L, o, a->prm.omega, s) : rings_pack<zf, 16>(L, o, a->prm.omega, s);
+  return L.N == 32 ? rings_pack<zb, 32>(L, o, a->prm.omega, s) : rings_pack<zb, 16>(L, o, a->prm.omega, s);
+}
+
+template <typename S, int N>
+static int launch_rings(const Level &L, const LevelOps &o, const void *rin, const void *xin, void *x, void *r, int nrhs,
+                        int sweeps, cudaStream_t s) {
+  const size_t smem = (size_t)(N / 2) * ring_bytes<S, N>() + sizeof(float4) * (N * N / 2 + N * N / 8) + 4 * sizeof(uint64_t);
+  static_assert((N / 2) * ring_bytes<S, N>() + 16 * (N * N / 2 + N * N / 8) + 32 <= 227 * 1024, "shared memory");
+  static std::atomic<unsigned long long> done{0};
+  WL_TRY(rb_smem_limit((const void *)k_kacz_rings<S, N>, smem, done));
+  int *flag = tile_timeout_flag();
+  if (!flag) return WL_ECUDA;
+  k_kacz_rings<S, N><<<nrhs, N * N / 8, smem, s>>>(L.geo, sweeps, o.rows.as<unsigned char>(), (const zf *)rin,
+                                                   (const zf *)xin, (zf *)x, (zf *)r, nrhs, flag);
+  wl_count_launches(1);
+  WL_CUDA(cudaGetLastError());
+  return WL_OK;
+}
+
+int rings_sweeps(wl_amg *a, int l, int prec, const void *rin, const void *xin, void *x, void *r, int nrhs, int sweeps,
+                 cudaStream_t s) {
+  const Level &L = a->lev[l];
+  const LevelOps &o = prec == WL_FP32 ? L.op32 : L.opbf;
+  if (prec == WL_FP32)
+    return L.N == 32 ? launch_rings<zf, 32>(L, o, rin, xin, x, r, nrhs, sweeps, s)
+                     : launch_rings<zf, 16>(L, o, rin, xin, x, r, nrhs, sweeps, s);
+  return L.N == 32 ? launch_rings<zb, 32>(L, o, rin, xin, x, r, nrhs, sweeps, s)
+                   : launch_rings<zb, 16>(L, o, rin, xin, x, r, nrhs, sweeps, s);
 }
 
 }  // namespace wl

@@ -1,4 +1,4 @@
-"""Row-block form of the tile-coloured Kaczmarz sweep (launch form 4 of amg_kaczmarz_form) on the GPU."""
+"""Row-block forms of the Kaczmarz sweep on the GPU (launch forms 4 and 5 of amg_kaczmarz_form)."""
 import numpy as np
 import pytest
 import torch
@@ -26,14 +26,14 @@ def f32(a):
 
 @pytest.fixture(scope="module")
 def hier(tmp_path_factory):
-    from oracle.hierfile import write
+    from oracle.hierfile import write_hierarchy
     out = {}
-    for name in ("T64", "T128"):  # fine grids 64 and 128, a coarse level of side 64
-        w = workload(name)
-        h = O.Hierarchy.setup(w["N"], w["U"], w["m"], O.setup_params(w["blocks"], k_r=w["k"], k_e=w["k"],
-                                                                     seed=w["seed"]))
+    # fine grids 64 and 128, coarse levels of side 64, 32 and (deep) 16
+    for name, blocks in (("T64", [2, 2]), ("T128", [2, 2, 2]), ("deep", [2, 2, 2])):
+        w = workload("T64" if name == "deep" else name)
+        h = O.Hierarchy.setup(w["N"], w["U"], w["m"], O.setup_params(blocks, k_r=w["k"], k_e=w["k"], seed=w["seed"]))
         path = str(tmp_path_factory.mktemp("rows") / (name + ".wlh"))
-        write(path, h.U, h.m, h.Nl, h.Bl, *h.export())
+        write_hierarchy(path, h)
         out[name] = (h, W.wilson_create(T(w["U"]), w["N"], w["m"]), path)
     return out
 
@@ -85,3 +85,29 @@ def test_row_block_form_refused(hier):
         with pytest.raises(W.WilsonAMGError):
             W.amg_kaczmarz_form(amg, 0, z, z.clone(), 1, 1, prec, 4, param)
         amg.close()
+
+
+@pytest.mark.parametrize("nrhs", [1, 5])
+def test_small_level_sweeps(hier, nrhs):
+    """The one-launch form on the 32x32 and 16x16 levels: three sweeps against the oracle's colour
+    order (1e-6 as above), and BF16-stored against the per-colour launches."""
+    h, op, path = hier["deep"]
+    assert h.Nl == [64, 32, 16, 8]
+    amg = W.amg_import(op, path, W.amg_params_default(zero_guess=1, precision=W.WL_FP32))
+    for l in (1, 2):
+        n = h.n(l)
+        x0 = f32(0.1 * np.stack([cgauss(450 + l, r, n) for r in range(nrhs)]))
+        r0 = f32(np.stack([cgauss(460 + l, r, n) for r in range(nrhs)]))
+        ref = [h.kaczmarz(l, x0[r], r0[r], order=O.ORDER_COLOUR, sweeps=3) for r in range(nrhs)]
+        xr, rr = np.stack([a for a, _ in ref]), np.stack([b for _, b in ref])
+        xg, rg = T(x0), T(r0)
+        W.amg_kaczmarz_form(amg, l, xg, rg, nrhs, 3, W.WL_FP32, 5, 0)
+        assert rel(xg.cpu().numpy(), xr) <= 1e-6 and rel(rg.cpu().numpy(), rr) <= 1e-6, l
+        xa, ra, xb, rb = T(x0), T(r0), T(x0), T(r0)
+        W.amg_kaczmarz_form(amg, l, xa, ra, nrhs, 3, W.WL_FP32_BF16, 0, 0)
+        W.amg_kaczmarz_form(amg, l, xb, rb, nrhs, 3, W.WL_FP32_BF16, 5, 0)
+        assert rel(xb.cpu().numpy(), xa.cpu().numpy()) <= 2e-6 and rel(rb.cpu().numpy(), ra.cpu().numpy()) <= 2e-6, l
+    z = T(np.zeros((1, h.n(0)), dtype=complex))
+    with pytest.raises(W.WilsonAMGError):  # a 64x64 level
+        W.amg_kaczmarz_form(amg, 0, z, z.clone(), 1, 1, W.WL_FP32, 5, 0)
+    amg.close()
