@@ -392,9 +392,10 @@ int wl_time_kernel(wl_amg *amg, int kind, int level, int nrhs, int prec, int rep
  * rows and denominators in shared memory too); *us = the autotuner's measured time of one
  * sweep in microseconds, 0 when the form was not measured (explicit
  * sweep_kernel, or no cycle of that width yet).  Errors: WL_EINVAL.
- * These forms agree bit for bit.  The sweeps of a cycle with an FP32 or BF16 precision and
- * no pinned form take the row-block forms instead (the same sweep, rounded differently): on
- * 32x32 and 16x16 levels, and on tile-ordered ones where the autotuner measured it faster. */
+ * These forms agree bit for bit.  The sweeps of a cycle without a pinned form take the
+ * row-block forms instead (the same sweep, rounded differently): FP32 or BF16 on 32x32 and
+ * 16x16 levels, and on tile-ordered ones (FP64: on 16-colour ones) where the autotuner measured
+ * them faster. */
 int amg_sweep_form(wl_amg *amg, int level, int nrhs, int prec, int *form, int *param, float *us);
 /* Pin the Kaczmarz launch form of `level` (not the coarsest) for `nrhs`
  * right-hand sides in precision `prec` (form and param as in
@@ -411,7 +412,8 @@ int amg_pin_sweep_form(wl_amg *amg, int level, int nrhs, int prec, int form, int
  * the same numbers.  Form 4 (tile ordering, FP32 or BF16, param = R | RPT << 8: right-hand
  * sides per block and per warp, one of (1, 1), (2, 1), (4, 1), (8, 1), (8, 2)) is the
  * row-block form of the cycle; form 5 (32x32 and 16x16 levels, FP32 or BF16, param 0) its
- * one-launch form there.  Errors: WL_EINVAL (no such form). */
+ * one-launch form there; form 6 (16-colour ordering, FP64) those of FP64 cycles: param 0 two
+ * launches a pass, 1 (32x32 and 64x64 levels) one launch of clusters.  Errors: WL_EINVAL (no such form). */
 int amg_kaczmarz_form(wl_amg *amg, int level, void *x, void *r, int nrhs, int sweeps, int prec, int form, int param);
 /* Number of kernels this library has launched in this process (a captured
  * graph counts each of its kernel nodes at every replay). */

@@ -249,7 +249,7 @@ struct LevelOps {
   DBuf A;    // stencil [n][9][2][2]
   DBuf den;  // Kaczmarz denominators ||A e_i||^2, [n][2] (real, T)
   DBuf P;    // interpolation weights to the next level [n][2][4]
-  DBuf rows; // packed tile rows of the row-block sweep (wl_rows.cu), made on first use
+  DBuf rows; // packed rows (FP64: triangular inverses) of the row-block sweeps (wl_rows.cu), made on first use
 };
 
 // launch form of a Kaczmarz sweep on one level, chosen by the autotuner
@@ -268,6 +268,7 @@ struct Level {
   LevelOps op64, op32, opbf;  // FP64 master, FP32 copy, BF16 copy (den in FP32)
   // cycle work vectors, [n][2][nrhs_cap] in the cycle precision
   DBuf x, r, f, t;
+  DBuf nums;                  // inner products of a ring pass (FP64 16-colour sweeps)
   std::vector<KTune> tune;    // autotuned sweep forms per (nrhs, precision)
   std::vector<KTune> rowtune; // where the row-block sweep measured faster: form 4, param = R | RPT << 8
 };
@@ -345,6 +346,12 @@ bool rings_ok(const wl_amg *a, int l, int prec);
 int rings_prepare(wl_amg *a, int l, int prec, cudaStream_t s);
 int rings_sweeps(wl_amg *a, int l, int prec, const void *rin, const void *xin, void *x, void *r, int nrhs, int sweeps,
                  cudaStream_t s);
+// the same blocks on 16-colour-ordered levels in FP64 (two launches a ring pass, or one of clusters)
+bool rings64_ok(const wl_amg *a, int l, int prec, int nrhs);
+int rings64_prepare(wl_amg *a, int l, int nrhs, cudaStream_t s);
+bool rings64_form(const wl_amg *a, int l, int param);
+int rings64_sweeps(wl_amg *a, int l, const void *rin, const void *xin, void *x, void *r, int nrhs, int sweeps, int param,
+                   cudaStream_t s);
 KTune sweep_form_of(wl_amg *a, int l, int prec, int nrhs);
 int restrict_op(wl_amg *a, int l, int prec, const void *r, void *fc, int nrhs, cudaStream_t s);
 int prolong_op(wl_amg *a, int l, int prec, const void *e, void *x, int nrhs, cudaStream_t s);

@@ -1554,17 +1554,23 @@ static bool use_rings(const wl_amg *a, int l, int prec, int nrhs) {
 }
 static int cycle_sweeps(wl_amg *a, int l, int prec, int nrhs, int sweeps, bool zero, cudaStream_t s) {
   Level &L = a->lev[l];
-  if (sweeps > 0 && use_rings(a, l, prec, nrhs))
-    return rings_sweeps(a, l, prec, zero ? L.f.p : L.r.p, zero ? nullptr : L.x.p, L.x.p, L.r.p, nrhs, sweeps, s);
+  const void *rin = zero ? L.f.p : L.r.p, *xin = zero ? nullptr : L.x.p;  // for the one-launch forms
+  if (sweeps > 0 && use_rings(a, l, prec, nrhs)) return rings_sweeps(a, l, prec, rin, xin, L.x.p, L.r.p, nrhs, sweeps, s);
+  const KTune *rows = nullptr;  // the row-block choice of a tuned level
+  if (sweeps > 0 && a->prm.sweep_kernel == 0 && !form_pinned(a, l, prec, nrhs) &&
+      (rows_ok(a, l, prec, nrhs) || rings64_ok(a, l, prec, nrhs)))
+    for (const KTune &k : L.rowtune)
+      if (k.nrhs == nrhs && k.prec == prec) rows = &k;
+  if (rows && rows->form == 6 && rows->param == 1)
+    return rings64_sweeps(a, l, rin, xin, L.x.p, L.r.p, nrhs, sweeps, 1, s);
   if (zero) {
     size_t vb = prec_bytes(prec) * (size_t)L.n * 2 * nrhs;
     WL_CUDA(cudaMemsetAsync(L.x.p, 0, vb, s));
     WL_CUDA(cudaMemcpyAsync(L.r.p, L.f.p, vb, cudaMemcpyDeviceToDevice, s));
   }
   if (sweeps <= 0) return WL_OK;
-  if (a->prm.sweep_kernel == 0 && rows_ok(a, l, prec, nrhs) && !form_pinned(a, l, prec, nrhs))
-    for (const KTune &k : L.rowtune)
-      if (k.nrhs == nrhs && k.prec == prec) return rows_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, sweeps, k.param, s);
+  if (rows && rows->form == 4) return rows_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, sweeps, rows->param, s);
+  if (rows) return rings64_sweeps(a, l, L.r.p, L.x.p, L.x.p, L.r.p, nrhs, sweeps, rows->param, s);
   return kaczmarz_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, sweeps, s);
 }
 
@@ -1625,11 +1631,17 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
       int prm[8], n = rows_candidates(nrhs, prm);
       for (int i = 0; i < n; ++i) cand.push_back(KTune{nrhs, prec, 4, prm[i], 0.f});
     }
+    if (rings64_ok(a, l, prec, nrhs)) {
+      if ((rc = rings64_prepare(a, l, nrhs, s))) break;
+      for (int q : {0, 1})
+        if (rings64_form(a, l, q)) cand.push_back(KTune{nrhs, prec, 6, q, 0.f});
+    }
     KTune best = cand[0], rows{nrhs, prec, 4, 0, 1e30f};
     float best_us = 1e30f;
     auto sweep = [&](const KTune &c) -> int {
-      return c.form == 4 ? rows_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c.param, s)
-                         : run_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c, s);
+      return c.form == 6   ? rings64_sweeps(a, l, L.r.p, L.x.p, L.x.p, L.r.p, nrhs, 1, c.param, s)
+             : c.form == 4 ? rows_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c.param, s)
+                           : run_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c, s);
     };
     for (KTune &c : cand) {
       rc = sweep(c);  // warm-up
@@ -1644,7 +1656,7 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
         break;
       }
       c.us = ms * 1e3f / 3;
-      if (c.form == 4) {
+      if (c.form >= 4) {
         if (c.us < rows.us) rows = c;
       } else if (c.us < best_us) {
         best_us = c.us;
@@ -1873,8 +1885,9 @@ static int kaczmarz_entry(wl_amg *a, int level, void *x, void *r, int nrhs, int 
     return WL_EINVAL;
   }
   const bool rings = form == 5 && param == 0 && wl::rings_ok(a, level, prec);
+  const bool rings64 = form == 6 && wl::rings64_ok(a, level, prec, 1) && wl::rings64_form(a, level, param);
   const bool rows = form == 4 && level < a->L - 1 && wl::rows_form_exists(a, level, prec, param);
-  if (form >= 0 && !rows && !rings && !form_exists(a, level, nrhs, prec, form, param)) {
+  if (form >= 0 && !rows && !rings && !rings64 && !form_exists(a, level, nrhs, prec, form, param)) {
     wl_set_error("%s: launch form %d / %d does not exist for this level and ordering", who, form, param);
     return WL_EINVAL;
   }
@@ -1892,6 +1905,11 @@ static int kaczmarz_entry(wl_amg *a, int level, void *x, void *r, int nrhs, int 
   } else if (rows) {
     WL_TRY(wl::rows_prepare(a, level, prec, s));
     WL_TRY(wl::rows_sweeps(a, level, prec, sb.b[0].p, sb.b[1].p, nrhs, sweeps, param, s));
+  } else if (rings64) {
+    WL_TRY(wl::ensure_workspace(a, nrhs, prec));
+    WL_TRY(wl::rings64_prepare(a, level, nrhs, s));
+    if (sweeps > 0)
+      WL_TRY(wl::rings64_sweeps(a, level, sb.b[1].p, sb.b[0].p, sb.b[0].p, sb.b[1].p, nrhs, sweeps, param, s));
   } else if (rings) {
     WL_TRY(wl::rings_prepare(a, level, prec, s));
     if (sweeps > 0)
@@ -1914,7 +1932,7 @@ extern "C" int amg_kaczmarz(wl_amg *a, int level, void *x, void *r, int nrhs, in
 extern "C" int amg_kaczmarz_form(wl_amg *a, int level, void *x, void *r, int nrhs, int sweeps, int prec, int form,
                                  int param) {
   if (form < 0) {
-    wl_set_error("amg_kaczmarz_form: form must be 0 to 5");
+    wl_set_error("amg_kaczmarz_form: form must be 0 to 6");
     return WL_EINVAL;
   }
   return kaczmarz_entry(a, level, x, r, nrhs, sweeps, prec, form, param, "amg_kaczmarz_form");

@@ -19,11 +19,15 @@
 // at most two columns apart, so a cell needs its own 8 inner products and, for
 // the left cell of an even row (the right cell of an odd one), 4 of the other
 // cell: T has 12 columns.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <atomic>
 
 #include "wl_common.cuh"
 #include "wl_tile_order.h"
+
+namespace cg = cooperative_groups;
 
 #define RB_KT 8
 #define RB_W 10    // window side: tile and halo
@@ -50,6 +54,11 @@ __device__ __forceinline__ void rb_origin(const Geo &g, int tc, int t, int &A0, 
   B0 = ((tc >> 1) + 2 * (t % nb4)) * RB_KT;
 }
 
+// stored coefficient as complex double (floats widened on the integer pipes)
+__device__ __forceinline__ zd rb_ld64(const zd *p) { return *p; }
+__device__ __forceinline__ zd rb_ld64(const zf *p) { return widen<double>(*p); }
+__device__ __forceinline__ zd rb_ld64(const zb *p) { return widen<double>(ld<float>(p)); }
+
 // K = <A e_(h2,t2), A e_(h,t)> for sites h, h2 of one row, h2 = h + delta
 // columns (|delta| <= 2): column (h, t) has the entries g_s g_t conj(A[h][d][t][s])
 template <typename S>
@@ -61,7 +70,7 @@ __device__ zd rb_gram(const S *__restrict__ A, int h, int t, int h2, int t2, int
       if (eb < 0 || eb > 2) continue;
       const S *p = A + ((long)h * 9 + da * 3 + db) * 4 + t * 2;
       const S *q = A + ((long)h2 * 9 + da * 3 + eb) * 4 + t2 * 2;
-      for (int s = 0; s < 2; ++s) k = k + widen<double>(ld<float>(p + s)) * cconj(widen<double>(ld<float>(q + s)));
+      for (int s = 0; s < 2; ++s) k = k + rb_ld64(p + s) * cconj(rb_ld64(q + s));
     }
   double f = (t ^ t2) ? -1.0 : 1.0;
   return mk(f * k.re, f * k.im);
@@ -603,6 +612,329 @@ __global__ void __launch_bounds__(N *N / 8) k_kacz_rings(Geo g, int sweeps, cons
   }
 }
 
+// --------------------------------------------------- 16-colour sweeps in FP64
+// The ring passes on a level of any size, two launches a pass: k_ring_dots forms
+// the inner products of every site of the rings a mod 4 = pass, k_ring_update
+// solves the cells' triangular systems and updates x and r.  In FP64 a warp
+// instruction takes the SM's FP64 unit 16 cycles and its warp 64, whatever the
+// number of active lanes, so a chain of FP64 instructions is what a small level
+// waits for: the products of a site are spread over 4 H lanes (row, real or
+// imaginary part, and with H = 2, 4 the spin and half of the offsets), the T rows
+// over 8 and the update over 12 a site, and nothing is divided.
+//
+// T [4][n / 4][2][12] (pass, ring and position, row): columns 0..7 the cell's own
+// unknowns, 8..11 the next cell's first four.
+__global__ void __launch_bounds__(16 * RBP_CELLS) k_ring64_pack(Geo g, const zd *__restrict__ A, double omega,
+                                                                zd *__restrict__ T) {
+  __shared__ zd Ms[RBP_CELLS][12][13];
+  const int N = g.N, lc = threadIdx.x >> 4, i = threadIdx.x & 15;
+  const int id = blockIdx.x * RBP_CELLS + lc;  // N / 4 cells a ring, N / 2 rings: the grid is exact
+  const int cell = id % (N / 4), rg = id / (N / 4), pass = rg / (N / 8), row = pass + 4 * (rg % (N / 8));
+  auto site = [&](int u) { return g.idx(row + u, row - u); };
+  auto column = [&](int v) { return cell * 4 + (v < 4 ? (v >> 1) + 4 * (v & 1) : v - 2); };  // as in k_rings_pack
+  if (i < 12)
+    for (int q = 0; q < 6; ++q)
+      for (int t2 = 0; t2 < 2; ++t2) {
+        const int cp = column(i >> 1), cq = column(q), dl = cq - cp;
+        zd k = mk(0.0, 0.0);
+        if (2 * q + t2 <= i && dl >= -2 && dl <= 2) k = rb_gram(A, site(cp), i & 1, site(cq), t2, dl);
+        if (2 * q + t2 == i) k = mk(k.re / omega, 0.0);
+        Ms[lc][i][2 * q + t2] = k;
+      }
+  __syncthreads();
+  if (i >= 12) return;
+  const int v = i >> 1;
+  const int k = (v < 4 ? ((v & 1) ? 8 : 0) + 2 * (v >> 1) : 2 * (v - 2)) + (i & 1);
+  zd X[12];
+#pragma unroll
+  for (int r = 0; r < 12; ++r) {
+    zd w = mk(r == i ? 1.0 : 0.0, 0.0);
+#pragma unroll
+    for (int c = 0; c < r; ++c) w = w - Ms[lc][r][c] * X[c];
+    double d = Ms[lc][r][r].re;
+    X[r] = mk(w.re / d, w.im / d);
+    const int u = column(r >> 1);
+    if (u < cell * 4 + 4) T[(((long)rg * N + u) * 2 + (r & 1)) * 12 + k] = X[r];
+  }
+}
+
+// v with its sign flipped where `neg` (on the integer pipe: a negation that is
+// not known at compile time costs an instruction of the FP64 unit, and the
+// update of a pass took 2860 instead of 1580 cycles with them)
+__device__ __forceinline__ double rb_flip(double v, bool neg) {
+  return __hiloint2double(__double2hiint(v) ^ (neg ? (int)0x80000000 : 0), __double2loint(v));
+}
+// component c of a v: c = 0: a.re v.re - a.im v.im, c = 1: a.re v.im + a.im v.re
+__device__ __forceinline__ void rb_cfma(double &acc, zd a, zd v, int c) {
+  acc = fma(a.re, c ? v.im : v.re, acc);
+  acc = fma(rb_flip(a.im, c == 0), c ? v.re : v.im, acc);
+}
+
+template <int H>
+__global__ void __launch_bounds__(128) k_ring_dots(Geo g, int pass, const zd *__restrict__ A, const zd *r,
+                                                   double *num, int nrhs) {
+  constexpr int ND = H == 4 ? 5 : 9, NS = H == 1 ? 2 : 1;
+  const int N = g.N, n4 = g.nsites() >> 2;
+  const long tid = (long)blockIdx.x * 128 + threadIdx.x;
+  const int l = (int)(tid % (4 * H)), c = l & 1, t = (l >> 1) & 1;
+  const long q = tid / (4 * H);
+  const int rh = (int)(q % nrhs);
+  const long sp = q / nrhs;
+  const bool act = sp < n4;
+  const int row = pass + 4 * (int)((act ? sp : 0) / N), u = (int)((act ? sp : 0) % N);
+  const int px = (row + u) & (N - 1), py = (row - u) & (N - 1);
+  const zd *Ah = A + (long)g.idx(px, py) * 36 + t * 2;
+  const int s0 = H == 1 ? 0 : (l >> 2) & 1, dh = H == 4 ? (l >> 3) * 5 : 0;  // offsets 0..4 or 5..8
+  zd a[ND][NS];
+#pragma unroll
+  for (int i = 0; i < ND; ++i)
+#pragma unroll
+    for (int s = 0; s < NS; ++s) a[i][s] = dh + i < 9 ? Ah[(dh + i) * 4 + s0 + s] : mk(0.0, 0.0);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+  double acc[NS];
+#pragma unroll
+  for (int s = 0; s < NS; ++s) acc[s] = 0;
+  zd rv[ND][NS];
+#pragma unroll
+  for (int i = 0; i < ND; ++i)
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+      rv[i][s] = r[((long)g.nb(px, py, min(dh + i, 8)) * 2 + s0 + s) * nrhs + rh];
+#pragma unroll
+  for (int i = 0; i < ND; ++i)
+#pragma unroll
+    for (int s = 0; s < NS; ++s) rb_cfma(acc[s], a[i][s], rv[i][s], c);
+  double v;
+  if (H == 1) {
+    v = acc[0] - acc[NS - 1];
+  } else {
+    v = rb_flip(acc[0], s0 != 0);
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    if (H == 4) v += __shfl_xor_sync(0xffffffffu, v, 8);
+  }
+  if (act && l < 4) num[((sp * 2 + t) * nrhs + rh) * 2 + c] = rb_flip(v, t != 0);
+}
+
+// W positions of a ring and C right-hand sides per block, W C 12 threads / NI:
+// the solutions s of the W sites and the two beside them go to shared memory,
+// then every thread sums the update of NI real numbers of r.
+template <int W, int C, int NI>
+__global__ void __launch_bounds__(W *C * 12 / NI) k_ring_update(Geo g, int pass, const zd *__restrict__ A,
+                                                                const zd *__restrict__ T, const double *num,
+                                                                double *x, double *r, int nrhs) {
+  constexpr int NT = W * C * 12 / NI;
+  __shared__ double sm[W + 2][2][C][2];
+  const int N = g.N, seg = N / W, tid = threadIdx.x;
+  const int ring = blockIdx.x / seg, u0 = (blockIdx.x % seg) * W, row = pass + 4 * ring;
+  const int r0 = blockIdx.y * C, Rc = min(C, nrhs - r0);
+  // this thread's numbers of r: component, right-hand side, spin, row of the window, position
+  zd a[NI][6];
+  long ro[NI];
+  bool in[NI];
+#pragma unroll
+  for (int i = 0; i < NI; ++i) {
+    int e = tid + i * NT, cc = (e >> 1) % C, q = (e >> 1) / C, s = q & 1, da = (q >> 1) % 3, uw = (q >> 1) / 3;
+    in[i] = cc < Rc;
+    int ra = row + da - 1, u = u0 + uw;
+    ro[i] = (((long)g.idx(ra + u, ra - u) * 2 + s) * nrhs + r0 + cc) * 2 + (e & 1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {  // the sites at u - 1, u, u + 1: this cell is their offset (da, 1 - k + 1)
+      const zd *p = A + (long)g.idx(row + u + k - 1, row - u - k + 1) * 36 + (da * 3 + 2 - k) * 4 + s;
+      a[i][2 * k] = p[0];
+      a[i][2 * k + 1] = p[2];
+    }
+  }
+  constexpr int NV = ((W + 2) * C * 8 + NT - 1) / NT;  // solution items a thread
+  zd tv[NV][6];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    int e = tid + i * NT, uu = min((e >> 3) / C, W + 1), u = (u0 + uu - 1) & (N - 1);
+    const zd *Tp = T + ((((long)pass * (N / 8) + ring) * N + u) * 2 + ((e >> 1) & 1)) * 12 + ((e >> 2) & 1) * 6;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) tv[i][k] = Tp[k];
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+  double rv[NI];
+#pragma unroll
+  for (int i = 0; i < NI; ++i) rv[i] = in[i] ? r[ro[i]] : 0.0;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int e = tid + i * NT;
+    if (e >= ((W + 2) * C * 8 + 31) / 32 * 32) break;  // whole warps: the halves meet by a shuffle
+    const int l = e & 7, c = l & 1, t = (l >> 1) & 1, hh = l >> 2, cc = (e >> 3) % C, uu = (e >> 3) / C;
+    const bool on = uu < W + 2 && cc < Rc;
+    const int u = (u0 + uu - 1) & (N - 1);
+    double v = 0, xv = 0;
+    double *xa = x + (((long)g.idx(row + u, row - u) * 2 + t) * nrhs + r0 + cc) * 2 + c;
+    const bool mine = on && hh == 0 && uu >= 1 && uu <= W;
+    if (on) {
+      if (mine) xv = *xa;
+      zd nv[6];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        int kk = hh * 6 + k, us = ((u & ~3) + (kk >> 1)) & (N - 1);
+        nv[k] = *(const zd *)(num + ((((long)ring * N + us) * 2 + (kk & 1)) * nrhs + r0 + cc) * 2);
+      }
+#pragma unroll
+      for (int k = 0; k < 6; ++k) rb_cfma(v, tv[i][k], nv[k], c);
+    }
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    if (on && hh == 0) sm[uu][t][cc][c] = v;
+    if (mine) *xa = xv + v;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NI; ++i) {
+    if (!in[i]) continue;
+    int e = tid + i * NT, c = e & 1, cc = (e >> 1) % C, q = (e >> 1) / C, s = q & 1, uw = (q >> 1) / 3;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {  // r -= g_s g_t s_t conj(a)
+        const double *sv = sm[uw + k][t][cc];
+        zd av = a[i][2 * k + t];
+        const bool neg = s == t;  // g_s g_t = 1: subtract
+        rv[i] = fma(rb_flip(av.re, neg), sv[c], rv[i]);
+        rv[i] = fma(rb_flip(av.im, neg == (c == 0)), sv[1 - c], rv[i]);
+      }
+    r[ro[i]] = rv[i];
+  }
+}
+
+// All sweeps of a 32 x 32 or 64 x 64 level in one launch: a cluster of 16 blocks
+// per right-hand side, block (ring group i, segment) holding rows 4 i .. 4 i + 3 of
+// W positions with their stencil rows and T in shared memory, and r with a halo
+// of one row and one position. Inner products and updated values of r that a
+// neighbour's halo holds are stored there as well (distributed shared memory), so
+// that every load is the block's own; a cluster barrier (390 cycles) follows the
+// inner products and another one the update, where the two launches of a pass
+// cost 4.4 us.
+template <int N>
+struct RingCluster {
+  static constexpr int NG = N / 8, SEG = 16 / NG, W = N / SEG, H = N == 32 ? 4 : 2;
+  static constexpr int NT = N == 32 ? 128 : 384;
+  zd A[4][W + 2][36];
+  zd T[4][W + 2][24];
+  zd r[6][W + 2][2];   // rows -1 .. 4, positions -1 .. W
+  zd num[W + 10][2];   // positions -4 .. W + 5 of the ring of the pass
+  zd s[W + 2][2];
+  zd x[4][W][2];
+};
+
+template <int N>
+__global__ void __launch_bounds__(RingCluster<N>::NT) k_ring64_cluster(Geo g, int sweeps, const zd *__restrict__ A,
+                                                                       const zd *__restrict__ T, const zd *rin,
+                                                                       const zd *xin, zd *x, zd *r, int nrhs) {
+  typedef RingCluster<N> C;
+  constexpr int W = C::W, SEG = C::SEG, NG = C::NG, NT = C::NT, H = C::H;
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  C *sm = (C *)sm_raw;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), ig = rank / SEG, u0 = (rank % SEG) * W, tid = threadIdx.x, rh = blockIdx.y;
+  auto site = [&](int row, int u) { return g.idx(row + u, row - u); };
+  for (int e = tid; e < 4 * (W + 2) * 36; e += NT) {
+    int k = e / ((W + 2) * 36), q = e / 36 % (W + 2), c = e % 36;
+    sm->A[k][q][c] = A[(long)site(4 * ig + k, u0 + q - 1) * 36 + c];
+  }
+  for (int e = tid; e < 4 * (W + 2) * 24; e += NT) {
+    int k = e / ((W + 2) * 24), q = e / 24 % (W + 2), c = e % 24, u = (u0 + q - 1) & (N - 1);
+    sm->T[k][q][c] = T[(((long)k * NG + ig) * N + u) * 24 + c];
+  }
+  for (int e = tid; e < 6 * (W + 2) * 2; e += NT) {
+    int k = e / (2 * (W + 2)), q = e / 2 % (W + 2), sp = e & 1;
+    sm->r[k][q][sp] = rin[((long)site(4 * ig + k - 1, u0 + q - 1) * 2 + sp) * nrhs + rh];
+  }
+  for (int e = tid; e < 4 * W * 2; e += NT) {
+    int k = e / (2 * W), w = e / 2 % W, sp = e & 1;
+    sm->x[k][w][sp] = xin ? xin[((long)site(4 * ig + k, u0 + w) * 2 + sp) * nrhs + rh] : mk(0.0, 0.0);
+  }
+  // the blocks beside this one along the rings
+  C *left = cl.map_shared_rank(sm, ig * SEG + (rank + SEG - 1) % SEG);
+  C *right = cl.map_shared_rank(sm, ig * SEG + (rank + 1) % SEG);
+  cl.sync();
+  for (int sw = 0; sw < sweeps; ++sw)
+    for (int k = 0; k < 4; ++k) {
+      if (tid < W * 4 * H) {  // whole warps
+        const int l = tid % (4 * H), w = tid / (4 * H), c = l & 1, t = (l >> 1) & 1, sp = (l >> 2) & 1;
+        const int d0 = H == 4 ? (l >> 3) * 5 : 0, d1 = H == 4 ? min(d0 + 5, 9) : 9;
+        double v = 0;
+#pragma unroll
+        for (int i = 0; i < (H == 4 ? 5 : 9); ++i) {
+          int d = d0 + i;
+          if (d < d1) rb_cfma(v, sm->A[k][w + 1][d * 4 + t * 2 + sp], sm->r[k + d / 3][w + d % 3][sp], c);
+        }
+        v = rb_flip(v, sp != 0);
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
+        if (H == 4) v += __shfl_xor_sync(0xffffffffu, v, 8);
+        if (l < 4) {
+          v = rb_flip(v, t != 0);
+          ((double *)&sm->num[w + 4][t])[c] = v;
+          if (w >= W - 4) ((double *)&right->num[w - W + 4][t])[c] = v;
+          if (w < 6) ((double *)&left->num[w + W + 4][t])[c] = v;
+        }
+      }
+      cl.sync();
+      if (tid < ((W + 2) * 8 + 31) / 32 * 32) {
+        const int l = tid & 7, c = l & 1, t = (l >> 1) & 1, hh = l >> 2, q = min(tid >> 3, W + 1);
+        const int cell = ((q + 3) & ~3) + hh * 3;  // in num: the cell of position q - 1, and the half's first site
+        double v = 0;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) rb_cfma(v, sm->T[k][q][t * 12 + hh * 6 + i], sm->num[cell + (i >> 1)][i & 1], c);
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
+        if (hh == 0) {
+          ((double *)&sm->s[q][t])[c] = v;
+          if ((tid >> 3) == q && q >= 1 && q <= W) ((double *)&sm->x[k][q - 1][t])[c] += v;
+        }
+      }
+      __syncthreads();
+      for (int e = tid; e < W * 12; e += NT) {
+        const int c = e & 1, sp = (e >> 1) & 1, i = (e >> 2) % 3, w = (e >> 2) / 3;
+        double v = ((const double *)&sm->r[k + i][w + 1][sp])[c];
+#pragma unroll
+        for (int q = 0; q < 3; ++q)  // the sites at positions w - 1, w, w + 1
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            const double *sv = (const double *)&sm->s[w + q][t];
+            zd a = sm->A[k][w + q][(i * 3 + 2 - q) * 4 + t * 2 + sp];
+            const bool neg = sp == t;
+            v = fma(rb_flip(a.re, neg), sv[c], v);
+            v = fma(rb_flip(a.im, neg == (c == 0)), sv[1 - c], v);
+          }
+        // to every block whose rows (with halo) hold this cell: its own group and,
+        // for a first or last row, the group before or after (half a turn on past
+        // the last ring); there to the segment and, at its ends, the next one's halo
+        int ro = 4 * ig + k + i - 1, u = u0 + w;
+        if (ro < 0) ro += N / 2, u += N / 2;
+        if (ro >= N / 2) ro -= N / 2, u += N / 2;
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+          int gr = ro >> 2, idx = (ro & 3) + 1, un = u;
+          if (n == 1) {
+            if (idx == 1) gr -= 1, idx = 5;
+            else if (idx == 4) gr += 1, idx = 0;
+            else break;
+            if (gr < 0) gr += NG, un += N / 2;
+            if (gr >= NG) gr -= NG, un += N / 2;
+          }
+          un &= N - 1;
+          const int sg = un / W, p = un % W;
+          ((double *)&cl.map_shared_rank(sm, gr * SEG + sg)->r[idx][p + 1][sp])[c] = v;
+          if (p == 0) ((double *)&cl.map_shared_rank(sm, gr * SEG + (sg + SEG - 1) % SEG)->r[idx][W + 1][sp])[c] = v;
+          if (p == W - 1) ((double *)&cl.map_shared_rank(sm, gr * SEG + (sg + 1) % SEG)->r[idx][0][sp])[c] = v;
+        }
+      }
+      cl.sync();
+    }
+  for (int e = tid; e < 4 * W * 2; e += NT) {
+    int k = e / (2 * W), w = e / 2 % W, sp = e & 1;
+    long o = ((long)site(4 * ig + k, u0 + w) * 2 + sp) * nrhs + rh;
+    r[o] = sm->r[k + 1][w + 1][sp];
+    x[o] = sm->x[k][w][sp];
+  }
+}
+
 namespace wl {
 
 // raise a kernel's dynamic shared-memory limit once per device
@@ -771,6 +1103,112 @@ int rings_sweeps(wl_amg *a, int l, int prec, const void *rin, const void *xin, v
                      : launch_rings<zf, 16>(L, o, rin, xin, x, r, nrhs, sweeps, s);
   return L.N == 32 ? launch_rings<zb, 32>(L, o, rin, xin, x, r, nrhs, sweeps, s)
                    : launch_rings<zb, 16>(L, o, rin, xin, x, r, nrhs, sweeps, s);
+}
+
+// ---- 16-colour sweeps in FP64
+bool rings64_ok(const wl_amg *a, int l, int prec, int nrhs) {
+  const Level &L = a->lev[l];
+  const bool tile = a->prm.kacz_order == 1 && L.N >= 64;
+  return prec == WL_FP64 && !tile && l < a->L - 1 && L.N >= 16 && a->prm.omega > 0.0 && !a->is_twin &&
+         !(a->prm.overlap && nrhs >= 16);
+}
+
+int rings64_prepare(wl_amg *a, int l, int nrhs, cudaStream_t s) {
+  Level &L = a->lev[l];
+  WL_TRY(L.nums.alloc(sizeof(zd) * (size_t)(L.n / 2) * std::max(nrhs, a->cap)));
+  if (L.op64.rows.p) return WL_OK;
+  WL_TRY(L.op64.rows.alloc(sizeof(zd) * (size_t)L.n * 24));
+  k_ring64_pack<<<L.n / 4 / RBP_CELLS, 16 * RBP_CELLS, 0, s>>>(L.geo, L.op64.A.as<zd>(), a->prm.omega,
+                                                              L.op64.rows.as<zd>());
+  wl_count_launches(1);
+  WL_CUDA(cudaGetLastError());
+  return WL_OK;
+}
+
+template <typename... P, typename... Q>
+static int rb_launch(void (*fn)(P...), dim3 grid, int nt, int pdl, cudaStream_t s, Q... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(nt);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = pdl;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  wl_count_launches(1);
+  WL_CUDA(cudaLaunchKernelEx(&cfg, fn, args...));
+  return WL_OK;
+}
+
+template <int N>
+static int launch_cluster(const Level &L, const void *rin, const void *xin, void *x, void *r, int nrhs, int sweeps,
+                          cudaStream_t s) {
+  const size_t smem = sizeof(RingCluster<N>);
+  static std::atomic<unsigned long long> done{0}, wide{0};
+  WL_TRY(rb_smem_limit((const void *)k_ring64_cluster<N>, smem, done));
+  int dev = 0;
+  WL_CUDA(cudaGetDevice(&dev));
+  unsigned long long bit = 1ull << (dev & 63);
+  if (!(wide.load(std::memory_order_acquire) & bit)) {  // clusters of 16 blocks
+    WL_CUDA(cudaFuncSetAttribute((const void *)k_ring64_cluster<N>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    wide.fetch_or(bit, std::memory_order_acq_rel);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(16, nrhs);
+  cfg.blockDim = dim3(RingCluster<N>::NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 16;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  wl_count_launches(1);
+  WL_CUDA(cudaLaunchKernelEx(&cfg, k_ring64_cluster<N>, L.geo, sweeps, (const zd *)L.op64.A.p, (const zd *)L.op64.rows.p,
+                             (const zd *)rin, (const zd *)xin, (zd *)x, (zd *)r, nrhs));
+  return WL_OK;
+}
+
+bool rings64_form(const wl_amg *a, int l, int param) {
+  return param == 0 || (param == 1 && (a->lev[l].N == 32 || a->lev[l].N == 64));
+}
+
+// param 0: two launches a pass; 1: one launch of clusters (32 x 32 and 64 x 64).
+// rin, xin as in rings_sweeps (param 0 takes r and x themselves)
+int rings64_sweeps(wl_amg *a, int l, const void *rin, const void *xin, void *x, void *r, int nrhs, int sweeps, int param,
+                   cudaStream_t s) {
+  Level &L = a->lev[l];
+  if (param == 1)
+    return L.N == 32 ? launch_cluster<32>(L, rin, xin, x, r, nrhs, sweeps, s)
+                     : launch_cluster<64>(L, rin, xin, x, r, nrhs, sweeps, s);
+  const zd *A = L.op64.A.as<zd>(), *T = L.op64.rows.as<zd>();
+  double *num = L.nums.as<double>();
+  const long items = (long)(L.n / 4) * nrhs;
+  // lanes a site: as many as leave at most a warp or so per SM partition
+  const int H = items <= 512 ? 4 : items <= 4096 ? 2 : 1;
+  const dim3 gd((unsigned)((items * 4 * H + 127) / 128));
+  const int rings = L.N / 8;
+  for (int sw = 0; sw < sweeps; ++sw)
+    for (int k = 0; k < 4; ++k) {
+      const int pdl = sw + k > 0;
+      if (H == 4) WL_TRY(rb_launch(k_ring_dots<4>, gd, 128, pdl, s, L.geo, k, A, (const zd *)r, num, nrhs));
+      else if (H == 2) WL_TRY(rb_launch(k_ring_dots<2>, gd, 128, pdl, s, L.geo, k, A, (const zd *)r, num, nrhs));
+      else WL_TRY(rb_launch(k_ring_dots<1>, gd, 128, pdl, s, L.geo, k, A, (const zd *)r, num, nrhs));
+      const double *nm = num;
+      if (nrhs == 1)
+        WL_TRY(rb_launch(k_ring_update<16, 1, 1>, dim3(rings * (L.N / 16)), 192, 1, s, L.geo, k, A, T, nm, (double *)x,
+                         (double *)r, nrhs));
+      else if (nrhs == 2)
+        WL_TRY(rb_launch(k_ring_update<8, 2, 1>, dim3(rings * (L.N / 8)), 192, 1, s, L.geo, k, A, T, nm, (double *)x,
+                         (double *)r, nrhs));
+      else
+        WL_TRY(rb_launch(k_ring_update<8, 4, 2>, dim3(rings * (L.N / 8), (nrhs + 3) / 4), 192, 1, s, L.geo, k, A, T, nm,
+                         (double *)x, (double *)r, nrhs));
+    }
+  return WL_OK;
 }
 
 }  // namespace wl

@@ -111,3 +111,40 @@ def test_small_level_sweeps(hier, nrhs):
     with pytest.raises(W.WilsonAMGError):  # a 64x64 level
         W.amg_kaczmarz_form(amg, 0, z, z.clone(), 1, 1, W.WL_FP32, 5, 0)
     amg.close()
+
+
+@pytest.mark.parametrize("name", ["T128", "deep"])
+@pytest.mark.parametrize("nrhs", [1, 2, 3, 9])
+def test_fp64_ring_sweeps(hier, name, nrhs):
+    """The FP64 forms on every 16-colour level (128x128 down to 16x16; every lane split
+    of the inner products, ragged chunks of right-hand sides) against the oracle, to the bound of
+    the other FP64 forms (1e-13 for one sweep, two here: 2e-13)."""
+    h, op, path = hier[name]
+    for omega in (1.0, 0.8):
+        amg = W.amg_import(op, path, W.amg_params_default(zero_guess=1, omega=omega))
+        for l in range(h.L - 1):
+            n = h.n(l)
+            x0 = 0.1 * np.stack([cgauss(470 + l, r, n) for r in range(nrhs)])
+            r0 = np.stack([cgauss(480 + l, r, n) for r in range(nrhs)])
+            xg, rg = T(x0), T(r0)
+            W.amg_kaczmarz_form(amg, l, xg, rg, nrhs, 2, W.WL_FP64, 6, 0)
+            outs = [(xg, rg)]
+            if h.Nl[l] in (32, 64):  # one launch of clusters
+                xc, rc = T(x0), T(r0)
+                W.amg_kaczmarz_form(amg, l, xc, rc, nrhs, 2, W.WL_FP64, 6, 1)
+                outs.append((xc, rc))
+            if omega == 1.0:
+                ref = [h.kaczmarz(l, x0[r], r0[r], order=O.ORDER_COLOUR, sweeps=2) for r in range(nrhs)]
+                xr, rr = np.stack([a for a, _ in ref]), np.stack([b for _, b in ref])
+            else:
+                xa, ra = T(x0), T(r0)
+                W.amg_kaczmarz_form(amg, l, xa, ra, nrhs, 2, W.WL_FP64, 0, 0)
+                xr, rr = xa.cpu().numpy(), ra.cpu().numpy()
+            for xg, rg in outs:
+                assert rel(xg.cpu().numpy(), xr) <= 2e-13 and rel(rg.cpu().numpy(), rr) <= 2e-13, (l, omega)
+        amg.close()
+    amg = W.amg_import(op, path, W.amg_params_default(zero_guess=1, kacz_order=1))
+    z = T(np.zeros((1, h.n(0)), dtype=complex))
+    with pytest.raises(W.WilsonAMGError):  # a tile-ordered level
+        W.amg_kaczmarz_form(amg, 0, z, z.clone(), 1, 1, W.WL_FP64, 6, 0)
+    amg.close()
