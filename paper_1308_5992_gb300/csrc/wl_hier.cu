@@ -108,72 +108,80 @@ __global__ void k_den_bf16(int n, const zb *__restrict__ A, float *__restrict__ 
   den[tid] = s;
 }
 
-// Gauss-Jordan inversion with partial pivoting, one block; M is overwritten
-// by junk, Inv receives M^-1 (both row major, n x n complex double).
-__global__ void __launch_bounds__(1024) k_gauss_jordan(int n, zd *M, zd *Inv, int *status) {
-  extern __shared__ unsigned char smem_raw[];
-  zd *fac = (zd *)smem_raw;                 // [n]
-  double *bv = (double *)(fac + n);          // [blockDim]
-  int *bi = (int *)(bv + blockDim.x);        // [blockDim]
-  int tid = threadIdx.x, nt = blockDim.x;
-  for (long i = tid; i < (long)n * n; i += nt) Inv[i] = mk((i / n == i % n) ? 1.0 : 0.0, 0.0);
-  __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    double best = -1.0;
-    int bidx = k;
-    for (int i = k + tid; i < n; i += nt) {
-      double v = cnorm2(M[(long)i * n + k]);
-      if (v > best) {
-        best = v;
-        bidx = i;
-      }
-    }
-    bv[tid] = best;
-    bi[tid] = bidx;
-    __syncthreads();
-    for (int s = nt / 2; s > 0; s >>= 1) {
-      if (tid < s && (bv[tid + s] > bv[tid] || (bv[tid + s] == bv[tid] && bi[tid + s] < bi[tid]))) {
-        bv[tid] = bv[tid + s];
-        bi[tid] = bi[tid + s];
-      }
-      __syncthreads();
-    }
-    int p = bi[0];
-    if (bv[0] <= 0.0) {
-      if (tid == 0) *status = 1;
-      return;
-    }
-    if (p != k)
-      for (int j = tid; j < n; j += nt) {
-        zd t = M[(long)k * n + j];
-        M[(long)k * n + j] = M[(long)p * n + j];
-        M[(long)p * n + j] = t;
-        t = Inv[(long)k * n + j];
-        Inv[(long)k * n + j] = Inv[(long)p * n + j];
-        Inv[(long)p * n + j] = t;
-      }
-    __syncthreads();
-    zd piv = M[(long)k * n + k];
-    double d = cnorm2(piv);
-    zd ip = mk(piv.re / d, -piv.im / d);
-    __syncthreads();
-    for (int j = tid; j < n; j += nt) {
-      M[(long)k * n + j] = ip * M[(long)k * n + j];
-      Inv[(long)k * n + j] = ip * Inv[(long)k * n + j];
-    }
-    __syncthreads();
-    for (int i = tid; i < n; i += nt) fac[i] = M[(long)i * n + k];
-    __syncthreads();
-    for (long q = tid; q < (long)n * n; q += nt) {
-      int i = (int)(q / n), j = (int)(q % n);
-      if (i == k) continue;
-      zd f = fac[i];
-      M[q] = M[q] - f * M[(long)k * n + j];
-      Inv[q] = Inv[q] - f * Inv[(long)k * n + j];
-    }
-    __syncthreads();
+// Gauss-Jordan inversion with partial pivoting, one launch per column k: every
+// block finds the pivot of column k itself (n values), and the step goes from
+// one copy of (M | Inv) to another, so no block waits for another one: row i of
+// the result comes from row k, p or i of the source.  A block does a tile of
+// GJ_R rows by GJ_C columns of (M | Inv), but not those left of k, which no later
+// step reads.  The inverse of a 256 x 256 coarsest operator took 57 ms in one
+// block (one SM's FP64 unit: 2 multiply-adds a clock); a step of all SMs takes
+// about 2 us, bound by its own FP64 chain (pivot norm, two divisions, update).
+#define GJ_R 32
+#define GJ_C 32
+__global__ void __launch_bounds__(256) k_gj_step(int n, int k, const zd *__restrict__ Ms, const zd *__restrict__ Is,
+                                                 zd *__restrict__ Md, zd *__restrict__ Id, int *status) {
+  __shared__ unsigned long long wv[8];
+  __shared__ int wi[8];
+  __shared__ zd ips, rowk[GJ_C];
+  const int tid = threadIdx.x;
+  if ((int)(blockIdx.x + 1) * GJ_C <= k) return;  // columns of M that are done with
+  // |M[i][k]|^2 is not negative, so its bits order as an integer; smallest row on ties
+  unsigned long long best = 0;
+  int bi = n;
+  for (int i = k + tid; i < n; i += 256) {
+    double m = cnorm2(Ms[(long)i * n + k]);
+    unsigned long long v = m > 0.0 ? (unsigned long long)__double_as_longlong(m) : 0ull;  // NaN is no pivot
+    if (bi == n || v > best) best = v, bi = i;
   }
-  if (tid == 0) *status = 0;
+  auto better = [&](unsigned long long v, int i) {
+    if (i < n && (bi == n || v > best || (v == best && i < bi))) best = v, bi = i;
+  };
+#pragma unroll
+  for (int off = 16; off; off >>= 1)
+    better(__shfl_xor_sync(0xffffffffu, best, off), __shfl_xor_sync(0xffffffffu, bi, off));
+  if ((tid & 31) == 0) wv[tid >> 5] = best, wi[tid >> 5] = bi;
+  __syncthreads();
+  for (int w = 0; w < 8; ++w) better(wv[w], wi[w]);
+  const int p = bi;
+  if (best == 0ull) {  // singular: reported, the rest is void
+    if (tid == 0) *status = 1;
+    return;
+  }
+  if (tid == 0) {
+    zd piv = Ms[(long)p * n + k];
+    double d = cnorm2(piv);
+    ips = mk(piv.re / d, -piv.im / d);
+  }
+  __syncthreads();
+  const int j0 = blockIdx.x * GJ_C, i0 = blockIdx.y * GJ_R;
+  if (tid < GJ_C && j0 + tid < 2 * n) {
+    int j = j0 + tid;
+    rowk[tid] = ips * (j < n ? Ms[(long)p * n + j] : Is[(long)p * n + j - n]);
+  }
+  __syncthreads();
+  const int jj = tid % GJ_C, j = j0 + jj;
+  if (j >= 2 * n) return;
+  const zd *src = j < n ? Ms : Is;
+  zd *dst = j < n ? Md : Id;
+  const int jc = j < n ? j : j - n;
+#pragma unroll
+  for (int q = 0; q < GJ_R * GJ_C / 256; ++q) {
+    const int i = i0 + tid / GJ_C + q * (256 / GJ_C);
+    if (i >= n) break;
+    const int si = i == k ? p : i == p ? k : i;
+    zd v = rowk[jj];
+    if (i != k) {
+      zd w = src[(long)si * n + jc];
+      cfms(w, Ms[(long)si * n + k], v);
+      v = w;
+    }
+    dst[(long)i * n + jc] = v;
+  }
+}
+
+__global__ void k_identity(int n, zd *I) {
+  long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < (long)n * n) I[e] = mk((e / n == e % n) ? 1.0 : 0.0, 0.0);
 }
 
 // dense coarsest operator from its stencil: M[(h,s),(nb(h,d),t)] += A[h][d][s][t]
@@ -199,23 +207,34 @@ int coarsest_invert(wl_amg *a) {
   Level &C = a->lev[a->L - 1];
   int n = 2 * C.n;
   a->nc = n;
-  DBuf M, st;
-  WL_TRY(M.alloc(sizeof(zd) * n * n));
+  const size_t nn = (size_t)n * n;
+  struct Bufs {  // freed on every way out
+    DBuf M, st;
+    ~Bufs() {
+      M.release();
+      st.release();
+    }
+  } w;
+  DBuf &M = w.M, &st = w.st;
+  WL_TRY(M.alloc(sizeof(zd) * nn * 3));  // two copies of M, the second copy of the inverse
   WL_TRY(st.alloc(sizeof(int)));
   WL_TRY(a->Ainv.alloc(sizeof(zd) * n * n));
   WL_TRY(a->Ainv32.alloc(sizeof(zf) * n * n));
   WL_CUDA(cudaMemsetAsync(M.p, 0, sizeof(zd) * n * n, s));
   k_stencil_dense<<<WL_GRID(C.n, 128), 128, 0, s>>>(C.geo, C.op64.A.as<zd>(), M.as<zd>());
-  size_t sm = sizeof(zd) * n + (sizeof(double) + sizeof(int)) * 1024;
-  WL_CUDA(cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  k_gauss_jordan<<<1, 1024, sm, s>>>(n, M.as<zd>(), a->Ainv.as<zd>(), st.as<int>());
+  // the last step writes Ainv
+  zd *m[2] = {M.as<zd>(), M.as<zd>() + nn}, *v[2] = {M.as<zd>() + 2 * nn, M.as<zd>() + 2 * nn};
+  v[n & 1] = a->Ainv.as<zd>();
+  WL_CUDA(cudaMemsetAsync(st.p, 0, sizeof(int), s));
+  k_identity<<<WL_GRID(nn, 256), 256, 0, s>>>(n, v[0]);
+  for (int k = 0; k < n; ++k)
+    k_gj_step<<<dim3((2 * n + GJ_C - 1) / GJ_C, (n + GJ_R - 1) / GJ_R), 256, 0, s>>>(n, k, m[k & 1], v[k & 1], m[~k & 1],
+                                                                                  v[~k & 1], st.as<int>());
   WL_CUDA(cudaGetLastError());
   k_to_f32<<<WL_GRID((long)n * n, 256), 256, 0, s>>>(a->Ainv.as<zd>(), a->Ainv32.as<zf>(), (long)n * n);
   int hs = 1;
   WL_CUDA(cudaMemcpyAsync(&hs, st.p, sizeof(int), cudaMemcpyDeviceToHost, s));
   WL_CUDA(cudaStreamSynchronize(s));
-  M.release();
-  st.release();
   if (hs) {
     wl_set_error("coarsest operator is singular");
     return WL_BAD_HIERARCHY;

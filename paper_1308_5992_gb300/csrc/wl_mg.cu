@@ -1632,7 +1632,7 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
       for (int i = 0; i < n; ++i) cand.push_back(KTune{nrhs, prec, 4, prm[i], 0.f});
     }
     if (rings64_ok(a, l, prec, nrhs)) {
-      if ((rc = rings64_prepare(a, l, nrhs, s))) break;
+      if ((rc = rings64_prepare(a, l, nrhs, false, s))) break;
       for (int q : {0, 1})
         if (rings64_form(a, l, q)) cand.push_back(KTune{nrhs, prec, 6, q, 0.f});
     }
@@ -1907,7 +1907,7 @@ static int kaczmarz_entry(wl_amg *a, int level, void *x, void *r, int nrhs, int 
     WL_TRY(wl::rows_sweeps(a, level, prec, sb.b[0].p, sb.b[1].p, nrhs, sweeps, param, s));
   } else if (rings64) {
     WL_TRY(wl::ensure_workspace(a, nrhs, prec));
-    WL_TRY(wl::rings64_prepare(a, level, nrhs, s));
+    WL_TRY(wl::rings64_prepare(a, level, nrhs, false, s));
     if (sweeps > 0)
       WL_TRY(wl::rings64_sweeps(a, level, sb.b[1].p, sb.b[0].p, sb.b[0].p, sb.b[1].p, nrhs, sweeps, param, s));
   } else if (rings) {

@@ -1113,10 +1113,10 @@ bool rings64_ok(const wl_amg *a, int l, int prec, int nrhs) {
          !(a->prm.overlap && nrhs >= 16);
 }
 
-int rings64_prepare(wl_amg *a, int l, int nrhs, cudaStream_t s) {
+int rings64_prepare(wl_amg *a, int l, int nrhs, bool stale, cudaStream_t s) {
   Level &L = a->lev[l];
   WL_TRY(L.nums.alloc(sizeof(zd) * (size_t)(L.n / 2) * std::max(nrhs, a->cap)));
-  if (L.op64.rows.p) return WL_OK;
+  if (L.op64.rows.p && !stale) return WL_OK;
   WL_TRY(L.op64.rows.alloc(sizeof(zd) * (size_t)L.n * 24));
   k_ring64_pack<<<L.n / 4 / RBP_CELLS, 16 * RBP_CELLS, 0, s>>>(L.geo, L.op64.A.as<zd>(), a->prm.omega,
                                                               L.op64.rows.as<zd>());

@@ -233,6 +233,61 @@ __global__ void k_ls_fit(Geo gf, Geo gc, int lgB, const zd *__restrict__ W, cons
   for (int a = 0; a < nc; ++a) out[idx[a]] = p[a];
 }
 
+// The terms of a Galerkin block (hc, d) are the same for every coarse site: fine
+// point i = (da, db) relative to the C point (B - 1 each way), its neighbour at
+// offset df, the corner ki of i's cell that is hc and the corner kj of the
+// neighbour's cell that is nb(hc, d).  Lists of them per d, packed
+// (da + 4) | (db + 4) << 4 | df << 8 | ki << 12 | kj << 14, in the order of
+// k_galerkin; first[d] .. first[d + 1] belong to d.
+static std::vector<unsigned short> galerkin_terms(int B, int *first) {
+  std::vector<unsigned short> out;
+  for (int d = 0; d < 9; ++d) {
+    first[d] = (int)out.size();
+    for (int da = -(B - 1); da <= B - 1; ++da)
+      for (int db = -(B - 1); db <= B - 1; ++db)
+        for (int df = 0; df < 9; ++df) {
+          int ja = da + df / 3 - 1, jb = db + df % 3 - 1;
+          int a0 = (ja + 2 * B) / B - 2, b0 = (jb + 2 * B) / B - 2;  // floor
+          for (int kj = 0; kj < 4; ++kj) {
+            int ka = kj & 1, kb = kj >> 1;
+            if ((ka && ja == a0 * B) || (kb && jb == b0 * B)) continue;
+            if (a0 + ka != d / 3 - 1 || b0 + kb != d % 3 - 1) continue;
+            int ki = (da < 0 ? 1 : 0) + (db < 0 ? 2 : 0);
+            out.push_back((unsigned short)((da + 4) | (db + 4) << 4 | df << 8 | ki << 12 | kj << 14));
+          }
+        }
+  }
+  first[9] = (int)out.size();
+  return out;
+}
+
+// Galerkin product from those lists, a thread per (hc, d, s, t): 36 threads a
+// coarse site instead of 9, and no search for the neighbour's corner (k_galerkin
+// tests 4 corners for each of 9 (2 B - 1)^2 neighbours, 1764 at B = 4, for the
+// 110 terms of a block).  256 x 256 to 64 x 64: 1.95 ms before.  Needs the nine
+// neighbours of a coarse site to be distinct (N_c >= 8).
+__global__ void __launch_bounds__(128) k_galerkin_list(Geo gf, Geo gc, int lgB, const int *__restrict__ first,
+                                                       const unsigned short *__restrict__ term,
+                                                       const zd *__restrict__ A, const zd *__restrict__ P,
+                                                       zd *__restrict__ Ac) {
+  const int nc = gc.nsites();
+  long tid = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (tid >= (long)nc * 36) return;
+  const int hc = (int)(tid % nc), q = (int)(tid / nc), d = q >> 2, s = (q >> 1) & 1, t = q & 1;
+  int xc, yc;
+  gc.xy(hc, xc, yc);
+  const int X = xc << lgB, Y = yc << lgB;
+  zd acc = mk(0.0, 0.0);
+  for (int e = first[d]; e < first[d + 1]; ++e) {
+    const int w = term[e], da = (w & 15) - 4, db = ((w >> 4) & 15) - 4, df = (w >> 8) & 15, ki = (w >> 12) & 3, kj = w >> 14;
+    const int ix = X + da + db, iy = Y + da - db, dfa = df / 3 - 1, dfb = df % 3 - 1;
+    const long hi = gf.idx(ix, iy), hj = gf.idx(ix + dfa + dfb, iy + dfa - dfb);
+    zd v = A[(hi * 9 + df) * 4 + s * 2 + t] * P[hj * 8 + t * 4 + kj];
+    cfmac(acc, P[hi * 8 + s * 4 + ki], v);
+  }
+  Ac[((long)hc * 9 + d) * 4 + s * 2 + t] = acc;
+}
+
 // Galerkin block (hc, d): sum over fine i in the box of hc and fine
 // neighbours j of i whose cell has nb(hc, d) as a corner:
 //   Ac[hc][d][s][t] = sum conj(P[i][s][k_i]) A[i][df][s][t] P[j][t][k_j]
@@ -375,6 +430,8 @@ struct Setup {
   DBuf red, dots, coef, W, wts;
   cudaStream_t s;
   cusolverDnHandle_t cs = nullptr;
+  DBuf first[2], term[2];       // Galerkin term lists for cells of 2 and 4
+  bool stale[8] = {};           // the level's operator changed since its row-block inverses were made
 };
 
 static int n2of(wl_amg *a, int l) { return a->lev[l].n * 2; }
@@ -435,13 +492,47 @@ static int ritz(Setup &S, int l, const zd *v, int k, std::vector<double> &lam, s
   return WL_OK;
 }
 
+// coarse operator P^H A P of level l + 1 from A on level l
+static int galerkin(Setup &S, int l, const zd *A, zd *Ac) {
+  Level &F = S.a->lev[l], &Cl = S.a->lev[l + 1];
+  const int lgB = ilog2(F.B);
+  if (Cl.N < 8) {
+    k_galerkin<<<WL_GRID(Cl.n * 9, 64), 64, 0, S.s>>>(F.geo, Cl.geo, lgB, A, F.op64.P.as<zd>(), Ac);
+    return WL_OK;
+  }
+  DBuf &fb = S.first[lgB - 1], &tb = S.term[lgB - 1];
+  if (!tb.p) {
+    int first[10];
+    std::vector<unsigned short> t = galerkin_terms(F.B, first);
+    WL_TRY(fb.alloc(sizeof(first)));
+    WL_TRY(tb.alloc(sizeof(unsigned short) * t.size()));
+    WL_CUDA(cudaMemcpyAsync(fb.p, first, sizeof(first), cudaMemcpyHostToDevice, S.s));
+    WL_CUDA(cudaMemcpyAsync(tb.p, t.data(), sizeof(unsigned short) * t.size(), cudaMemcpyHostToDevice, S.s));
+    WL_CUDA(cudaStreamSynchronize(S.s));  // the host lists go out of scope
+  }
+  k_galerkin_list<<<WL_GRID((long)Cl.n * 36, 128), 128, 0, S.s>>>(F.geo, Cl.geo, lgB, fb.as<int>(),
+                                                                 tb.as<unsigned short>(), A, F.op64.P.as<zd>(), Ac);
+  return WL_OK;
+}
+
+// the setup's relaxations: the FP64 row-block sweeps (wl_rows.cu), whose
+// triangular inverses follow the level's operator
+static int setup_sweeps(Setup &S, int l, zd *V, zd *r, int k, int sweeps) {
+  wl_amg *a = S.a;
+  if (sweeps <= 0) return WL_OK;
+  if (!(a->prm.omega > 0.0) || a->lev[l].N < 16) return wl::kaczmarz_sweeps(a, l, WL_FP64, V, r, k, sweeps, S.s);
+  WL_TRY(wl::rings64_prepare(a, l, k, S.stale[l], S.s));
+  S.stale[l] = false;
+  return wl::rings64_sweeps(a, l, r, V, V, r, k, sweeps, a->lev[l].N == 32, S.s);
+}
+
 // Eq. 3.6: Kaczmarz on A_l v = 0
 static int relax_homog(Setup &S, int l, zd *V, int k, int sweeps) {
   if (sweeps <= 0 || k <= 0) return WL_OK;
   wl_amg *a = S.a;
   SetupLevel &SL = S.S[l];
   WL_TRY(wl::stencil_apply(a, l, WL_FP64, V, SL.tmp1.p, SL.zero.p, k, S.s));
-  return wl::kaczmarz_sweeps(a, l, WL_FP64, V, SL.tmp1.p, k, sweeps, S.s);
+  return setup_sweeps(S, l, V, SL.tmp1.as<zd>(), k, sweeps);
 }
 
 // Thm. 3.1 (ii): Kaczmarz on A_l v = lambda Gamma5 T_l v, rhs frozen per
@@ -460,7 +551,7 @@ static int relax_eig(Setup &S, int l, int sweeps) {
     WL_CUDA(cudaMemcpyAsync(S.coef.p, SL.lam.data(), sizeof(double) * k, cudaMemcpyHostToDevice, S.s));
     k_scale_vec<<<WL_GRID(n2 * k, 256), 256, 0, S.s>>>(SL.tmp2.as<zd>(), SL.tmp2.as<zd>(), S.coef.as<double>(), n2 / 2, k, 1);
     WL_TRY(wl::stencil_apply(a, l, WL_FP64, V, SL.tmp1.p, SL.tmp2.p, k, S.s));
-    WL_TRY(wl::kaczmarz_sweeps(a, l, WL_FP64, V, SL.tmp1.p, k, 1, S.s));
+    WL_TRY(setup_sweeps(S, l, V, SL.tmp1.as<zd>(), k, 1));
     WL_TRY(ritz(S, l, V, k, SL.lam, tn));
   }
   std::vector<double> lam2;
@@ -506,12 +597,12 @@ static int fit_level(Setup &S, int l) {
   int lgB = ilog2(F.B);
   k_ls_fit<<<WL_GRID(2 * F.n, 128), 128, 0, S.s>>>(F.geo, Cl.geo, lgB, S.W.as<zd>(), S.wts.as<double>() + 64, k,
                                                    F.op64.P.as<zd>());
-  k_galerkin<<<WL_GRID(Cl.n * 9, 64), 64, 0, S.s>>>(F.geo, Cl.geo, lgB, F.op64.A.as<zd>(), F.op64.P.as<zd>(),
-                                                    Cl.op64.A.as<zd>());
+  WL_TRY(galerkin(S, l, F.op64.A.as<zd>(), Cl.op64.A.as<zd>()));
+  S.stale[l + 1] = true;
   WL_TRY(wl::symmetrise_stencil(Cl.N, Cl.op64.A.as<zd>(), S.s));
   WL_TRY(wl::compute_den64(Cl.N, Cl.op64.A.as<zd>(), Cl.op64.den.as<double>(), S.s));
   const zd *Tf = S.S[l].T.as<zd>();
-  k_galerkin<<<WL_GRID(Cl.n * 9, 64), 64, 0, S.s>>>(F.geo, Cl.geo, lgB, Tf, F.op64.P.as<zd>(), S.S[l + 1].T.as<zd>());
+  WL_TRY(galerkin(S, l, Tf, S.S[l + 1].T.as<zd>()));
   k_herm_stencil<<<WL_GRID(Cl.n * 5, 128), 128, 0, S.s>>>(Cl.geo, S.S[l + 1].T.as<zd>());
   WL_CUDA(cudaGetLastError());
   WL_CUDA(cudaStreamSynchronize(S.s));
@@ -682,12 +773,23 @@ static int adaptive_step(Setup &S) {
   a->prm.cycle = WL_CYCLE_W;
   Level &L0 = a->lev[0];
   int rc = WL_OK;
+  // its sweeps take the row-block form, as the setup's own relaxations, whatever
+  // form the solve phase asks for
+  a->prm.sweep_kernel = 0;
+  if (a->prm.omega > 0.0)
+    for (int l = 0; l < a->L - 1 && !rc; ++l) {
+      if (a->lev[l].N < 16) continue;
+      rc = wl::rings64_prepare(a, l, 1, S.stale[l], S.s);
+      S.stale[l] = false;
+      a->lev[l].rowtune.push_back(KTune{1, WL_FP64, 6, a->lev[l].N == 32, 1.f});
+    }
   for (int it = 0; it < 2 && !rc; ++it) {
     k_get_col<<<WL_GRID(n2, 256), 256, 0, S.s>>>(Vb, S.S[0].tmp2.as<zd>(), n2, kb, qb, 1.0);
     rc = wl::stencil_apply(a, 0, WL_FP64, S.S[0].tmp2.p, L0.f.p, S.S[0].zero.p, 1, S.s);  // f = -A v
     if (!rc) rc = wl::cycle_direct(a, 1, WL_FP64, S.s);
     if (!rc) k_axpy_col<<<WL_GRID(n2, 256), 256, 0, S.s>>>(Vb, L0.x.as<zd>(), n2, kb, qb);
   }
+  for (int l = 0; l < a->L; ++l) a->lev[l].rowtune.clear();
   a->prm = save;
   WL_TRY(rc);
   // T-normalise the updated vector (T_0 = I) and refresh its Ritz value
@@ -771,6 +873,11 @@ extern "C" int amg_setup(wl_op *op, const amg_params *params, wl_amg **out) {
                                      : visit(S, 1, false, prm.setup_mu[1]);
   if (!rc) rc = interp_e(S, 0);
   a->prm.kacz_order = prm.kacz_order;
+  cudaStreamSynchronize(S.s);
+  for (int l = 0; l < a->L; ++l) {  // made again on first use, from the final operators
+    a->lev[l].op64.rows.release();
+    a->lev[l].nums.release();
+  }
   if (!rc) rc = wl::hier_finish(a);
   if (S.cs) cusolverDnDestroy(S.cs);
   cudaStreamSynchronize(S.s);
@@ -786,6 +893,10 @@ extern "C" int amg_setup(wl_op *op, const amg_params *params, wl_amg **out) {
   S.coef.release();
   S.W.release();
   S.wts.release();
+  for (int i = 0; i < 2; ++i) {
+    S.first[i].release();
+    S.term[i].release();
+  }
   if (rc) {
     wl::amg_free(a);
     return rc;
