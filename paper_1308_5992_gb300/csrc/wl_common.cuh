@@ -323,8 +323,9 @@ int cycle_run(wl_amg *a, int nrhs, int prec, cudaStream_t s);  // lev[0].f -> le
 int cycle_prepare(wl_amg *a, int nrhs, int prec, cudaStream_t s, const wl_amg::G **out);  // capture only
 int cycle_direct(wl_amg *a, int nrhs, int prec, cudaStream_t s);
 int dhat_apply_dev(wl_op *op, const void *x, int x_is_f32, zd *y, int nrhs, cudaStream_t s);
-int stencil_apply32_to64(wl_amg *a, const void *x, zd *y, int nrhs, cudaStream_t s);
-int stencil_apply32_to_df(wl_amg *a, const void *x, zdf *y, int nrhs, cudaStream_t s);  // lo = 0
+// xo (or NULL): receives a copy of x
+int stencil_apply32_to64(wl_amg *a, const void *x, zd *y, int nrhs, zf *xo, cudaStream_t s);
+int stencil_apply32_to_df(wl_amg *a, const void *x, zdf *y, int nrhs, zf *xo, cudaStream_t s);  // lo = 0
 int stencil_apply(wl_amg *a, int l, int prec, const void *x, void *y, const void *f, int nrhs,
                   cudaStream_t s);
 int kaczmarz_sweeps(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int sweeps,

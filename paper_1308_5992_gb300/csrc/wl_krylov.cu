@@ -156,21 +156,33 @@ static void launch_mdot(int kc, int nblk, int nt, size_t sm, cudaStream_t s, con
   }
 }
 
-// out[r][k0 + k] (= or +=) sum over blocks of part[b][k][r]: one warp per
-// (k, r), lanes stride the blocks, shuffle tree (fixed order: deterministic)
-__global__ void k_mdot_final(const zd *__restrict__ part, int nblk, int kc, int R, zd *out, int ostride,
-                             int k0, int accumulate, zd *copy_to) {
-  int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (wid >= kc * R) return;
-  int k = wid / R, r = wid % R;
+// Sums of block partials: one block of FIN_T threads per (k, r), thread t taking
+// the blocks t, t + FIN_T, ...; shuffles and the warps' sums in a fixed order
+// (deterministic).  With at most 608 partials a thread adds 5 of them: a warp per
+// (k, r) added 19 each, 9 us of dependent FP64 or double-float sums.
+#define FIN_T 128
+
+// out[r][k0 + k] (= or +=) sum over blocks of part[b][k][r]; re (or NULL) gets the
+// real part, and with reset the counters of k_givens are zeroed
+__global__ void __launch_bounds__(FIN_T) k_mdot_final(const zd *__restrict__ part, int nblk, int kc, int R, zd *out,
+                                                      int ostride, int k0, int accumulate, zd *copy_to, double *re,
+                                                      int *reset) {
+  __shared__ zd ws[FIN_T / 32];
+  const int k = blockIdx.x / R, r = blockIdx.x % R;
   zd s = mk(0.0, 0.0);
-  for (int b = lane; b < nblk; b += 32) s = s + part[((long)b * kc + k) * R + r];
+  for (int b = threadIdx.x; b < nblk; b += FIN_T) s = s + part[((long)b * kc + k) * R + r];
 #pragma unroll
   for (int off = 16; off; off >>= 1) {
     s.re += __shfl_down_sync(0xffffffffu, s.re, off);
     s.im += __shfl_down_sync(0xffffffffu, s.im, off);
   }
-  if (lane) return;
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x) return;
+  s = (ws[0] + ws[1]) + (ws[2] + ws[3]);
+  if (reset && blockIdx.x == 0) reset[0] = reset[1] = 0;
+  if (re) re[r] = s.re;
+  if (!out) return;
   zd *o = out + (long)r * ostride + k0 + k;
   if (copy_to) copy_to[(long)(k0 + k) * R + r] = s;  // rhs innermost
   *o = accumulate ? (*o + s) : s;
@@ -372,16 +384,16 @@ __device__ __forceinline__ void put_coef_df(float4 *c, zd s) {
   c[1] = make_float4(cim.x, -cim.x, cim.y, -cim.y);
 }
 
-// the sums of k_mdot_df over blocks, one warp per (k, r) in a fixed order,
-// converted to FP64: out[r][k0 + k] (= or +=) V_k^H w; with coef, the
-// coefficients for k_maxpy_df: {crh, crh, crl, crl} and {cih, -cih, cil, -cil}
-__global__ void k_mdot_final_df(const float4 *__restrict__ part, int nblk, int kc, int R, zd *out, int ostride,
-                                int k0, int accumulate, float4 *coef) {
-  int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (wid >= kc * R) return;
-  int k = wid / R, r = wid % R;
+// the sums of k_mdot_df over blocks as k_mdot_final takes them, converted to
+// FP64: out[r][k0 + k] (= or +=) V_k^H w; with coef, the coefficients for
+// k_maxpy_df: {crh, crh, crl, crl} and {cih, -cih, cil, -cil}; re and reset as there
+__global__ void __launch_bounds__(FIN_T) k_mdot_final_df(const float4 *__restrict__ part, int nblk, int kc, int R,
+                                                         zd *out, int ostride, int k0, int accumulate, float4 *coef,
+                                                         double *re, int *reset) {
+  __shared__ float4 ws[FIN_T / 32][2];
+  const int k = blockIdx.x / R, r = blockIdx.x % R;
   DF2 A{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, B = A;
-  for (int b = lane; b < nblk; b += 32) {
+  for (int b = threadIdx.x; b < nblk; b += FIN_T) {
     const float4 *p = part + (((long)b * kc + k) * R + r) * 2;
     float4 x = p[0], y = p[1];
     df_add(A, DF2{make_float2(x.x, x.y), make_float2(x.z, x.w)});
@@ -401,9 +413,22 @@ __global__ void k_mdot_final_df(const float4 *__restrict__ part, int nblk, int k
     df_add(A, a2);
     df_add(B, b2);
   }
-  if (lane) return;
+  if ((threadIdx.x & 31) == 0) {
+    ws[threadIdx.x >> 5][0] = make_float4(A.s.x, A.s.y, A.c.x, A.c.y);
+    ws[threadIdx.x >> 5][1] = make_float4(B.s.x, B.s.y, B.c.x, B.c.y);
+  }
+  __syncthreads();
+  if (threadIdx.x) return;
+  for (int w = 1; w < FIN_T / 32; ++w) {
+    float4 x = ws[w][0], y = ws[w][1];
+    df_add(A, DF2{make_float2(x.x, x.y), make_float2(x.z, x.w)});
+    df_add(B, DF2{make_float2(y.x, y.y), make_float2(y.z, y.w)});
+  }
   zd s = mk(((double)A.s.x + (double)A.s.y) + ((double)A.c.x + (double)A.c.y),
             ((double)B.s.x - (double)B.s.y) + ((double)B.c.x - (double)B.c.y));
+  if (reset && blockIdx.x == 0) reset[0] = reset[1] = 0;
+  if (re) re[r] = s.re;
+  if (!out) return;
   zd *o = out + (long)r * ostride + k0 + k;
   *o = accumulate ? (*o + s) : s;
   if (coef) put_coef_df(coef + ((long)(k0 + k) * R + r) * 2, s);
@@ -561,51 +586,83 @@ __global__ void k_scale_first_df(const zd *__restrict__ in, zdf *__restrict__ ou
 }
 
 // ------------------------------------------------------------------ Givens
-// column j of the Arnoldi process for every active right-hand side
-__global__ void k_givens(KS k, int j, double tol) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= k.nrhs) return;
-  int m = k.m;
-  if (!k.active[r] || k.stop[r]) {
+// v with its sign flipped where `neg`, on the integer pipe (a run-time negation
+// would go through the FP64 unit)
+__device__ __forceinline__ double flip(double v, bool neg) {
+  return __hiloint2double(__double2hiint(v) ^ (neg ? (int)0x80000000 : 0), __double2loint(v));
+}
+
+// Column j of the Arnoldi process for every active right-hand side, four lanes
+// each.  A chain of FP64 instructions, 64 cycles apiece: lane (o, c) computes
+// component c of the rotation's output o (o = 0: the entry of R, o = 1: the one
+// the next rotation takes), and the new rotation's four divisions are one per
+// lane (one thread per right-hand side took 10 to 17 us).
+__global__ void __launch_bounds__(128) k_givens(KS k, int j, double tol) {
+  const int id = blockIdx.x * 128 + threadIdx.x, r = id >> 2, l = id & 3, c = l & 1, o = l >> 1;
+  const unsigned mask = 0xffffffffu;
+  const bool in = r < k.nrhs;
+  const bool run = in && k.active[r] && !k.stop[r];
+  if (in && !run && l == 0) {
     k.inv[r] = 0.0;
     k.invdf[r] = make_float2(0.f, 0.f);
-    return;
   }
-  zd *hc = k.hcol + (long)r * (m + 1);
-  double hn = sqrt(fmax(k.nrm2[r], 0.0));
-  hc[j + 1] = mk(hn, 0.0);
-  zd *cs = k.cs + (long)r * m;
-  double *cc = k.cc + (long)r * m;
-  for (int i = 0; i < j; ++i) {
-    zd a = hc[i], b = hc[i + 1];
-    zd t = cc[i] * a + cs[i] * b;
-    hc[i + 1] = mk(0.0, 0.0) - cconj(cs[i]) * a + cc[i] * b;
-    hc[i] = t;
+  if (!__any_sync(mask, run)) return;
+  const int m = k.m, rr = run ? r : 0;
+  zd *hc = k.hcol + (long)rr * (m + 1);
+  zd *cs = k.cs + (long)rr * m;
+  double *cc = k.cc + (long)rr * m;
+  zd *g = k.g + (long)rr * (m + 1);
+  zd *H = k.H + (long)rr * (m + 1) * m;
+  const double hn = run ? sqrt(fmax(k.nrm2[rr], 0.0)) : 0.0;
+  // a: the entry the rotations carry on; own component and the other one
+  double a = run ? ((const double *)hc)[c] : 0.0, ao = run ? ((const double *)hc)[1 - c] : 0.0;
+  for (int i0 = 0; i0 < j; i0 += 8) {  // the data of 8 rotations at a time, then their chain
+    double ci[8], sr[8], si[8], b[8], bo[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int i = i0 + q;
+      const bool on = run && i < j;
+      ci[q] = on ? cc[i] : 0.0;
+      sr[q] = on ? flip(cs[i].re, o != 0) : 0.0;
+      si[q] = on ? flip(cs[i].im, c == 0) : 0.0;
+      b[q] = on ? ((const double *)(hc + i + 1))[c] : 0.0;
+      bo[q] = on ? ((const double *)(hc + i + 1))[1 - c] : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int i = i0 + q;
+      if (i >= j) break;
+      // o = 0: cc a + cs b; o = 1: cc b - conj(cs) a: component c of s y is
+      // s.re y_c -+ s.im y_(1-c) (minus for c = 0), of conj(s) y with +-
+      double v = fma(sr[q], o ? a : b[q], ci[q] * (o ? b[q] : a));
+      v = fma(si[q], o ? ao : bo[q], v);
+      if (run && o == 0) ((double *)(H + i * m + j))[c] = v;
+      // the next rotation's a: output 1, both components
+      a = __shfl_sync(mask, v, (threadIdx.x & 28) | 2 | c);
+      ao = __shfl_sync(mask, v, (threadIdx.x & 28) | 2 | (1 - c));
+    }
   }
-  double aa = sqrt(cnorm2(hc[j])), bb = hn;
-  double den = sqrt(aa * aa + bb * bb);
-  zd *g = k.g + (long)r * (m + 1);
-  if (den == 0.0) {
-    cc[j] = 1.0;
-    cs[j] = mk(0.0, 0.0);
-  } else if (aa == 0.0) {
-    cc[j] = 0.0;
-    cs[j] = mk(1.0, 0.0);
-  } else {
-    cc[j] = aa / den;
-    zd ph = mk(hc[j].re / aa, hc[j].im / aa);
-    cs[j] = (bb / den) * ph;  // conj(h_{j+1}) = h_{j+1} (real)
-  }
-  hc[j] = cc[j] * hc[j] + cs[j] * hc[j + 1];
-  hc[j + 1] = mk(0.0, 0.0);
+  const double are = c ? ao : a, aim = c ? a : ao;
+  const double a2 = are * are + aim * aim, aa = sqrt(a2), bb = hn, den = sqrt(a2 + bb * bb);
+  // one division a lane: Re(h) / |h|, Im(h) / |h|, |h| / den, bb / den
+  const double q = (l == 0 ? are : l == 1 ? aim : l == 2 ? aa : bb) / (l < 2 ? aa : den);
+  const int base = threadIdx.x & 28;
+  double pr = __shfl_sync(mask, q, base), pi = __shfl_sync(mask, q, base | 1), cj = __shfl_sync(mask, q, base | 2),
+         bd = __shfl_sync(mask, q, base | 3);
+  double sr = bd * pr, si = bd * pi;
+  if (den == 0.0) cj = 1.0, sr = si = 0.0;
+  else if (aa == 0.0) cj = 0.0, sr = 1.0, si = 0.0;
+  if (!run || l) return;
+  cc[j] = cj;
+  cs[j] = mk(sr, si);
+  H[j * m + j] = cj * mk(are, aim) + bb * mk(sr, si);
   zd gj = g[j];
-  g[j + 1] = mk(0.0, 0.0) - cconj(cs[j]) * gj;
-  g[j] = cc[j] * gj;
-  zd *H = k.H + (long)r * (m + 1) * m;
-  for (int i = 0; i <= j; ++i) H[i * m + j] = hc[i];
+  zd gn = mk(0.0, 0.0) - cconj(cs[j]) * gj;
+  g[j + 1] = gn;
+  g[j] = cj * gj;
   k.iters[r] += 1;
   k.jend[r] = j + 1;
-  double res = sqrt(cnorm2(g[j + 1]));
+  double res = sqrt(cnorm2(gn));
   bool bad = !isfinite(res);
   bool done = !(res > tol * k.bnorm[r]) || hn == 0.0 || bad;
   if (bad) {  // NaN / Inf seen: this right-hand side stops; the others go on
@@ -619,28 +676,31 @@ __global__ void k_givens(KS k, int j, double tol) {
 }
 
 // y = H^-1 g (upper triangular, jend columns), zero beyond jend / inactive
-// (with df, y also as double-float coefficients for k_xupd_df, in hpd)
-__global__ void k_trisolve(KS k, int df) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
+// (with df, y also as double-float coefficients for k_xupd_df, in hpd).  A warp
+// per right-hand side, lane i (m <= 32) holding row i: the diagonal's squared
+// norms are inverted at once, then each y_i is taken off the rows above it (one
+// thread per right-hand side took 22 to 50 us).
+__global__ void __launch_bounds__(128) k_trisolve(KS k, int df) {
+  const int r = (blockIdx.x * 128 + threadIdx.x) >> 5, i = threadIdx.x & 31;
   if (r >= k.nrhs) return;
-  int m = k.m, je = k.active[r] ? k.jend[r] : 0;
+  const int m = k.m, je = k.active[r] ? k.jend[r] : 0;
   const zd *H = k.H + (long)r * (m + 1) * m;
-  const zd *g = k.g + (long)r * (m + 1);
-  zd *y = k.y + (long)r * m;
-  for (int i = m - 1; i >= 0; --i) {
-    if (i >= je) {
-      y[i] = mk(0.0, 0.0);
-      continue;
-    }
-    zd s = g[i];
-    for (int q = i + 1; q < je; ++q) s = s - H[i * m + q] * y[q];
-    zd d = H[i * m + i];
-    double dn = cnorm2(d);
-    y[i] = (dn > 0) ? mk((s.re * d.re + s.im * d.im) / dn, (s.im * d.re - s.re * d.im) / dn) : mk(0.0, 0.0);
+  const bool row = i < je;
+  zd s = row ? k.g[(long)r * (m + 1) + i] : mk(0.0, 0.0);
+  zd d = row ? H[i * m + i] : mk(0.0, 0.0);
+  const double dn = cnorm2(d);
+  const double inv = dn > 0 ? 1.0 / dn : 0.0;
+  zd y = mk(0.0, 0.0);
+  for (int q = je - 1; q >= 0; --q) {
+    zd h = i < q ? H[i * m + q] : mk(0.0, 0.0);
+    if (i == q) y = inv * cmulc(d, s);
+    zd yq = mk(__shfl_sync(0xffffffffu, y.re, q), __shfl_sync(0xffffffffu, y.im, q));
+    if (i < q) cfms(s, h, yq);
   }
-  for (int i = 0; i < m; ++i) k.yT[(long)i * k.nrhs + r] = y[i];
-  if (df)
-    for (int i = 0; i < m; ++i) put_coef_df(k.hpd + ((long)i * k.nrhs + r) * 2, y[i]);
+  if (i >= m) return;
+  k.y[(long)r * m + i] = y;
+  k.yT[(long)i * k.nrhs + r] = y;
+  if (df) put_coef_df(k.hpd + ((long)i * k.nrhs + r) * 2, y);
 }
 
 // start of a cycle: beta = ||r||, inv = active ? 1/beta : 0, g = (beta, 0..)
@@ -660,23 +720,12 @@ __global__ void k_cycle_start(KS k) {
   for (int i = 0; i <= m; ++i) k.hcol[(long)r * (m + 1) + i] = mk(0.0, 0.0);
 }
 
-__global__ void k_zero_hcol(KS k) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= k.nrhs) return;
-  for (int i = 0; i <= k.m; ++i) k.hcol[(long)r * (k.m + 1) + i] = mk(0.0, 0.0);
-}
-
 // zero the entries (and squared norm) of the right-hand sides flagged in mask
 __global__ void k_zero_masked(zd *__restrict__ v, long E, int R, const int *__restrict__ mask,
                               double *__restrict__ nrm2) {
   long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e < E && mask[e % R]) v[e] = mk(0.0, 0.0);
   if (e < R && mask[e]) nrm2[e] = 0.0;
-}
-
-__global__ void k_re_of(const zd *a, double *b, int n) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) b[i] = a[i].re;
 }
 
 namespace wl {
@@ -707,8 +756,8 @@ static int mdots(wl_amg *a, const cx<Tv> *V, long vstride, int kc, const zd *w, 
     size_t sm = sizeof(zd) * kk * c.nt;
     wl_count_launches(2);
     launch_mdot<Tv>(kk, c.nblk, c.nt, sm, s, V + k0 * vstride, vstride, w, E, R, a->red.as<zd>());
-    k_mdot_final<<<WL_GRID(kk * R * 32, 256), 256, 0, s>>>(a->red.as<zd>(), c.nblk, kk, R, out, ostride, k0,
-                                                           accumulate, copy_to);
+    k_mdot_final<<<kk * R, FIN_T, 0, s>>>(a->red.as<zd>(), c.nblk, kk, R, out, ostride, k0, accumulate, copy_to,
+                                          nullptr, nullptr);
   }
   WL_CUDA(cudaGetLastError());
   return WL_OK;
@@ -724,33 +773,31 @@ static int mdots_df(wl_amg *a, const zdf *V, long vstride, int kc, const zdf *w,
     kk = (kc - k0 + (nl - l) - 1) / (nl - l);
     wl_count_launches(2);
     launch_mdot_df(kk, c.nblk, c.nt, s, V + k0 * vstride, vstride, w, E, R, a->red.as<float4>());
-    k_mdot_final_df<<<WL_GRID(kk * R * 32, 256), 256, 0, s>>>(a->red.as<float4>(), c.nblk, kk, R, out, ostride, k0,
-                                                              accumulate, coef);
+    k_mdot_final_df<<<kk * R, FIN_T, 0, s>>>(a->red.as<float4>(), c.nblk, kk, R, out, ostride, k0, accumulate, coef,
+                                             nullptr, nullptr);
   }
   WL_CUDA(cudaGetLastError());
   return WL_OK;
 }
 
 
-// w -= sum_k V_k coef_k and out[r] = |w_r|^2 in one pass (double-float)
+// w -= sum_k V_k coef_k and out[r] = |w_r|^2 in one pass (double-float); reset:
+// the counters of k_givens, zeroed
 static int maxpy_norm_df(wl_amg *a, const zdf *V, long vstride, int kc, const float4 *coef, zdf *w, long E, int R,
-                         zd *tmp, double *out, cudaStream_t s) {
+                         double *out, int *reset, cudaStream_t s) {
   RedCfg c = red_cfg(E, R);
   k_maxpy_df<<<c.nblk, c.nt, 0, s>>>(V, vstride, kc, coef, w, E, R, a->red.as<float4>());
-  k_mdot_final_df<<<WL_GRID(R * 32, 256), 256, 0, s>>>(a->red.as<float4>(), c.nblk, 1, R, tmp, 1, 0, 0, nullptr);
-  k_re_of<<<WL_GRID(R, 128), 128, 0, s>>>(tmp, out, R);
-  wl_count_launches(3);
+  k_mdot_final_df<<<R, FIN_T, 0, s>>>(a->red.as<float4>(), c.nblk, 1, R, nullptr, 1, 0, 0, nullptr, out, reset);
+  wl_count_launches(2);
   WL_CUDA(cudaGetLastError());
   return WL_OK;
 }
 
-static int norms2(wl_amg *a, const zd *w, long E, int R, zd *tmp, double *out, cudaStream_t s) {
+static int norms2(wl_amg *a, const zd *w, long E, int R, double *out, int *reset, cudaStream_t s) {
   RedCfg c = red_cfg(E, R);
   k_norm2<<<c.nblk, c.nt, sizeof(double) * c.nt, s>>>(w, E, R, a->red.as<zd>());
-  k_mdot_final<<<WL_GRID(R * 32, 256), 256, 0, s>>>(a->red.as<zd>(), c.nblk, 1, R, tmp, 1, 0, 0, nullptr);
+  k_mdot_final<<<R, FIN_T, 0, s>>>(a->red.as<zd>(), c.nblk, 1, R, nullptr, 1, 0, 0, nullptr, out, reset);
   wl_count_launches(2);
-  k_re_of<<<WL_GRID(R, 128), 128, 0, s>>>(tmp, out, R);
-  wl_count_launches(1);
   WL_CUDA(cudaGetLastError());
   return WL_OK;
 }
@@ -760,8 +807,7 @@ int fg_norms(wl_amg *a, const zd *v, int nrhs, double *out) {
   cudaStream_t s = a->op->stream;
   long E = (long)a->lev[0].n * 2 * nrhs;
   KS k = ks_layout(a->small.p, a->prm.fgmres_m, nrhs);
-  zd *tmpc = a->small.as<zd>() + (a->small.bytes / sizeof(zd)) - 2 * (size_t)nrhs - 8;
-  WL_TRY(norms2(a, v, E, nrhs, tmpc, k.nrm2, s));
+  WL_TRY(norms2(a, v, E, nrhs, k.nrm2, nullptr, s));
   double *h_d = (double *)a->h_small;
   WL_CUDA(cudaMemcpyAsync(h_d, k.nrm2, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
   WL_CUDA(cudaStreamSynchronize(s));
@@ -783,8 +829,7 @@ int fg_residual(wl_amg *a, const zd *bh, const zd *xh, int nrhs, double *rnorm) 
   k_sub<<<WL_GRID(E, 256), 256, 0, s>>>(bh, w, rr, E);
   wl_count_launches(1);
   KS k = ks_layout(a->small.p, a->prm.fgmres_m, nrhs);
-  zd *tmpc = a->small.as<zd>() + (a->small.bytes / sizeof(zd)) - 2 * (size_t)nrhs - 8;
-  WL_TRY(norms2(a, rr, E, nrhs, tmpc, k.nrm2, s));
+  WL_TRY(norms2(a, rr, E, nrhs, k.nrm2, nullptr, s));
   double *h_d = (double *)a->h_small;
   WL_CUDA(cudaMemcpyAsync(h_d, k.nrm2, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
   WL_CUDA(cudaStreamSynchronize(s));
@@ -853,33 +898,33 @@ int fg_cycle(wl_amg *a, const zd *bnorm_h, zd *xh, int nrhs, double tol, const i
     void *zj = Zb + (size_t)j * vs * zb_;
     // z_j = M(v_j) in the cycle precision (lev[0].f holds v_j)
     WL_TRY(cycle_run(a, nrhs, prec, s));
-    WL_CUDA(cudaMemcpyAsync(zj, a->lev[0].x.p, zb_ * E, cudaMemcpyDeviceToDevice, s));
-    // w = Dhat z_j (FP64)
-    if (df) WL_TRY(stencil_apply32_to_df(a, zj, wd, nrhs, s));
-    else if (prec != WL_FP64 && a->prm.arnoldi_matvec == 1) WL_TRY(stencil_apply32_to64(a, zj, w, nrhs, s));
-    else WL_TRY(dhat_apply_dev(op, zj, prec != WL_FP64, w, nrhs, s));
+    // w = Dhat z_j; the FP32 product keeps z_j as it reads it
+    if (df) {
+      WL_TRY(stencil_apply32_to_df(a, a->lev[0].x.p, wd, nrhs, (zf *)zj, s));
+    } else if (prec != WL_FP64 && a->prm.arnoldi_matvec == 1) {
+      WL_TRY(stencil_apply32_to64(a, a->lev[0].x.p, w, nrhs, (zf *)zj, s));
+    } else {
+      WL_CUDA(cudaMemcpyAsync(zj, a->lev[0].x.p, zb_ * E, cudaMemcpyDeviceToDevice, s));
+      WL_TRY(dhat_apply_dev(op, zj, prec != WL_FP64, w, nrhs, s));
+    }
     // Gram-Schmidt against v_0 .. v_j
-    k_zero_hcol<<<WL_GRID(nrhs, 128), 128, 0, s>>>(k);
-    wl_count_launches(1);
-    zd *tmpc = a->small.as<zd>() + (a->small.bytes / sizeof(zd)) - 2 * (size_t)nrhs - 8;
     for (int pass = 0; pass < a->prm.gs_passes; ++pass) {
       if (df) {
-        WL_TRY(mdots_df(a, Vd, vs, j + 1, wd, E, nrhs, k.hcol, m + 1, 1, k.hpd, s));
+        WL_TRY(mdots_df(a, Vd, vs, j + 1, wd, E, nrhs, k.hcol, m + 1, pass > 0, k.hpd, s));
         if (pass + 1 == a->prm.gs_passes) {  // the last pass also forms |w|^2
-          WL_TRY(maxpy_norm_df(a, Vd, vs, j + 1, k.hpd, wd, E, nrhs, tmpc, k.nrm2, s));
+          WL_TRY(maxpy_norm_df(a, Vd, vs, j + 1, k.hpd, wd, E, nrhs, k.nrm2, k.running, s));
         } else {
           k_maxpy_df<<<gE, 256, 0, s>>>(Vd, vs, j + 1, k.hpd, wd, E, nrhs, nullptr);
           wl_count_launches(1);
         }
       } else {
-        WL_TRY(mdots<double>(a, V, vs, j + 1, w, E, nrhs, k.hcol, m + 1, 1, k.hpass, s));
+        WL_TRY(mdots<double>(a, V, vs, j + 1, w, E, nrhs, k.hcol, m + 1, pass > 0, k.hpass, s));
         k_maxpy<double, 1><<<gE, 256, 0, s>>>(V, vs, j + 1, k.hpass, nrhs, w, E, nrhs);
         wl_count_launches(1);
       }
     }
-    if (!df) WL_TRY(norms2(a, w, E, nrhs, tmpc, k.nrm2, s));
-    WL_CUDA(cudaMemsetAsync(k.running, 0, sizeof(int) * 2, s));
-    k_givens<<<WL_GRID(nrhs, 128), 128, 0, s>>>(k, j, tol);
+    if (!df) WL_TRY(norms2(a, w, E, nrhs, k.nrm2, k.running, s));
+    k_givens<<<WL_GRID(nrhs * 4, 128), 128, 0, s>>>(k, j, tol);
     wl_count_launches(1);
     if (j + 1 < m) {
       if (df) {
@@ -897,7 +942,7 @@ int fg_cycle(wl_amg *a, const zd *bnorm_h, zd *xh, int nrhs, double tol, const i
     jdone = j + 1;
     if (run[0] == 0) break;
   }
-  k_trisolve<<<WL_GRID(nrhs, 128), 128, 0, s>>>(k, df ? 1 : 0);
+  k_trisolve<<<WL_GRID(nrhs * 32, 128), 128, 0, s>>>(k, df ? 1 : 0);
   if (df) k_xupd_df<<<gE, 256, 0, s>>>(a->Z.as<zf>(), vs, jdone, k.hpd, xh, E, nrhs);
   else if (prec == WL_FP64) k_maxpy<double, 0><<<gE, 256, 0, s>>>(a->Z.as<zd>(), vs, jdone, k.yT, nrhs, xh, E, nrhs);
   else k_maxpy<float, 0><<<gE, 256, 0, s>>>(a->Z.as<zf>(), vs, jdone, k.yT, nrhs, xh, E, nrhs);

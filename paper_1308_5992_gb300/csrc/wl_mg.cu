@@ -21,10 +21,10 @@ namespace cg = cooperative_groups;
 // ------------------------------------------------------------ stencil apply
 // y = A x, or y = f - A x when f != nullptr (y may alias f); arithmetic in T,
 // y stored as Y (the Arnoldi matvec widens an FP32 result to FP64, or keeps
-// it as the high part of a double-float).
+// it as the high part of a double-float).  xo (or NULL) receives a copy of x.
 template <typename T, typename S, typename Y = cx<T>>
 __global__ void __launch_bounds__(256) k_stencil(Geo g, const S *__restrict__ A, const cx<T> *__restrict__ x,
-                                                 const Y *f, Y *y, int nrhs) {
+                                                 const Y *f, Y *y, int nrhs, cx<T> *xo) {
   long tid = (long)blockIdx.x * blockDim.x + threadIdx.x;
   int n = g.nsites();
   if (tid >= (long)n * nrhs) return;
@@ -37,6 +37,10 @@ __global__ void __launch_bounds__(256) k_stencil(Geo g, const S *__restrict__ A,
   for (int d = 0; d < 9; ++d) {
     long j = (long)g.nb(px, py, d) * 2 * nrhs + r;
     cx<T> x0 = x[j], x1 = x[j + nrhs];
+    if (d == 4 && xo) {
+      xo[j] = x0;
+      xo[j + nrhs] = x1;
+    }
     cfma(y0, ld<T>(Ah + d * 4 + 0), x0);
     cfma(y0, ld<T>(Ah + d * 4 + 1), x1);
     cfma(y1, ld<T>(Ah + d * 4 + 2), x0);
@@ -1115,7 +1119,7 @@ static int launch_coop(const Level &L, const LevelOps &o, int sweeps, void *x, v
 // same order, as k_stencil.  x must not alias y.
 template <typename T, typename S, typename Y, int R, int WF>
 __global__ void __launch_bounds__(256) k_stencil_tile(Geo g, const S *__restrict__ A, const cx<T> *__restrict__ x,
-                                                      const Y *f, Y *y, int nrhs, int vec) {
+                                                      const Y *f, Y *y, int nrhs, int vec, cx<T> *xo) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   cx<T> *xs = (cx<T> *)sm_raw;                  // [100][2][R]
   S *As = (S *)(xs + KTH * KTH * 2 * R);        // [64][36]
@@ -1187,6 +1191,11 @@ __global__ void __launch_bounds__(256) k_stencil_tile(Geo g, const S *__restrict
       cfma(y1, ld<T>(Ah + d * 4 + 3), x1);
     }
     long o = (long)hs[(i + 1) * KTH + j + 1] * 2 * nrhs + r0 + q;
+    if (xo) {
+      int lc = ((i + 1) * KTH + j + 1) * 2;
+      xo[o] = xs[lc * R + q];
+      xo[o + nrhs] = xs[(lc + 1) * R + q];
+    }
     Y z0 = store_as<Y>(y0), z1 = store_as<Y>(y1);
     if constexpr (WF) {
       z0 = fv[u][0] - z0;
@@ -1204,7 +1213,7 @@ static size_t stencil_tile_smem(int R) {
 
 template <typename T, typename S, typename Y, int R>
 static int launch_stencil_tile_r(const Level &L, const S *A, const void *x, const void *f, void *y, int nrhs,
-                                 cudaStream_t s) {
+                                 cudaStream_t s, cx<T> *xo) {
   size_t smem = stencil_tile_smem<T, S>(R);
   static std::atomic<unsigned long long> limit_set[2];
   int vec = ((uintptr_t)x % 16 == 0) && (sizeof(T) == 8 || nrhs % 2 == 0);
@@ -1215,11 +1224,11 @@ static int launch_stencil_tile_r(const Level &L, const S *A, const void *x, cons
     } else {
       WL_TRY(set_smem_limit((const void *)k_stencil_tile<T, S, Y, R, 1>, smem, limit_set[1]));
       k_stencil_tile<T, S, Y, R, 1><<<grid, 256, smem, s>>>(L.geo, A, (const cx<T> *)x, (const Y *)f, (Y *)y, nrhs,
-                                                             vec);
+                                                             vec, xo);
     }
   } else {
     WL_TRY(set_smem_limit((const void *)k_stencil_tile<T, S, Y, R, 0>, smem, limit_set[0]));
-    k_stencil_tile<T, S, Y, R, 0><<<grid, 256, smem, s>>>(L.geo, A, (const cx<T> *)x, nullptr, (Y *)y, nrhs, vec);
+    k_stencil_tile<T, S, Y, R, 0><<<grid, 256, smem, s>>>(L.geo, A, (const cx<T> *)x, nullptr, (Y *)y, nrhs, vec, xo);
   }
   return WL_OK;
 }
@@ -1227,16 +1236,16 @@ static int launch_stencil_tile_r(const Level &L, const S *A, const void *x, cons
 // the tiled form for grids the tiling covers and batches of at least 8
 template <typename T, typename S, typename Y>
 static bool launch_stencil_tile(const Level &L, const S *A, const void *x, const void *f, void *y, int nrhs,
-                                cudaStream_t s, int *rc) {
+                                cudaStream_t s, int *rc, cx<T> *xo = nullptr) {
   if (L.N < 64 || L.N % (4 * KT) || nrhs < 8) return false;
   if constexpr (sizeof(T) == 4) {
     if (nrhs >= 32) {
-      *rc = launch_stencil_tile_r<T, S, Y, 32>(L, A, x, f, y, nrhs, s);
+      *rc = launch_stencil_tile_r<T, S, Y, 32>(L, A, x, f, y, nrhs, s, xo);
       return true;
     }
   }
-  if (nrhs >= 16) *rc = launch_stencil_tile_r<T, S, Y, 16>(L, A, x, f, y, nrhs, s);
-  else *rc = launch_stencil_tile_r<T, S, Y, 8>(L, A, x, f, y, nrhs, s);
+  if (nrhs >= 16) *rc = launch_stencil_tile_r<T, S, Y, 16>(L, A, x, f, y, nrhs, s, xo);
+  else *rc = launch_stencil_tile_r<T, S, Y, 8>(L, A, x, f, y, nrhs, s, xo);
   return true;
 }
 
@@ -1250,13 +1259,13 @@ int stencil_apply(wl_amg *a, int l, int prec, const void *x, void *y, const void
   int rc = WL_OK;
   if (prec == WL_FP64) {
     if (!launch_stencil_tile<double, zd, zd>(L, o.A.as<zd>(), x, f, y, nrhs, s, &rc))
-      k_stencil<double, zd><<<grid, 256, 0, s>>>(L.geo, o.A.as<zd>(), (const zd *)x, (const zd *)f, (zd *)y, nrhs);
+      k_stencil<double, zd><<<grid, 256, 0, s>>>(L.geo, o.A.as<zd>(), (const zd *)x, (const zd *)f, (zd *)y, nrhs, nullptr);
   } else if (prec == WL_FP32) {
     if (!launch_stencil_tile<float, zf, zf>(L, o.A.as<zf>(), x, f, y, nrhs, s, &rc))
-      k_stencil<float, zf><<<grid, 256, 0, s>>>(L.geo, o.A.as<zf>(), (const zf *)x, (const zf *)f, (zf *)y, nrhs);
+      k_stencil<float, zf><<<grid, 256, 0, s>>>(L.geo, o.A.as<zf>(), (const zf *)x, (const zf *)f, (zf *)y, nrhs, nullptr);
   } else {
     if (!launch_stencil_tile<float, zb, zf>(L, o.A.as<zb>(), x, f, y, nrhs, s, &rc))
-      k_stencil<float, zb><<<grid, 256, 0, s>>>(L.geo, o.A.as<zb>(), (const zf *)x, (const zf *)f, (zf *)y, nrhs);
+      k_stencil<float, zb><<<grid, 256, 0, s>>>(L.geo, o.A.as<zb>(), (const zf *)x, (const zf *)f, (zf *)y, nrhs, nullptr);
   }
   WL_TRY(rc);
   WL_CUDA(cudaGetLastError());
@@ -1676,25 +1685,26 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
 
 // y = A_0 x in FP32 arithmetic from the FP32 copy of the level-0 stencil
 // (Dhat), x float, y widened to double or stored as a double-float with a
-// zero low part: the Arnoldi matvec of an FP32 cycle
+// zero low part: the Arnoldi matvec of an FP32 cycle; xo (or NULL) receives a
+// copy of x (the Krylov solver keeps z_j)
 template <typename Y>
-static int stencil_apply32_to(wl_amg *a, const void *x, Y *y, int nrhs, cudaStream_t s) {
+static int stencil_apply32_to(wl_amg *a, const void *x, Y *y, int nrhs, zf *xo, cudaStream_t s) {
   const Level &L = a->lev[0];
   long tot = (long)L.n * nrhs;
   wl_count_launches(1);
   int rc = WL_OK;
-  if (!launch_stencil_tile<float, zf, Y>(L, L.op32.A.as<zf>(), x, nullptr, y, nrhs, s, &rc))
+  if (!launch_stencil_tile<float, zf, Y>(L, L.op32.A.as<zf>(), x, nullptr, y, nrhs, s, &rc, xo))
     k_stencil<float, zf, Y><<<WL_GRID(tot, 256), 256, 0, s>>>(L.geo, L.op32.A.as<zf>(), (const zf *)x, nullptr, y,
-                                                              nrhs);
+                                                              nrhs, xo);
   WL_TRY(rc);
   WL_CUDA(cudaGetLastError());
   return WL_OK;
 }
-int stencil_apply32_to64(wl_amg *a, const void *x, zd *y, int nrhs, cudaStream_t s) {
-  return stencil_apply32_to<zd>(a, x, y, nrhs, s);
+int stencil_apply32_to64(wl_amg *a, const void *x, zd *y, int nrhs, zf *xo, cudaStream_t s) {
+  return stencil_apply32_to<zd>(a, x, y, nrhs, xo, s);
 }
-int stencil_apply32_to_df(wl_amg *a, const void *x, zdf *y, int nrhs, cudaStream_t s) {
-  return stencil_apply32_to<zdf>(a, x, y, nrhs, s);
+int stencil_apply32_to_df(wl_amg *a, const void *x, zdf *y, int nrhs, zf *xo, cudaStream_t s) {
+  return stencil_apply32_to<zdf>(a, x, y, nrhs, xo, s);
 }
 
 int restrict_op(wl_amg *a, int l, int prec, const void *r, void *fc, int nrhs, cudaStream_t s) {
