@@ -291,6 +291,8 @@ struct wl_amg {
   DBuf small;     // per-rhs scalars (Hessenberg, Givens, flags)
   DBuf pinned_small;  // host-pinned mirror of flags
   void *h_small;
+  size_t slots_at = 0;                            // byte offset in h_small of the per-iteration verdicts
+  cudaEvent_t lag_ev[2] = {nullptr, nullptr};     // recorded after iteration j's verdict, alternating
   // captured cycle graphs, one per (nrhs, precision)
   struct G {
     int nrhs, prec;

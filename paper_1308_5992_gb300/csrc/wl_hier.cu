@@ -306,7 +306,8 @@ int ensure_workspace(wl_amg *a, int nrhs, int prec) {
   WL_TRY(a->small.alloc(sizeof(zd) * (size_t)cap * 8 * (m + 2) * (m + 2)));
   if (a->h_small) cudaFreeHost(a->h_small);
   a->h_small = nullptr;
-  WL_CUDA(cudaMallocHost(&a->h_small, sizeof(double) * (size_t)cap * 16 + 64));
+  a->slots_at = sizeof(double) * (size_t)cap * 16 + 64;
+  WL_CUDA(cudaMallocHost(&a->h_small, a->slots_at + sizeof(int) * 4 * 32));
   a->cap = cap;
   return WL_OK;
 }
@@ -427,6 +428,8 @@ void amg_free(wl_amg *a) {
   a->red.release();
   a->small.release();
   if (a->h_small) cudaFreeHost(a->h_small);
+  for (cudaEvent_t ev : a->lag_ev)
+    if (ev) cudaEventDestroy(ev);
   wl_op *op = a->op;
   delete a;
   if (op) op_release(op);

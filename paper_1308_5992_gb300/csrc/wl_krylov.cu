@@ -40,7 +40,7 @@ struct KS {
   double *bnorm, *beta, *nrm2, *inv;  // [nrhs]
   int *active, *stop, *jend, *iters;  // [nrhs]
   int *nanf;                          // [nrhs] non-finite value seen (Arnoldi residual, or masked input)
-  int *running;                       // [1]
+  int *running;  // [3]: right-hand sides that go on, non-finite seen, the largest of their residuals over tol |bhat| (float bits)
   float4 *hpd;   // [m+1][nrhs][2] the coefficients of hpass as double-floats, for k_maxpy_df
   float2 *invdf; // [nrhs] inv as a double-float (hi, lo)
 };
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(FIN_T) k_mdot_final(const zd *__restrict__ par
   __syncthreads();
   if (threadIdx.x) return;
   s = (ws[0] + ws[1]) + (ws[2] + ws[3]);
-  if (reset && blockIdx.x == 0) reset[0] = reset[1] = 0;
+  if (reset && blockIdx.x == 0) reset[0] = reset[1] = reset[2] = 0;
   if (re) re[r] = s.re;
   if (!out) return;
   zd *o = out + (long)r * ostride + k0 + k;
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(FIN_T) k_mdot_final_df(const float4 *__restric
   }
   zd s = mk(((double)A.s.x + (double)A.s.y) + ((double)A.c.x + (double)A.c.y),
             ((double)B.s.x - (double)B.s.y) + ((double)B.c.x - (double)B.c.y));
-  if (reset && blockIdx.x == 0) reset[0] = reset[1] = 0;
+  if (reset && blockIdx.x == 0) reset[0] = reset[1] = reset[2] = 0;
   if (re) re[r] = s.re;
   if (!out) return;
   zd *o = out + (long)r * ostride + k0 + k;
@@ -671,8 +671,12 @@ __global__ void __launch_bounds__(128) k_givens(KS k, int j, double tol) {
   }
   k.inv[r] = (done || hn == 0.0) ? 0.0 : 1.0 / hn;
   k.invdf[r] = split_df(k.inv[r]);
-  if (done) k.stop[r] = 1;
-  else atomicAdd(k.running, 1);
+  if (done) {
+    k.stop[r] = 1;
+  } else {
+    atomicAdd(k.running, 1);
+    atomicMax(k.running + 2, __float_as_int((float)(res / (tol * k.bnorm[r]))));  // positive floats order as ints
+  }
 }
 
 // y = H^-1 g (upper triangular, jend columns), zero beyond jend / inactive
@@ -873,7 +877,6 @@ int fg_cycle(wl_amg *a, const zd *bnorm_h, zd *xh, int nrhs, double tol, const i
   size_t zb_ = prec_bytes(prec);
   char *Zb = (char *)a->Z.p;
   unsigned gE = WL_GRID(E, 256);
-  double *h_d = (double *)a->h_small;
   (void)bnorm_h;
   WL_CUDA(cudaMemcpyAsync(k.active, active, sizeof(int) * nrhs, cudaMemcpyHostToDevice, s));
   WL_CUDA(cudaMemsetAsync(k.iters, 0, sizeof(int) * nrhs, s));
@@ -893,7 +896,11 @@ int fg_cycle(wl_amg *a, const zd *bnorm_h, zd *xh, int nrhs, double tol, const i
   } else {
     scale_next(rr, V);
   }
-  int jdone = 0;
+  if (!a->lag_ev[0])
+    for (cudaEvent_t &ev : a->lag_ev) WL_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+  int *slots = (int *)((char *)a->h_small + a->slots_at);  // pinned, 4 ints an iteration
+  int jdone = 0, known = 0;          // iterations run, verdicts read
+  double ratio = 0.0, rho = 1.0 / 30;  // of the last verdict read
   for (int j = 0; j < m; ++j) {
     void *zj = Zb + (size_t)j * vs * zb_;
     // z_j = M(v_j) in the cycle precision (lev[0].f holds v_j)
@@ -935,12 +942,32 @@ int fg_cycle(wl_amg *a, const zd *bnorm_h, zd *xh, int nrhs, double tol, const i
       }
     }
     WL_CUDA(cudaGetLastError());
-    int run[2];
-    WL_CUDA(cudaMemcpyAsync(h_d + nrhs, k.running, sizeof(int) * 2, cudaMemcpyDeviceToHost, s));
-    WL_CUDA(cudaStreamSynchronize(s));
-    memcpy(run, h_d + nrhs, sizeof(int) * 2);
+    WL_CUDA(cudaMemcpyAsync(slots + 4 * j, k.running, sizeof(int) * 3, cudaMemcpyDeviceToHost, s));
+    WL_CUDA(cudaEventRecord(a->lag_ev[j & 1], s));
     jdone = j + 1;
-    if (run[0] == 0) break;
+    if (j + 1 == m) break;
+    // Going on needs to know that some right-hand side does.  Waiting for this
+    // iteration's verdict leaves the GPU idle while the host launches the next one
+    // (about 100 us of an iteration), so while the residuals known are far from the
+    // tolerance, the verdict of the iteration before is enough: with their last
+    // contraction (1 / 30 before one is known) this iteration leaves some residual
+    // at 3 times the tolerance or more.  An iteration run past the end does no harm:
+    // its right-hand sides are stopped, their vectors zero.
+    bool more = true;
+    for (; known <= j; ++known) {
+      if (known == j && ratio * std::min(1.0, rho) > 3.0) break;
+      WL_CUDA(cudaEventSynchronize(a->lag_ev[known & 1]));
+      const int *run = slots + 4 * known;
+      if (run[0] == 0) {
+        more = false;
+        break;
+      }
+      float now;
+      memcpy(&now, run + 2, sizeof(float));
+      if (known > 0) rho = now / ratio;
+      ratio = now;
+    }
+    if (!more) break;
   }
   k_trisolve<<<WL_GRID(nrhs * 32, 128), 128, 0, s>>>(k, df ? 1 : 0);
   if (df) k_xupd_df<<<gE, 256, 0, s>>>(a->Z.as<zf>(), vs, jdone, k.hpd, xh, E, nrhs);
