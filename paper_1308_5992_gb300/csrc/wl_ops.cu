@@ -117,6 +117,95 @@ __global__ void k_hop(Geo g, const cx<Tc> *__restrict__ V, int par_out,
   out[o + nrhs] = ccast<Tout>(o1);
 }
 
+// double -> float, round to nearest even, on the integer pipes (as f2d: the
+// hardware conversion takes the FP64 unit): for a result in the normal range the
+// exponent is rebiased, the mantissa's lower 29 bits rounded away, a carry going
+// into the exponent; everything else takes the hardware conversion.
+__device__ __forceinline__ float d2f(double d) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+  const unsigned e = (unsigned)(u >> 52) & 0x7ffu;
+  if (e - 897u > 253u) return (float)d;  // float exponent 1 .. 254
+  const unsigned low = (unsigned)u & 0x1fffffffu;
+  unsigned m = ((e - 896u) << 23) | ((unsigned)(u >> 29) & 0x7fffffu);
+  m += (low > 0x10000000u) || (low == 0x10000000u && (m & 1u));
+  return __uint_as_float(m | (unsigned)(u >> 32) & 0x80000000u);
+}
+template <typename T>
+__device__ __forceinline__ cx<T> narrow(zd v);
+template <>
+__device__ __forceinline__ zd narrow<double>(zd v) { return v; }
+template <>
+__device__ __forceinline__ zf narrow<float>(zd v) { return mk(d2f(v.re), d2f(v.im)); }
+
+// hop_acc with the complex product's roundings fixed, so that an FP32 result does
+// not depend on where the compiler contracts it: re = fma(l.re, w.re, -(l.im w.im)),
+// im = fma(l.re, w.im, l.im w.re), the form k_hop compiles to
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+template <typename T>
+__device__ __forceinline__ void hop_acc_rn(cx<T> &o0, cx<T> &o1, int mu, int fwd, cx<T> link, cx<T> v0, cx<T> v1) {
+  cx<T> w = mu == 0 ? (fwd ? v0 - v1 : v0 + v1) : (fwd ? v0 + ci(v1) : v0 - ci(v1));
+  const cx<T> l = fwd ? link : cconj(link);
+  w = mk(fma(l.re, w.re, -mul_rn(l.im, w.im)), fma(l.re, w.im, mul_rn(l.im, w.re)));
+  o0 = o0 + w;
+  if (mu == 0) o1 = fwd ? o1 - w : o1 + w;
+  else o1 = fwd ? o1 - ci(w) : o1 + ci(w);
+}
+
+// y = Dhat x in one kernel, x and y in the ABI layout [nrhs][n][2]: a block per
+// TX x TY tile of the lattice and right-hand side keeps x of the tile's even sites
+// and two sites around, then K_oe x on its odd sites and one around, in shared
+// memory.  The arithmetic is k_hop's, step for step.  Two k_hop launches between
+// two layout transposes, with three buffers allocated and freed a call, took
+// 380 us at 512 x 512 with 12 right-hand sides in FP32 (60 us of it on the GPU) and
+// 39 us at 64 x 64 in FP64; a call now takes 61 and 18 us.
+template <typename Tc, int TX, int TY, int NT>
+__global__ void __launch_bounds__(NT) k_dhat_tile(Geo g, const cx<Tc> *__restrict__ V, const zd *__restrict__ in,
+                                                  zd *__restrict__ out) {
+  constexpr int XC = (TX + 4) / 2, OC = (TX + 2) / 2;  // even, odd sites a staged row
+  __shared__ cx<Tc> xs[TY + 4][XC][2], ts[TY + 2][OC][2];
+  const int N = g.N, tx = N / TX, tiles = tx * (N / TY), tid = threadIdx.x;
+  const int tile = blockIdx.x % tiles, x0 = (tile % tx) * TX, y0 = (tile / tx) * TY;
+  const long base = (long)(blockIdx.x / tiles) * g.nsites() * 2;
+  for (int e = tid; e < (TY + 4) * XC; e += NT) {  // even sites: row y0 - 2 + r, x = x0 - 2 + (r & 1) + 2 c
+    int r = e / XC, c = e % XC;
+    const zd *p = in + base + (long)g.idx(x0 - 2 + (r & 1) + 2 * c, y0 - 2 + r) * 2;
+    xs[r][c][0] = narrow<Tc>(p[0]);
+    xs[r][c][1] = narrow<Tc>(p[1]);
+  }
+  __syncthreads();
+  for (int e = tid; e < (TY + 2) * OC; e += NT) {  // odd sites: row y0 - 1 + r, x = x0 - (r & 1) + 2 c
+    int r = e / OC, c = e % OC, x = x0 - (r & 1) + 2 * c, y = y0 - 1 + r;
+    const int xw = x & (N - 1), yw = y & (N - 1), xm = (x - 1) & (N - 1), ym = (y - 1) & (N - 1);
+    cx<Tc> o0 = mk<Tc>(0, 0), o1 = mk<Tc>(0, 0);
+    // the even neighbours: this row's column index is x - x0 + 1 over 2 to the left, one more to the right
+    const int q = r + 1, cl = (x - 1 - x0 + 2) >> 1, cm = (x - x0 + 2) >> 1;
+    hop_acc_rn(o0, o1, 0, 1, V[(long)yw * N + xw], xs[q][cl + 1][0], xs[q][cl + 1][1]);
+    hop_acc_rn(o0, o1, 0, 0, V[(long)yw * N + xm], xs[q][cl][0], xs[q][cl][1]);
+    hop_acc_rn(o0, o1, 1, 1, V[((long)N + yw) * N + xw], xs[q + 1][cm][0], xs[q + 1][cm][1]);
+    hop_acc_rn(o0, o1, 1, 0, V[((long)N + ym) * N + xw], xs[q - 1][cm][0], xs[q - 1][cm][1]);
+    ts[r][c][0] = o0;
+    ts[r][c][1] = o1;
+  }
+  __syncthreads();
+  for (int e = tid; e < TY * TX / 2; e += NT) {  // even sites: row y0 + r, x = x0 + (r & 1) + 2 c
+    int r = e / (TX / 2), c = e % (TX / 2), x = x0 + (r & 1) + 2 * c, y = y0 + r;
+    const int xm = (x - 1) & (N - 1), ym = (y - 1) & (N - 1);
+    cx<Tc> o0 = mk<Tc>(0, 0), o1 = mk<Tc>(0, 0);
+    const int q = r + 1, rx = x - x0;  // in a row q of ts: column (x' - x0 + (q & 1)) / 2 of odd site x'
+    const int cl = (rx - 1 + (q & 1)) >> 1, cm = (rx + (1 - (q & 1))) >> 1;
+    hop_acc_rn(o0, o1, 0, 1, V[(long)y * N + x], ts[q][cl + 1][0], ts[q][cl + 1][1]);
+    hop_acc_rn(o0, o1, 0, 0, V[(long)y * N + xm], ts[q][cl][0], ts[q][cl][1]);
+    hop_acc_rn(o0, o1, 1, 1, V[((long)N + y) * N + x], ts[q + 1][cm][0], ts[q + 1][cm][1]);
+    hop_acc_rn(o0, o1, 1, 0, V[((long)N + ym) * N + x], ts[q - 1][cm][0], ts[q - 1][cm][1]);
+    o0 = xs[r + 2][(rx + 2) >> 1][0] - o0;
+    o1 = xs[r + 2][(rx + 2) >> 1][1] - o1;
+    zd *p = out + base + (long)g.idx(x, y) * 2;
+    p[0] = widen<double>(o0);
+    p[1] = widen<double>(o1);
+  }
+}
+
 // D psi on the full lattice, ABI layout [nrhs][N][N][2]: D = c (I - K);
 // g5 = 1 gives Z psi = Gamma5 D psi (Thm. 3.1: the spin-1 row negated, an
 // exact sign flip of the D result)
@@ -131,20 +220,22 @@ __global__ void k_wilson_full(int N, double c, const cx<Tc> *__restrict__ V,
   int y = z / N, x = z % N;
   const zd *b = in + (long)r * nz * 2;
   cx<Tc> o0 = mk<Tc>(0, 0), o1 = mk<Tc>(0, 0);
+#pragma unroll
   for (int mu = 0; mu < 2; ++mu)
+#pragma unroll
     for (int fwd = 1; fwd >= 0; --fwd) {
       int dx = (mu == 0) ? (fwd ? 1 : -1) : 0, dy = (mu == 1) ? (fwd ? 1 : -1) : 0;
       int xn = (x + dx) & (N - 1), yn = (y + dy) & (N - 1);
       int lx = fwd ? x : xn, ly = fwd ? y : yn;
       cx<Tc> link = V[(mu * N + ly) * N + lx];
       long j = ((long)yn * N + xn) * 2;
-      hop_acc(o0, o1, mu, fwd, link, ccast<Tc>(b[j]), ccast<Tc>(b[j + 1]));
+      hop_acc(o0, o1, mu, fwd, link, narrow<Tc>(b[j]), narrow<Tc>(b[j + 1]));
     }
   long o = ((long)r * nz + z) * 2;
-  cx<Tc> p0 = ccast<Tc>(in[o]), p1 = ccast<Tc>(in[o + 1]);
+  cx<Tc> p0 = narrow<Tc>(in[o]), p1 = narrow<Tc>(in[o + 1]);
   Tc cc = (Tc)c;
-  out[o] = ccast<double>(cc * (p0 - o0));
-  out[o + 1] = ccast<double>((g5 ? -cc : cc) * (p1 - o1));
+  out[o] = widen<double>(cc * (p0 - o0));
+  out[o + 1] = widen<double>((g5 ? -cc : cc) * (p1 - o1));
 }
 
 // bhat_e = b_e/c + K_eo (b_o/c); b in ABI layout [nrhs][N][N][2], bhat
@@ -559,42 +650,23 @@ extern "C" int wl_apply(wl_op *op, int which, const void *x, void *y, int nrhs, 
     WL_CUDA(cudaGetLastError());
     return WL_OK;
   }
-  long n = g.nsites();
-  size_t eb = prec == WL_FP64 ? sizeof(zd) : sizeof(zf);
-  DBuf xi, yi, t;
-  int rc = xi.alloc(eb * n * 2 * nrhs);
-  if (!rc) rc = yi.alloc(eb * n * 2 * nrhs);
-  if (!rc) rc = t.alloc(eb * n * 2 * nrhs);
-  if (!rc) rc = wl::to_internal((const zd *)x, xi.p, (int)(2 * n), nrhs, prec, s);
-  if (!rc) {
-    unsigned grid = WL_GRID(n * nrhs, 256);
-    if (prec == WL_FP64) {
-      const zd *V = op->Uf64.as<zd>();
-      k_hop<double, double, double, double><<<grid, 256, 0, s>>>(g, V, 1, xi.as<zd>(), nullptr, t.as<zd>(), nrhs);
-      k_hop<double, double, double, double><<<grid, 256, 0, s>>>(g, V, 0, t.as<zd>(), xi.as<zd>(), yi.as<zd>(), nrhs);
-    } else {
-      const zf *V = op->Uf32.as<zf>();
-      k_hop<float, float, float, float><<<grid, 256, 0, s>>>(g, V, 1, xi.as<zf>(), nullptr, t.as<zf>(), nrhs);
-      k_hop<float, float, float, float><<<grid, 256, 0, s>>>(g, V, 0, t.as<zf>(), xi.as<zf>(), yi.as<zf>(), nrhs);
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      wl_set_error("wl_apply: %s", cudaGetErrorString(e));
-      rc = WL_ECUDA;
-    }
+  // large tiles where they fill the GPU twice over, else 8 x 8: at 64 x 64 with one
+  // right-hand side those spread over 64 SMs what would be 8 tiles
+  const long sites = (long)g.nsites() * nrhs;
+  const bool large = N >= 32 && sites >= 256 * 304;
+  const zd *xx = (const zd *)x;
+  zd *yy = (zd *)y;
+  if (prec == WL_FP64) {
+    if (large) k_dhat_tile<double, 32, 16, 320><<<(unsigned)(sites / 256), 320, 0, s>>>(g, op->Uf64.as<zd>(), xx, yy);
+    else k_dhat_tile<double, 8, 8, 64><<<(unsigned)(sites / 32), 64, 0, s>>>(g, op->Uf64.as<zd>(), xx, yy);
+  } else {
+    if (large) k_dhat_tile<float, 32, 16, 320><<<(unsigned)(sites / 256), 320, 0, s>>>(g, op->Uf32.as<zf>(), xx, yy);
+    else k_dhat_tile<float, 8, 8, 64><<<(unsigned)(sites / 32), 64, 0, s>>>(g, op->Uf32.as<zf>(), xx, yy);
   }
-  if (!rc) rc = wl::from_internal(yi.p, (zd *)y, (int)(2 * n), nrhs, prec, s);
-  if (!rc) {
-    cudaError_t e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) {
-      wl_set_error("wl_apply: %s", cudaGetErrorString(e));
-      rc = WL_ECUDA;
-    }
-  }
-  xi.release();
-  yi.release();
-  t.release();
-  return rc;
+  wl_count_launches(1);
+  WL_CUDA(cudaGetLastError());
+  WL_CUDA(cudaStreamSynchronize(s));
+  return WL_OK;
 }
 
 extern "C" int wl_eo_reduce(wl_op *op, const void *b, void *bhat, int nrhs) {
