@@ -333,7 +333,7 @@ int stencil_apply(wl_amg *a, int l, int prec, const void *x, void *y, const void
 int kaczmarz_sweeps(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int sweeps,
                     cudaStream_t s);
 int kaczmarz_colour(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int c, cudaStream_t s);
-int kaczmarz_tile(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int tc, cudaStream_t s, int R = 0);
+int kaczmarz_tile(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int tc, cudaStream_t s, int R = 0, int pdl = 0);
 int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s);  // every level but the coarsest
 int tile_timeout_take(cudaStream_t s);  // 1 if a tile launch's bounded wait ran out (flag cleared)
 int *tile_timeout_flag();               // device address of that flag on the current device
