@@ -58,6 +58,62 @@ __global__ void __launch_bounds__(256) k_stencil(Geo g, const S *__restrict__ A,
   y[o + nrhs] = z1;
 }
 
+// Signs and components for lanes that hold one component of a complex product
+// (the sign flips go to the integer pipe: a run-time negation of a double takes
+// the FP64 unit)
+__device__ __forceinline__ double flip_if(double v, bool neg) {
+  return __hiloint2double(__double2hiint(v) ^ (neg ? (int)0x80000000 : 0), __double2loint(v));
+}
+__device__ __forceinline__ float flip_if(float v, bool neg) {
+  return __int_as_float(__float_as_int(v) ^ (neg ? (int)0x80000000 : 0));
+}
+// acc += component c of a v (CONJ: of conj(a) v)
+template <typename T, bool CONJ>
+__device__ __forceinline__ void cfma_part(T &acc, cx<T> a, cx<T> v, int c) {
+  acc = fma(a.re, c ? v.im : v.re, acc);
+  acc = fma(flip_if(a.im, (c == 0) != CONJ), c ? v.re : v.im, acc);
+}
+
+// The cycle's stencil apply and transfers for small batches, several lanes a site:
+// with one thread a site a level's launch is one chain of up to 392 dependent FMAs
+// (in FP64 64 cycles each) and strided loads of its 288 or 576 byte row.
+//
+// k_stencil for nrhs < 8: lane (s, t, c) of a (site, right-hand side) sums
+// component c of A[h][d][s][t] x_t over the nine offsets, the pair of t meets by a
+// shuffle; 18 FMAs and an addition a lane.  One right-hand side, FP64: 9.7 -> 3.0
+// us on 128 x 128 to 32 x 32.  FP32 on 128 x 128 and 32 x 32: 6.7 -> 4.4 us; on
+// 512 x 512 the loads that several lanes repeat make it slower (13.6 -> 16.2 us for
+// one right-hand side, 23.6 -> 56.8 us for five).
+template <typename T, typename S, typename Y>
+__global__ void __launch_bounds__(256) k_stencil_lanes(Geo g, const S *__restrict__ A, const cx<T> *__restrict__ x,
+                                                       const Y *f, Y *y, int nrhs, cx<T> *xo) {
+  const long tid = (long)blockIdx.x * 256 + threadIdx.x, q = tid >> 3;
+  const int c = (int)tid & 1, t = (int)(tid >> 1) & 1, s = (int)(tid >> 2) & 1;
+  const bool act = q < (long)g.nsites() * nrhs;
+  const int h = act ? (int)(q / nrhs) : 0, r = act ? (int)(q - (long)h * nrhs) : 0;
+  int px, py;
+  g.xy(h, px, py);
+  const S *Ah = A + (long)h * 36 + s * 2 + t;
+  cx<T> a[9], v[9];
+#pragma unroll
+  for (int d = 0; d < 9; ++d) a[d] = ld<T>(Ah + d * 4);
+#pragma unroll
+  for (int d = 0; d < 9; ++d) v[d] = x[((long)g.nb(px, py, d) * 2 + t) * nrhs + r];
+  T acc = 0;
+#pragma unroll
+  for (int d = 0; d < 9; ++d) cfma_part<T, false>(acc, a[d], v[d], c);
+  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+  T other = __shfl_xor_sync(0xffffffffu, acc, 1);
+  if (!act || c || t) return;
+  const long o = ((long)h * 2 + s) * nrhs + r;
+  Y z = store_as<Y>(mk(acc, other));
+  if constexpr (!std::is_same<Y, zdf>::value) {
+    if (f) z = f[o] - z;
+  }
+  if (xo) xo[o] = x[o];
+  y[o] = z;
+}
+
 // ---------------------------------------------------------------- Kaczmarz
 // One colour of the multicolour sweep.  Colour k = 4 (a mod 4) + (b mod 4);
 // item q enumerates a = ka + 4 (q / (N/8)), b = kb + 4 (q mod N/8).
@@ -964,6 +1020,34 @@ __global__ void k_restrict(Geo gf, Geo gc, int lgB, const S *__restrict__ P,
   fc[o + nrhs] = a1;
 }
 
+// The same with 16 lanes a (coarse site, right-hand side): lane (spin, i) takes the
+// taps i, i + 8, ...; each spin's eight lanes meet by shuffles (first halves of the
+// lanes keep the real, the others the imaginary part).  512 x 512 to 128 x 128, one
+// right-hand side, FP32: 12.4 us with one thread of 98 products each, 3.7 us.
+template <typename T, typename S>
+__global__ void __launch_bounds__(256) k_restrict_lanes(Geo gf, Geo gc, int lgB, const S *__restrict__ P,
+                                                        const cx<T> *__restrict__ r, cx<T> *__restrict__ fc, int nrhs) {
+  const long tid = (long)blockIdx.x * 256 + threadIdx.x, q = tid >> 4;
+  const int i = (int)tid & 7, s = (int)(tid >> 3) & 1;
+  const bool act = q < (long)gc.nsites() * nrhs;
+  const int hc = act ? (int)(q / nrhs) : 0, rh = act ? (int)(q - (long)hc * nrhs) : 0;
+  int xc, yc;
+  gc.xy(hc, xc, yc);
+  const int B = 1 << lgB, W = 2 * B - 1, X = xc << lgB, Y = yc << lgB;
+  cx<T> acc = mk<T>(0, 0);
+  for (int e = i; e < W * W; e += 8) {
+    const int da = e / W - (B - 1), db = e % W - (B - 1);
+    const long hf = gf.idx(X + da + db, Y + da - db);
+    const int k = (da < 0 ? 1 : 0) + (db < 0 ? 2 : 0);
+    cfmac(acc, ld<T>(P + hf * 8 + s * 4 + k), r[(hf * 2 + s) * nrhs + rh]);
+  }
+  const bool im = i & 4;  // the component this lane keeps
+  T v = (im ? acc.im : acc.re) + __shfl_xor_sync(0xffffffffu, im ? acc.re : acc.im, 4);
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  if (act && (i & 3) == 0) ((T *)fc)[(((long)hc * 2 + s) * nrhs + rh) * 2 + (im ? 1 : 0)] = v;
+}
+
 // x += P e: fine site (a, b) with cell origin (a0, b0) = B floor((a, b)/B)
 // interpolates from the existing corners (a0 + ka B, b0 + kb B).
 template <typename T, typename S>
@@ -995,25 +1079,27 @@ __global__ void k_prolong(Geo gf, Geo gc, int lgB, const S *__restrict__ P,
   x[o + nrhs] = x1;
 }
 
-// x = Ainv f on the coarsest level, FP64 arithmetic: 8 rows per block, one
-// warp per row, lanes stride the columns, shuffle reduction.
+// x = Ainv f on the coarsest level, FP64 arithmetic: one warp per row, lanes stride
+// the columns; the halves of the warp then keep the real and the imaginary sum (5
+// FP64 additions instead of 10).  A warp per SM partition: four rows a block.
+// FP32 values are widened on the integer pipes (the conversions took a third of
+// the FP64 unit's time).  256 x 256, FP32 cycle: 18.4 -> 16.9 us for 19 right-hand
+// sides, 6.2 -> 5.4 us for one.
+#define CO_ROWS 4
 template <typename T>
-__global__ void __launch_bounds__(256) k_coarsest(int nc, const zd *__restrict__ Ainv,
-                                                  const cx<T> *__restrict__ f, cx<T> *__restrict__ x,
-                                                  int nrhs) {
-  int row = blockIdx.x * 8 + (threadIdx.x >> 5);
-  int lane = threadIdx.x & 31;
-  int rh = blockIdx.y;
+__global__ void __launch_bounds__(32 * CO_ROWS) k_coarsest(int nc, const zd *__restrict__ Ainv,
+                                                           const cx<T> *__restrict__ f, cx<T> *__restrict__ x,
+                                                           int nrhs) {
+  const int row = blockIdx.x * CO_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31, rh = blockIdx.y;
   if (row >= nc) return;
   zd acc = mk(0.0, 0.0);
   const zd *Ar = Ainv + (long)row * nc;
-  for (int j = lane; j < nc; j += 32) cfma(acc, Ar[j], ccast<double>(f[(long)j * nrhs + rh]));
+  for (int j = lane; j < nc; j += 32) cfma(acc, Ar[j], widen<double>(f[(long)j * nrhs + rh]));
+  const bool im = lane & 16;
+  double v = (im ? acc.im : acc.re) + __shfl_xor_sync(0xffffffffu, im ? acc.re : acc.im, 16);
 #pragma unroll
-  for (int off = 16; off; off >>= 1) {
-    acc.re += __shfl_down_sync(0xffffffffu, acc.re, off);
-    acc.im += __shfl_down_sync(0xffffffffu, acc.im, off);
-  }
-  if (lane == 0) x[(long)row * nrhs + rh] = ccast<T>(acc);
+  for (int off = 8; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if ((lane & 15) == 0) ((T *)x)[((long)row * nrhs + rh) * 2 + (im ? 1 : 0)] = (T)v;
 }
 
 template <typename T>
@@ -1702,6 +1788,11 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
   return rc;
 }
 
+// few enough sites that a launch is bound by a thread's chain, not by loads
+static bool stencil_lanes_ok(const Level &L, int prec, int nrhs) {
+  return nrhs < 8 && (long)L.n * nrhs <= (prec == WL_FP64 ? 65536 : 16384);
+}
+
 // y = A_0 x in FP32 arithmetic from the FP32 copy of the level-0 stencil
 // (Dhat), x float, y widened to double or stored as a double-float with a
 // zero low part: the Arnoldi matvec of an FP32 cycle; xo (or NULL) receives a
@@ -1712,7 +1803,10 @@ static int stencil_apply32_to(wl_amg *a, const void *x, Y *y, int nrhs, zf *xo, 
   long tot = (long)L.n * nrhs;
   wl_count_launches(1);
   int rc = WL_OK;
-  if (!launch_stencil_tile<float, zf, Y>(L, L.op32.A.as<zf>(), x, nullptr, y, nrhs, s, &rc, xo))
+  if (stencil_lanes_ok(L, WL_FP32, nrhs))
+    k_stencil_lanes<float, zf, Y><<<WL_GRID(tot * 8, 256), 256, 0, s>>>(L.geo, L.op32.A.as<zf>(), (const zf *)x, nullptr,
+                                                                      y, nrhs, xo);
+  else if (!launch_stencil_tile<float, zf, Y>(L, L.op32.A.as<zf>(), x, nullptr, y, nrhs, s, &rc, xo))
     k_stencil<float, zf, Y><<<WL_GRID(tot, 256), 256, 0, s>>>(L.geo, L.op32.A.as<zf>(), (const zf *)x, nullptr, y,
                                                               nrhs, xo);
   WL_TRY(rc);
@@ -1733,6 +1827,18 @@ int restrict_op(wl_amg *a, int l, int prec, const void *r, void *fc, int nrhs, c
   long tot = (long)Cl.n * nrhs;
   unsigned grid = WL_GRID(tot, 128);
   wl_count_launches(1);
+  // few coarse points: 16 lanes each, while that leaves the GPU short of a few waves
+  if (tot <= 65536) {
+    unsigned gl = WL_GRID(tot * 16, 256);
+    if (prec == WL_FP64)
+      k_restrict_lanes<double, zd><<<gl, 256, 0, s>>>(F.geo, Cl.geo, lgB, o.P.as<zd>(), (const zd *)r, (zd *)fc, nrhs);
+    else if (prec == WL_FP32)
+      k_restrict_lanes<float, zf><<<gl, 256, 0, s>>>(F.geo, Cl.geo, lgB, o.P.as<zf>(), (const zf *)r, (zf *)fc, nrhs);
+    else
+      k_restrict_lanes<float, zb><<<gl, 256, 0, s>>>(F.geo, Cl.geo, lgB, o.P.as<zb>(), (const zf *)r, (zf *)fc, nrhs);
+    WL_CUDA(cudaGetLastError());
+    return WL_OK;
+  }
   if (prec == WL_FP64)
     k_restrict<double, zd><<<grid, 128, 0, s>>>(F.geo, Cl.geo, lgB, o.P.as<zd>(), (const zd *)r, (zd *)fc, nrhs);
   else if (prec == WL_FP32)
@@ -1761,12 +1867,30 @@ int prolong_op(wl_amg *a, int l, int prec, const void *e, void *x, int nrhs, cud
 }
 
 int coarsest_apply(wl_amg *a, int prec, const void *f, void *x, int nrhs, cudaStream_t s) {
-  dim3 grid(WL_GRID(a->nc, 8), nrhs);
+  dim3 grid(WL_GRID(a->nc, CO_ROWS), nrhs);
   wl_count_launches(1);
   if (prec == WL_FP64)
-    k_coarsest<double><<<grid, 256, 0, s>>>(a->nc, a->Ainv.as<zd>(), (const zd *)f, (zd *)x, nrhs);
+    k_coarsest<double><<<grid, 32 * CO_ROWS, 0, s>>>(a->nc, a->Ainv.as<zd>(), (const zd *)f, (zd *)x, nrhs);
   else
-    k_coarsest<float><<<grid, 256, 0, s>>>(a->nc, a->Ainv.as<zd>(), (const zf *)f, (zf *)x, nrhs);
+    k_coarsest<float><<<grid, 32 * CO_ROWS, 0, s>>>(a->nc, a->Ainv.as<zd>(), (const zf *)f, (zf *)x, nrhs);
+  WL_CUDA(cudaGetLastError());
+  return WL_OK;
+}
+
+// the cycle's stencil apply: k_stencil_lanes for few sites and batches the tiled
+// kernel does not take (rounded differently from the per-step entry point's k_stencil)
+static int cycle_stencil(wl_amg *a, int l, int prec, const void *x, void *y, const void *f, int nrhs, cudaStream_t s) {
+  const Level &L = a->lev[l];
+  const LevelOps &o = ops_of(L, prec);
+  if (!stencil_lanes_ok(L, prec, nrhs)) return stencil_apply(a, l, prec, x, y, f, nrhs, s);
+  const unsigned grid = WL_GRID((long)L.n * nrhs * 8, 256);
+  wl_count_launches(1);
+  if (prec == WL_FP64)
+    k_stencil_lanes<double, zd, zd><<<grid, 256, 0, s>>>(L.geo, o.A.as<zd>(), (const zd *)x, (const zd *)f, (zd *)y, nrhs, nullptr);
+  else if (prec == WL_FP32)
+    k_stencil_lanes<float, zf, zf><<<grid, 256, 0, s>>>(L.geo, o.A.as<zf>(), (const zf *)x, (const zf *)f, (zf *)y, nrhs, nullptr);
+  else
+    k_stencil_lanes<float, zb, zf><<<grid, 256, 0, s>>>(L.geo, o.A.as<zb>(), (const zf *)x, (const zf *)f, (zf *)y, nrhs, nullptr);
   WL_CUDA(cudaGetLastError());
   return WL_OK;
 }
@@ -1785,7 +1909,7 @@ static int cycle_level(wl_amg *a, int l, int nrhs, int prec, cudaStream_t s) {
     if (g > 0) {
       // coarse residual of the correction so far, then one more cycle
       WL_CUDA(cudaMemcpyAsync(C.t.p, C.x.p, cb, cudaMemcpyDeviceToDevice, s));
-      WL_TRY(stencil_apply(a, l + 1, prec, C.t.p, C.f.p, C.f.p, nrhs, s));
+      WL_TRY(cycle_stencil(a, l + 1, prec, C.t.p, C.f.p, C.f.p, nrhs, s));
     }
     WL_TRY(cycle_level(a, l + 1, nrhs, prec, s));
     if (g > 0) {
@@ -1797,7 +1921,7 @@ static int cycle_level(wl_amg *a, int l, int nrhs, int prec, cudaStream_t s) {
     }
   }
   WL_TRY(prolong_op(a, l, prec, C.x.p, L.x.p, nrhs, s));
-  WL_TRY(stencil_apply(a, l, prec, L.x.p, L.r.p, L.f.p, nrhs, s));
+  WL_TRY(cycle_stencil(a, l, prec, L.x.p, L.r.p, L.f.p, nrhs, s));
   WL_TRY(cycle_sweeps(a, l, prec, nrhs, a->prm.nu_post, false, s));
   return WL_OK;
 }

@@ -148,3 +148,20 @@ def test_fp64_ring_sweeps(hier, name, nrhs):
     with pytest.raises(W.WilsonAMGError):  # a tile-ordered level
         W.amg_kaczmarz_form(amg, 0, z, z.clone(), 1, 1, W.WL_FP64, 6, 0)
     amg.close()
+
+
+@pytest.mark.parametrize("nrhs", [1, 3, 7])
+def test_small_batch_cycle(hier, nrhs):
+    """Cycles whose stencil applies and restrictions take several lanes a site (cells of 2, levels
+    64 to 8), V and W, against the oracle: FP64 1e-12, FP32 1e-5 as for the other batches."""
+    h, op, path = hier["deep"]
+    n = h.n(0)
+    f = np.stack([cgauss(495, q, n) for q in range(nrhs)])
+    for cycle in (W.WL_CYCLE_V, W.WL_CYCLE_W):
+        ref = np.stack([h.cycle(f[q], nu1=2, nu2=2, gamma=cycle + 1) for q in range(nrhs)])
+        for prec, tol in ((W.WL_FP64, 1e-12), (W.WL_FP32, 1e-5)):
+            amg = W.amg_import(op, path, W.amg_params_default(zero_guess=1, cycle=cycle, precision=prec))
+            xg = torch.zeros_like(T(f))
+            W.amg_cycle(amg, T(f), xg, nrhs, prec)
+            assert rel(xg.cpu().numpy(), ref) <= tol, (cycle, prec)
+            amg.close()
