@@ -745,14 +745,20 @@ __global__ void __launch_bounds__(W *C * 12 / NI) k_ring_update(Geo g, int pass,
       a[i][2 * k + 1] = p[2];
     }
   }
-  constexpr int NV = ((W + 2) * C * 8 + NT - 1) / NT;  // solution items a thread
+  // solution items: lane (component, row, hh) takes the columns of unknown hh of the
+  // six sites 0..5 from the cell's first; a site of colour j needs its own colours
+  // up to j, the next cell's first for j >= 2 and its second for j = 3.  With C >= 4 a
+  // warp is one position, so the others cost it nothing (3.25 of 6 on average).
+  constexpr int NV = ((W + 2) * C * 8 + NT - 1) / NT;  // items a thread
+  auto needed = [](int j, int k) { return k <= j || (k == 4 && j >= 2) || (k == 5 && j == 3); };
   zd tv[NV][6];
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
     int e = tid + i * NT, uu = min((e >> 3) / C, W + 1), u = (u0 + uu - 1) & (N - 1);
-    const zd *Tp = T + ((((long)pass * (N / 8) + ring) * N + u) * 2 + ((e >> 1) & 1)) * 12 + ((e >> 2) & 1) * 6;
+    const zd *Tp = T + ((((long)pass * (N / 8) + ring) * N + u) * 2 + ((e >> 1) & 1)) * 12 + ((e >> 2) & 1);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) tv[i][k] = Tp[k];
+    for (int k = 0; k < 6; ++k)
+      if (needed(u & 3, k)) tv[i][k] = Tp[2 * k];
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;");
@@ -774,11 +780,12 @@ __global__ void __launch_bounds__(W *C * 12 / NI) k_ring_update(Geo g, int pass,
       zd nv[6];
 #pragma unroll
       for (int k = 0; k < 6; ++k) {
-        int kk = hh * 6 + k, us = ((u & ~3) + (kk >> 1)) & (N - 1);
-        nv[k] = *(const zd *)(num + ((((long)ring * N + us) * 2 + (kk & 1)) * nrhs + r0 + cc) * 2);
+        int us = ((u & ~3) + k) & (N - 1);
+        if (needed(u & 3, k)) nv[k] = *(const zd *)(num + ((((long)ring * N + us) * 2 + hh) * nrhs + r0 + cc) * 2);
       }
 #pragma unroll
-      for (int k = 0; k < 6; ++k) rb_cfma(v, tv[i][k], nv[k], c);
+      for (int k = 0; k < 6; ++k)
+        if (needed(u & 3, k)) rb_cfma(v, tv[i][k], nv[k], c);
     }
     v += __shfl_xor_sync(0xffffffffu, v, 4);
     if (on && hh == 0) sm[uu][t][cc][c] = v;
