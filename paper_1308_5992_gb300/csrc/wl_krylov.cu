@@ -108,6 +108,19 @@ __global__ void k_mdot(const cx<Tv> *__restrict__ V, long vstride, const zd *__r
 #pragma unroll
   for (int k = 0; k < KC; ++k) sm[k * nt + t] = acc[k];
   __syncthreads();
+  if (R == 1) {  // G = 256: a warp per dot (a tree over all dots is 8 levels of 2 KC FP64 additions)
+    const int lane = t & 31;
+    for (int k = t >> 5; k < KC; k += nt >> 5) {
+      zd s = sm[k * nt + lane];
+      for (int i = lane + 32; i < nt; i += 32) s = s + sm[k * nt + i];
+      const bool im = lane & 16;  // real sums in the lower half of the warp, imaginary in the upper
+      double v = (im ? s.im : s.re) + __shfl_xor_sync(0xffffffffu, im ? s.re : s.im, 16);
+#pragma unroll
+      for (int off = 8; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+      if ((lane & 15) == 0) ((double *)(part + (long)blockIdx.x * KC + k))[im ? 1 : 0] = v;
+    }
+    return;
+  }
   for (int s = G >> 1; s > 0; s >>= 1) {
     if (q < s)
 #pragma unroll
@@ -436,46 +449,42 @@ __global__ void __launch_bounds__(FIN_T) k_mdot_final_df(const float4 *__restric
 
 // w -= sum_k V_k c_k[r] in double-float (c from k_mdot_final_df): P sums
 // (cr vr, cr vi) and Q sums (ci vr, -ci vi), so Re = P.x + Q.y and
-// Im = P.y + Q.x; the k loop is unrolled by 4 with the loads issued first.
-// With part != NULL the squared norm of the new w is summed as well, in the
-// thread layout of k_mdot_df (a fixed grid, thread t on right-hand side
-// t % R), and written as k_mdot_df's partials of one dot with B = 0: one
-// pass over w instead of two.
-__global__ void __launch_bounds__(256) k_maxpy_df(const zdf *__restrict__ V, long vstride, int kc,
-                                                  const float4 *__restrict__ coef, zdf *__restrict__ w, long E,
-                                                  int R, float4 *__restrict__ part) {
+// Im = P.y + Q.x.  The thread layout of k_mdot_df (a fixed grid, thread t on
+// right-hand side t % R).  Bound by HBM: four basis vectors are loaded while the
+// four before them are summed, and w first of all (loads and sums in turn took
+// their times together, 560 us a launch at 1024 x 1024 with 16 right-hand sides).
+// With part != NULL the squared norm of the new w is summed as well and written as
+// k_mdot_df's partials of one dot with B = 0: one pass over w instead of two.
+__global__ void __launch_bounds__(256, 3) k_maxpy_df(const zdf *__restrict__ V, long vstride, int kc,
+                                                     const float4 *__restrict__ coef, zdf *__restrict__ w, long E,
+                                                     int R, float4 *__restrict__ part) {
   __shared__ float4 sm[256];
   int t = threadIdx.x, nt = blockDim.x;
   DF2 N2{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
   long stride = (long)gridDim.x * nt;
+  const float4 *cr = coef + (t % R) * 2;
   for (long e = (long)blockIdx.x * nt + t; e < E; e += stride) {
-    int r = (int)(e % R);
     DF2 P{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, Q = P;
-    auto step = [&](float4 v, float4 c0, float4 c1) {
-      float2 vh = make_float2(v.x, v.y), vl = make_float2(v.z, v.w);
-      df_acc(P, make_float2(c0.x, c0.y), make_float2(c0.z, c0.w), vh, vl);
-      df_acc(Q, make_float2(c1.x, c1.y), make_float2(c1.z, c1.w), vh, vl);
-    };
-    int k = 0;
-    for (; k + 4 <= kc; k += 4) {
-      float4 v[4], c[4][2];
+    float4 wv = ld4(w + e), v[4], nv[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = ld4(V + (k + u) * vstride + e);
+    for (int u = 0; u < 4; ++u)
+      if (u < kc) v[u] = ld4(V + u * vstride + e);
+    for (int k = 0; k < kc; k += 4) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k + 4 + u < kc) nv[u] = ld4(V + (k + 4 + u) * vstride + e);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const float4 *cp = coef + ((long)(k + u) * R + r) * 2;
-        c[u][0] = cp[0];
-        c[u][1] = cp[1];
+        if (k + u >= kc) break;
+        const float4 c0 = cr[(long)(k + u) * R * 2], c1 = cr[(long)(k + u) * R * 2 + 1];
+        float2 vh = make_float2(v[u].x, v[u].y), vl = make_float2(v[u].z, v[u].w);
+        df_acc(P, make_float2(c0.x, c0.y), make_float2(c0.z, c0.w), vh, vl);
+        df_acc(Q, make_float2(c1.x, c1.y), make_float2(c1.z, c1.w), vh, vl);
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) step(v[u], c[u][0], c[u][1]);
-    }
-    for (; k < kc; ++k) {
-      const float4 *cp = coef + ((long)k * R + r) * 2;
-      step(ld4(V + k * vstride + e), cp[0], cp[1]);
+      for (int u = 0; u < 4; ++u) v[u] = nv[u];
     }
     df_add(P, DF2{swap2(Q.s), swap2(Q.c)});
-    float4 wv = ld4(w + e);
     DF2 Wn{make_float2(wv.x, wv.y), make_float2(wv.z, wv.w)};
     df_add(Wn, DF2{neg2(P.s), neg2(P.c)});
     st4(w + e, Wn.s, Wn.c);
@@ -921,7 +930,8 @@ int fg_cycle(wl_amg *a, const zd *bnorm_h, zd *xh, int nrhs, double tol, const i
         if (pass + 1 == a->prm.gs_passes) {  // the last pass also forms |w|^2
           WL_TRY(maxpy_norm_df(a, Vd, vs, j + 1, k.hpd, wd, E, nrhs, k.nrm2, k.running, s));
         } else {
-          k_maxpy_df<<<gE, 256, 0, s>>>(Vd, vs, j + 1, k.hpd, wd, E, nrhs, nullptr);
+          RedCfg c = red_cfg(E, nrhs);
+          k_maxpy_df<<<c.nblk, c.nt, 0, s>>>(Vd, vs, j + 1, k.hpd, wd, E, nrhs, nullptr);
           wl_count_launches(1);
         }
       } else {
@@ -1371,9 +1381,10 @@ extern "C" int wl_time_kernel(wl_amg *a, int kind, int level, int nrhs, int prec
         return WL_OK;
       }
       default:
-        if (a->prm.gs_arith == 1)
-          k_maxpy_df<<<WL_GRID(E, 256), 256, 0, s>>>(a->V.as<zdf>(), E, kc, k.hpd, a->w.as<zdf>(), E, nrhs, nullptr);
-        else
+        if (a->prm.gs_arith == 1) {
+          wl::RedCfg c = wl::red_cfg(E, nrhs);
+          k_maxpy_df<<<c.nblk, c.nt, 0, s>>>(a->V.as<zdf>(), E, kc, k.hpd, a->w.as<zdf>(), E, nrhs, nullptr);
+        } else
           k_maxpy<double, 1><<<WL_GRID(E, 256), 256, 0, s>>>(a->V.as<zd>(), E, kc, k.hpass, nrhs, a->w.as<zd>(), E,
                                                               nrhs);
         wl_count_launches(1);
