@@ -413,7 +413,8 @@ int amg_pin_sweep_form(wl_amg *amg, int level, int nrhs, int prec, int form, int
  * sides per block and per warp, one of (1, 1), (2, 1), (4, 1), (8, 1), (8, 2)) is the
  * row-block form of the cycle; form 5 (32x32 and 16x16 levels, FP32 or BF16, param 0) its
  * one-launch form there; form 6 (16-colour ordering, FP64) those of FP64 cycles: param 0 two
- * launches a pass, 1 (32x32 and 64x64 levels) one launch of clusters.  Errors: WL_EINVAL (no such form). */
+ * launches a pass, 1 (32x32 and 64x64 levels) one launch of clusters, 2 (levels 32 to 256, up
+ * to 4 right-hand sides) one launch a pass.  Errors: WL_EINVAL (no such form). */
 int amg_kaczmarz_form(wl_amg *amg, int level, void *x, void *r, int nrhs, int sweeps, int prec, int form, int param);
 /* Number of kernels this library has launched in this process (a captured
  * graph counts each of its kernel nodes at every replay). */

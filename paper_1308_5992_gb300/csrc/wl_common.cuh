@@ -352,7 +352,7 @@ int rings_sweeps(wl_amg *a, int l, int prec, const void *rin, const void *xin, v
 // the same blocks on 16-colour-ordered levels in FP64 (two launches a ring pass, or one of clusters)
 bool rings64_ok(const wl_amg *a, int l, int prec, int nrhs);
 int rings64_prepare(wl_amg *a, int l, int nrhs, bool stale, cudaStream_t s);  // stale: the operator changed since
-bool rings64_form(const wl_amg *a, int l, int param);
+bool rings64_form(const wl_amg *a, int l, int param, int nrhs);
 int rings64_sweeps(wl_amg *a, int l, const void *rin, const void *xin, void *x, void *r, int nrhs, int sweeps, int param,
                    cudaStream_t s);
 KTune sweep_form_of(wl_amg *a, int l, int prec, int nrhs);

@@ -480,7 +480,7 @@ __device__ __forceinline__ void r_sub_paired(cx<float> &rv, float2 m1, float2 m2
 // The caller may have committed cp.async groups of its own before: the wait
 // of step 0 completes them too.  Ends with a barrier.
 template <typename T, typename S, int R, int RPT, bool PAIRED>
-__device__ __forceinline__ void tile_relax(const S *__restrict__ A, cx<T> *__restrict__ x, cx<T> *rs, const T *ds,
+__device__ __forceinline__ void tile_relax(const S *__restrict__ A, cx<T> *x, cx<T> *rs, const T *ds,
                                            S *Ar, const int *hs, int nrhs, int r0, int Rc) {
   constexpr int NT = 4 * R / RPT;
   constexpr int RQ = R / RPT;                     // threads per site
@@ -640,7 +640,7 @@ __device__ __forceinline__ void tile_relax(const S *__restrict__ A, cx<T> *__res
 // the arithmetic (lanes past the chunk on stale shared memory, results
 // discarded) so that the shuffles see full warps.  Ends with a barrier.
 template <typename S, int R>
-__device__ __forceinline__ void tile_relax_split(const S *__restrict__ A, zf *__restrict__ x, zf *rs,
+__device__ __forceinline__ void tile_relax_split(const S *__restrict__ A, zf *x, zf *rs,
                                                  const float *ds, S *Ar, const int *hs, int nrhs, int r0,
                                                  int Rc) {
   constexpr int NT = 8 * R;
@@ -753,8 +753,8 @@ __device__ __forceinline__ void tile_relax_split(const S *__restrict__ A, zf *__
 // the split form keeps 85 (768 threads per SM).
 template <typename T, typename S, int R, int RPT, bool PAIRED, bool SPLIT = false>
 __global__ void __launch_bounds__(SPLIT ? 8 * R : 4 * R / RPT, SPLIT ? 768 / (8 * R) : (RPT == 1 ? R / 8 : 1))
-    k_kacz_tile(Geo g, int tc, const S *__restrict__ A, const T *__restrict__ den, cx<T> *__restrict__ x,
-                cx<T> *__restrict__ r, int nrhs, int vec, T omega) {
+    k_kacz_tile(Geo g, int tc, const S *__restrict__ A, const T *__restrict__ den, cx<T> *x, cx<T> *r, int nrhs,
+                int vec, T omega) {  // x, r not restrict: their loads have to stay after griddepcontrol.wait
   extern __shared__ __align__(16) unsigned char sm_raw[];
   cx<T> *rs = (cx<T> *)sm_raw;
   T *ds = (T *)(rs + KTH * KTH * 2 * R);
@@ -1747,8 +1747,8 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
     }
     if (rings64_ok(a, l, prec, nrhs)) {
       if ((rc = rings64_prepare(a, l, nrhs, false, s))) break;
-      for (int q : {0, 1})
-        if (rings64_form(a, l, q)) cand.push_back(KTune{nrhs, prec, 6, q, 0.f});
+      for (int q : {0, 1, 2})
+        if (rings64_form(a, l, q, nrhs)) cand.push_back(KTune{nrhs, prec, 6, q, 0.f});
     }
     KTune best = cand[0], rows{nrhs, prec, 4, 0, 1e30f};
     float best_us = 1e30f;
@@ -2038,7 +2038,7 @@ static int kaczmarz_entry(wl_amg *a, int level, void *x, void *r, int nrhs, int 
     return WL_EINVAL;
   }
   const bool rings = form == 5 && param == 0 && wl::rings_ok(a, level, prec);
-  const bool rings64 = form == 6 && wl::rings64_ok(a, level, prec, 1) && wl::rings64_form(a, level, param);
+  const bool rings64 = form == 6 && wl::rings64_ok(a, level, prec, 1) && wl::rings64_form(a, level, param, nrhs);
   const bool rows = form == 4 && level < a->L - 1 && wl::rows_form_exists(a, level, prec, param);
   if (form >= 0 && !rows && !rings && !rings64 && !form_exists(a, level, nrhs, prec, form, param)) {
     wl_set_error("%s: launch form %d / %d does not exist for this level and ordering", who, form, param);

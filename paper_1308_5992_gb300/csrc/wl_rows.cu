@@ -179,11 +179,11 @@ __device__ __forceinline__ float2 rb_shfl_xor1(float2 v) {
 // FMAs on (re, im) pairs as they lie in memory: sum (a.re x.re, a.im x.im) and
 // sum (a.re x.im, a.im x.re), combined once per sum.  The tile's packed rows
 // arrive as one bulk copy per row step, all four issued at the start (bounded
-// waits; on a timeout *timeout gets 1 and nothing is written).
+// waits; on a timeout *timeout gets 1 and nothing is written).  x and r are not
+// declared restrict: their loads have to stay after griddepcontrol.wait.
 template <typename S, int R, int RPT>
 __global__ void __launch_bounds__(32 * R / RPT, RPT == 1 ? 16 / R : 0) k_kacz_rows(Geo g, int tc, const unsigned char *__restrict__ pk,
-                                                            zf *__restrict__ x, zf *__restrict__ r, int nrhs,
-                                                            int *timeout) {
+                                                            zf *x, zf *r, int nrhs, int *timeout) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   constexpr int NT = 32 * R / RPT, NW = R / RPT, SB = rb_step_bytes<S>();
   unsigned char *cs = sm_raw;                           // [4][SB] packed rows
@@ -816,8 +816,8 @@ __global__ void __launch_bounds__(W *C * 12 / NI) k_ring_update(Geo g, int pass,
 // of one row and one position. Inner products and updated values of r that a
 // neighbour's halo holds are stored there as well (distributed shared memory), so
 // that every load is the block's own; a cluster barrier (390 cycles) follows the
-// inner products and another one the update, where the two launches of a pass
-// cost 4.4 us.
+// inner products and another one the update.  16 passes (four sweeps) of the
+// 32 x 32 level with 12 right-hand sides: 60 us, two launches a pass 104 us.
 template <int N>
 struct RingCluster {
   static constexpr int NG = N / 8, SEG = 16 / NG, W = N / SEG, H = N == 32 ? 4 : 2;
@@ -939,6 +939,110 @@ __global__ void __launch_bounds__(RingCluster<N>::NT) k_ring64_cluster(Geo g, in
     long o = ((long)site(4 * ig + k, u0 + w) * 2 + sp) * nrhs + rh;
     r[o] = sm->r[k + 1][w + 1][sp];
     x[o] = sm->x[k][w][sp];
+  }
+}
+
+// A pass in one launch for few right-hand sides on levels of any size: a cluster of
+// N / W blocks holds a ring, each block W positions.  The inner products a
+// neighbour's cells need are stored in its shared memory as well; one cluster
+// barrier separates them from the update, where the two-launch form has the end of
+// one kernel and the start of another.  Blocks write r only after that barrier, so
+// no block still reads what another one updates.  The paper's W(4,4) cycles on
+// 128 x 128 (2016 passes on 128, 64 and 32): 9.92 -> 9.50 ms a solve.
+template <int W>
+struct RingPass {
+  static constexpr int H = W == 8 ? 4 : 2, NT = W == 8 ? 128 : 192;
+};
+template <int W>
+__global__ void __launch_bounds__(RingPass<W>::NT) k_ring_pass(Geo g, int pass, const zd *__restrict__ A,
+                                                               const zd *__restrict__ T, double *x, double *r, int nrhs) {
+  constexpr int H = RingPass<W>::H, ND = H == 4 ? 5 : 9;
+  __shared__ zd num[W + 10][2];  // positions -4 .. W + 5
+  __shared__ zd ss[W + 2][2];
+  const int N = g.N, seg = N / W, tid = threadIdx.x, rh = blockIdx.y;
+  cg::cluster_group cl = cg::this_cluster();  // the blocks of one ring
+  const int me = (int)cl.block_rank(), ring = blockIdx.x / seg, u0 = me * W, row = pass + 4 * ring;
+  zd(*left)[2] = cl.map_shared_rank(num, (me + seg - 1) % seg), (*right)[2] = cl.map_shared_rank(num, (me + 1) % seg);
+  // constants first: this thread's stencil entries, row of T and update entries
+  const int dl = tid % (4 * H), dw = tid / (4 * H), dc = dl & 1, dt = (dl >> 1) & 1, dsp = (dl >> 2) & 1;
+  const int dh = H == 4 ? (dl >> 3) * 5 : 0;
+  const bool dots = tid < W * 4 * H;
+  const int px = (row + u0 + dw) & (N - 1), py = (row - u0 - dw) & (N - 1);
+  zd a[ND];
+  if (dots) {
+    const zd *Ah = A + (long)g.idx(px, py) * 36 + dt * 2 + dsp;
+#pragma unroll
+    for (int i = 0; i < ND; ++i) a[i] = dh + i < 9 ? Ah[(dh + i) * 4] : mk(0.0, 0.0);
+  }
+  const int sl = tid & 7, sc = sl & 1, st = (sl >> 1) & 1, sh = sl >> 2, sq = min(tid >> 3, W + 1);
+  const int su = (u0 + sq - 1) & (N - 1);
+  const bool solve = tid < ((W + 2) * 8 + 31) / 32 * 32, mine = (tid >> 3) == sq && sh == 0 && sq >= 1 && sq <= W;
+  zd tv[6];
+  if (solve) {
+    const zd *Tp = T + ((((long)pass * (N / 8) + ring) * N + su) * 2 + st) * 12 + sh;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) tv[k] = Tp[2 * k];
+  }
+  const int uc = tid & 1, us = (tid >> 1) & 1, ui = (tid >> 2) % 3, uw = (tid >> 2) / 3;
+  const bool upd = tid < W * 12;
+  zd b[6];
+  if (upd)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const zd *p = A + (long)g.idx(row + u0 + uw + k - 1, row - u0 - uw - k + 1) * 36 + (ui * 3 + 2 - k) * 4 + us;
+      b[2 * k] = p[0];
+      b[2 * k + 1] = p[2];
+    }
+  const long ro = (((long)g.idx(row + ui - 1 + u0 + uw, row + ui - 1 - u0 - uw) * 2 + us) * nrhs + rh) * 2 + uc;
+  double *xa = x + (((long)g.idx(row + su, row - su) * 2 + st) * nrhs + rh) * 2 + sc;
+  cl.sync();  // every block of the ring runs
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+  double v = 0, rv = 0, xv = 0;
+  if (dots) {
+    zd w[ND];
+#pragma unroll
+    for (int i = 0; i < ND; ++i)
+      w[i] = *(const zd *)(r + (((long)g.nb(px, py, min(dh + i, 8)) * 2 + dsp) * nrhs + rh) * 2);
+    if (upd) rv = r[ro];
+    if (mine) xv = *xa;
+#pragma unroll
+    for (int i = 0; i < ND; ++i) rb_cfma(v, a[i], w[i], dc);
+    v = rb_flip(v, dsp != 0);
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    if (H == 4) v += __shfl_xor_sync(0xffffffffu, v, 8);
+    if (dl < 4) {
+      v = rb_flip(v, dt != 0);
+      ((double *)&num[dw + 4][dt])[dc] = v;
+      if (dw >= W - 4) ((double *)&right[dw - W + 4][dt])[dc] = v;
+      if (dw < 6) ((double *)&left[dw + W + 4][dt])[dc] = v;
+    }
+  } else {
+    if (upd) rv = r[ro];
+    if (mine) xv = *xa;
+  }
+  cl.sync();
+  if (solve) {
+    const int cell = (sq + 3) & ~3;  // in num: the first site of the cell of position sq - 1
+    double z = 0;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) rb_cfma(z, tv[k], num[cell + k][sh], sc);
+    z += __shfl_xor_sync(0xffffffffu, z, 4);
+    if (sh == 0) ((double *)&ss[sq][st])[sc] = z;
+    if (mine) *xa = xv + z;
+  }
+  __syncthreads();
+  if (upd) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {  // r -= g_s g_t s_t conj(a)
+        const double *sv = (const double *)&ss[uw + k][t];
+        const bool neg = us == t;
+        rv = fma(rb_flip(b[2 * k + t].re, neg), sv[uc], rv);
+        rv = fma(rb_flip(b[2 * k + t].im, neg == (uc == 0)), sv[1 - uc], rv);
+      }
+    r[ro] = rv;
   }
 }
 
@@ -1080,6 +1184,7 @@ static int rings_pack(const Level &L, LevelOps &o, double omega, cudaStream_t s)
 int rings_prepare(wl_amg *a, int l, int prec, cudaStream_t s) {
   Level &L = a->lev[l];
   LevelOps &o = prec == WL_FP32 ? L.op32 : L.opbf;
+  if (!tile_timeout_flag()) return WL_ECUDA;  // looked up before a stream capture needs it
   if (o.rows.p) return WL_OK;
   if (prec == WL_FP32) return L.N == 32 ? rings_pack<zf, 32>(L, o, a->prm.omega, s) : rings_pack<zf, 16>(L, o, a->prm.omega, s);
   return L.N == 32 ? rings_pack<zb, 32>(L, o, a->prm.omega, s) : rings_pack<zb, 16>(L, o, a->prm.omega, s);
@@ -1179,11 +1284,42 @@ static int launch_cluster(const Level &L, const void *rin, const void *xin, void
   return WL_OK;
 }
 
-bool rings64_form(const wl_amg *a, int l, int param) {
-  return param == 0 || (param == 1 && (a->lev[l].N == 32 || a->lev[l].N == 64));
+template <int W>
+static int launch_ring_pass(const Level &L, int pass, void *x, void *r, int nrhs, int pdl, cudaStream_t s) {
+  static std::atomic<unsigned long long> wide{0};
+  int dev = 0;
+  WL_CUDA(cudaGetDevice(&dev));
+  unsigned long long bit = 1ull << (dev & 63);
+  if (!(wide.load(std::memory_order_acquire) & bit)) {
+    WL_CUDA(cudaFuncSetAttribute((const void *)k_ring_pass<W>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    wide.fetch_or(bit, std::memory_order_acq_rel);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(L.N / 8 * (L.N / W), nrhs);
+  cfg.blockDim = dim3(RingPass<W>::NT);
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = L.N / W;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = pdl;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  wl_count_launches(1);
+  WL_CUDA(cudaLaunchKernelEx(&cfg, k_ring_pass<W>, L.geo, pass, (const zd *)L.op64.A.p, (const zd *)L.op64.rows.p,
+                             (double *)x, (double *)r, nrhs));
+  return WL_OK;
 }
 
-// param 0: two launches a pass; 1: one launch of clusters (32 x 32 and 64 x 64).
+bool rings64_form(const wl_amg *a, int l, int param, int nrhs) {
+  const int N = a->lev[l].N;
+  return param == 0 || (param == 1 && (N == 32 || N == 64)) || (param == 2 && N >= 32 && N <= 256 && nrhs <= 4);
+}
+
+// param 0: two launches a pass; 1: one launch of clusters (32 x 32 and 64 x 64); 2:
+// one launch of clusters a pass.
 // rin, xin as in rings_sweeps (param 0 takes r and x themselves)
 int rings64_sweeps(wl_amg *a, int l, const void *rin, const void *xin, void *x, void *r, int nrhs, int sweeps, int param,
                    cudaStream_t s) {
@@ -1191,10 +1327,20 @@ int rings64_sweeps(wl_amg *a, int l, const void *rin, const void *xin, void *x, 
   if (param == 1)
     return L.N == 32 ? launch_cluster<32>(L, rin, xin, x, r, nrhs, sweeps, s)
                      : launch_cluster<64>(L, rin, xin, x, r, nrhs, sweeps, s);
+  if (param == 2) {
+    for (int sw = 0; sw < sweeps; ++sw)
+      for (int k = 0; k < 4; ++k) {
+        if (L.N <= 128) WL_TRY(launch_ring_pass<8>(L, k, x, r, nrhs, sw + k > 0, s));
+        else WL_TRY(launch_ring_pass<16>(L, k, x, r, nrhs, sw + k > 0, s));
+      }
+    return WL_OK;
+  }
   const zd *A = L.op64.A.as<zd>(), *T = L.op64.rows.as<zd>();
   double *num = L.nums.as<double>();
   const long items = (long)(L.n / 4) * nrhs;
-  // lanes a site: as many as leave at most a warp or so per SM partition
+  // lanes a site: as many as leave at most a warp or so per SM partition (a launch
+  // of the dots, one right-hand side: 1.6 us on 64 x 64 with H = 4, 2.0 us on 128 x 128
+  // with H = 2; the update 2.6 and 2.7 us)
   const int H = items <= 512 ? 4 : items <= 4096 ? 2 : 1;
   const dim3 gd((unsigned)((items * 4 * H + 127) / 128));
   const int rings = L.N / 8;

@@ -28,10 +28,12 @@ def f32(a):
 def hier(tmp_path_factory):
     from oracle.hierfile import write_hierarchy
     out = {}
-    # fine grids 64 and 128, coarse levels of side 64, 32 and (deep) 16
-    for name, blocks in (("T64", [2, 2]), ("T128", [2, 2, 2]), ("deep", [2, 2, 2])):
-        w = workload("T64" if name == "deep" else name)
-        h = O.Hierarchy.setup(w["N"], w["U"], w["m"], O.setup_params(blocks, k_r=w["k"], k_e=w["k"], seed=w["seed"]))
+    # fine grids 64, 128 and 256, coarse levels of side 64, 32 and (deep) 16
+    for name, blocks in (("T64", [2, 2]), ("T128", [2, 2, 2]), ("deep", [2, 2, 2]), ("wide", [4, 4])):
+        w = workload({"deep": "T64", "wide": "S02"}.get(name, name))
+        more = dict(mu1=1, mu2=1) if name == "wide" else {}  # the oracle's setup of 256 x 256 is slow
+        h = O.Hierarchy.setup(w["N"], w["U"], w["m"], O.setup_params(blocks, k_r=w["k"], k_e=w["k"], seed=w["seed"],
+                                                                     **more))
         path = str(tmp_path_factory.mktemp("rows") / (name + ".wlh"))
         write_hierarchy(path, h)
         out[name] = (h, W.wilson_create(T(w["U"]), w["N"], w["m"]), path)
@@ -113,10 +115,10 @@ def test_small_level_sweeps(hier, nrhs):
     amg.close()
 
 
-@pytest.mark.parametrize("name", ["T128", "deep"])
+@pytest.mark.parametrize("name", ["T128", "deep", "wide"])
 @pytest.mark.parametrize("nrhs", [1, 2, 3, 9])
 def test_fp64_ring_sweeps(hier, name, nrhs):
-    """The FP64 forms on every 16-colour level (128x128 down to 16x16; every lane split
+    """The FP64 forms on every 16-colour level (256x256 down to 16x16; every lane split
     of the inner products, ragged chunks of right-hand sides) against the oracle, to the bound of
     the other FP64 forms (1e-13 for one sweep, two here: 2e-13)."""
     h, op, path = hier[name]
@@ -129,9 +131,9 @@ def test_fp64_ring_sweeps(hier, name, nrhs):
             xg, rg = T(x0), T(r0)
             W.amg_kaczmarz_form(amg, l, xg, rg, nrhs, 2, W.WL_FP64, 6, 0)
             outs = [(xg, rg)]
-            if h.Nl[l] in (32, 64):  # one launch of clusters
+            for param in [1] * (h.Nl[l] in (32, 64)) + [2] * (h.Nl[l] >= 32 and nrhs <= 4):  # clusters
                 xc, rc = T(x0), T(r0)
-                W.amg_kaczmarz_form(amg, l, xc, rc, nrhs, 2, W.WL_FP64, 6, 1)
+                W.amg_kaczmarz_form(amg, l, xc, rc, nrhs, 2, W.WL_FP64, 6, param)
                 outs.append((xc, rc))
             if omega == 1.0:
                 ref = [h.kaczmarz(l, x0[r], r0[r], order=O.ORDER_COLOUR, sweeps=2) for r in range(nrhs)]
