@@ -718,6 +718,21 @@ extern "C" int wl_apply(wl_op *op, int which, const void *x, void *y, int nrhs, 
   const bool large = N >= 32 && sites >= 256 * 304;
   const zd *xx = (const zd *)x;
   zd *yy = (zd *)y;
+  // blocks read sites that others write: where x and y share memory (an in-place
+  // call), the kernel reads a copy of x
+  const size_t bytes = sizeof(zd) * 2 * sites;
+  const uintptr_t xa = (uintptr_t)x, ya = (uintptr_t)y;
+  DBuf copy;
+  if ((xa > ya ? xa - ya : ya - xa) < bytes) {
+    WL_TRY(copy.alloc(bytes));
+    cudaError_t e = cudaMemcpyAsync(copy.p, x, bytes, cudaMemcpyDefault, s);
+    if (e != cudaSuccess) {
+      wl_set_error("wl_apply: %s", cudaGetErrorString(e));
+      copy.release();
+      return WL_ECUDA;
+    }
+    xx = copy.as<zd>();
+  }
   if (prec == WL_FP64) {
     if (large) k_dhat_tile<double, 32, 16, 320><<<(unsigned)(sites / 256), 320, 0, s>>>(g, op->Uf64.as<zd>(), xx, yy);
     else k_dhat_tile<double, 8, 8, 64><<<(unsigned)(sites / 32), 64, 0, s>>>(g, op->Uf64.as<zd>(), xx, yy);
@@ -726,8 +741,10 @@ extern "C" int wl_apply(wl_op *op, int which, const void *x, void *y, int nrhs, 
     else k_dhat_tile<float, 8, 8, 64><<<(unsigned)(sites / 32), 64, 0, s>>>(g, op->Uf32.as<zf>(), xx, yy);
   }
   wl_count_launches(1);
-  WL_CUDA(cudaGetLastError());
-  WL_CUDA(cudaStreamSynchronize(s));
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  copy.release();
+  WL_CUDA(e);
   return WL_OK;
 }
 

@@ -47,3 +47,19 @@ def test_fp32_rounds_to_nearest():
             f = float(np.float32(v))
         assert got.real == f and got.imag == -f, (v, got, f)
     op.close()
+
+
+@pytest.mark.parametrize("N,nrhs", [(16, 1), (64, 3), (256, 3), (512, 1)])
+@pytest.mark.parametrize("prec", [W.WL_FP64, W.WL_FP32])
+def test_in_place(N, nrhs, prec):
+    """y = x, and y one right-hand side into x: the same bits as a call on separate arrays."""
+    op = W.wilson_create(torch.from_numpy(metropolis_u1(N, 6.0, 5, 3)).to(DEV), N, -0.05)
+    x = torch.from_numpy(np.stack([cgauss(620 + r, 1, N * N) for r in range(nrhs)])).to(DEV)
+    ref = torch.zeros_like(x)
+    W.wl_apply(op, W.WL_OP_DHAT, x, ref, nrhs, prec)
+    buf = torch.zeros(nrhs + 1, N * N, dtype=torch.complex128, device=DEV)
+    for shift in (0, 1):
+        buf[:nrhs] = x
+        W.wl_apply(op, W.WL_OP_DHAT, buf[:nrhs], buf[shift:shift + nrhs], nrhs, prec)
+        assert torch.equal(buf[shift:shift + nrhs], ref)
+    op.close()
