@@ -1740,15 +1740,19 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
           if (!dup) cand.push_back(KTune{nrhs, prec, 1, b, 0.f});
         }
     }
+    // the row-block forms' constants are memory the others do without: where there is
+    // no room for them, those forms are left out
     if (rows_ok(a, l, prec, nrhs)) {
-      if ((rc = rows_prepare(a, l, prec, s))) break;
-      int prm[8], n = rows_candidates(nrhs, prm);
+      rc = rows_prepare(a, l, prec, s);
+      if (rc && rc != WL_OOM) break;
+      int prm[8], n = rc ? 0 : rows_candidates(nrhs, prm);
       for (int i = 0; i < n; ++i) cand.push_back(KTune{nrhs, prec, 4, prm[i], 0.f});
     }
     if (rings64_ok(a, l, prec, nrhs)) {
-      if ((rc = rings64_prepare(a, l, nrhs, false, s))) break;
+      rc = rings64_prepare(a, l, nrhs, false, s);
+      if (rc && rc != WL_OOM) break;
       for (int q : {0, 1, 2})
-        if (rings64_form(a, l, q, nrhs)) cand.push_back(KTune{nrhs, prec, 6, q, 0.f});
+        if (!rc && rings64_form(a, l, q, nrhs)) cand.push_back(KTune{nrhs, prec, 6, q, 0.f});
     }
     KTune best = cand[0], rows{nrhs, prec, 4, 0, 1e30f};
     float best_us = 1e30f;
@@ -1942,7 +1946,10 @@ int cycle_prepare(wl_amg *a, int nrhs, int prec, cudaStream_t s, const wl_amg::G
     }
   WL_TRY(autotune_sweeps(a, nrhs, prec, s));  // measured launch forms, before the capture
   for (int l = 0; l < a->L - 1; ++l)
-    if (a->prm.sweep_kernel == 0 && rings_ok(a, l, prec)) WL_TRY(rings_prepare(a, l, prec, s));
+    if (a->prm.sweep_kernel == 0 && rings_ok(a, l, prec)) {
+      int rc = rings_prepare(a, l, prec, s);
+      if (rc && rc != WL_OOM) return rc;  // no room: use_rings sees no constants
+    }
   cudaGraph_t graph;
   long long before = wl_launch_count();
   WL_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
