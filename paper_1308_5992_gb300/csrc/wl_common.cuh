@@ -268,7 +268,6 @@ struct Level {
   LevelOps op64, op32, opbf;  // FP64 master, FP32 copy, BF16 copy (den in FP32)
   // cycle work vectors, [n][2][nrhs_cap] in the cycle precision
   DBuf x, r, f, t;
-  DBuf nums;                  // inner products of a ring pass (FP64 16-colour sweeps)
   std::vector<KTune> tune;    // autotuned sweep forms per (nrhs, precision)
   std::vector<KTune> rowtune; // where the row-block sweep measured faster: form 4, param = R | RPT << 8
 };
@@ -351,10 +350,11 @@ int rings_sweeps(wl_amg *a, int l, int prec, const void *rin, const void *xin, v
                  cudaStream_t s);
 // the same blocks on 16-colour-ordered levels in FP64 (two launches a ring pass, or one of clusters)
 bool rings64_ok(const wl_amg *a, int l, int prec, int nrhs);
-int rings64_prepare(wl_amg *a, int l, int nrhs, bool stale, cudaStream_t s);  // stale: the operator changed since
+int rings64_prepare(wl_amg *a, int l, bool stale, cudaStream_t s);  // stale: the operator changed since
 bool rings64_form(const wl_amg *a, int l, int param, int nrhs);
-int rings64_sweeps(wl_amg *a, int l, const void *rin, const void *xin, void *x, void *r, int nrhs, int sweeps, int param,
-                   cudaStream_t s);
+// num: scratch of n / 2 x nrhs complex doubles for a pass's inner products
+int rings64_sweeps(wl_amg *a, int l, const void *rin, const void *xin, void *x, void *r, void *num, int nrhs, int sweeps,
+                   int param, cudaStream_t s);
 KTune sweep_form_of(wl_amg *a, int l, int prec, int nrhs);
 int restrict_op(wl_amg *a, int l, int prec, const void *r, void *fc, int nrhs, cudaStream_t s);
 int prolong_op(wl_amg *a, int l, int prec, const void *e, void *x, int nrhs, cudaStream_t s);

@@ -413,7 +413,6 @@ void amg_free(wl_amg *a) {
     L.r.release();
     L.f.release();
     L.t.release();
-    L.nums.release();
   }
   a->Ainv.release();
   a->Ainv32.release();

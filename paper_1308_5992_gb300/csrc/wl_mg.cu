@@ -1657,6 +1657,9 @@ int kaczmarz_sweeps(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int 
 // measured them faster, unless the launch form is explicit (sweep_kernel) or
 // pinned; per-step calls (amg_kaczmarz) keep kaczmarz_sweeps, whose forms
 // agree bit for bit.  zero: start from x = 0 and r = f (both written).
+// The inner products of the FP64 ring passes go to a->w, the Krylov solver's Dhat z_j: no
+// caller has anything in it while a cycle runs, and it moves only where ensure_workspace
+// drops the captured graphs.
 static bool form_pinned(const wl_amg *a, int l, int prec, int nrhs) {
   for (const KTune &k : a->lev[l].tune)
     if (k.nrhs == nrhs && k.prec == prec && k.us == 0.f) return true;
@@ -1676,7 +1679,7 @@ static int cycle_sweeps(wl_amg *a, int l, int prec, int nrhs, int sweeps, bool z
     for (const KTune &k : L.rowtune)
       if (k.nrhs == nrhs && k.prec == prec) rows = &k;
   if (rows && rows->form == 6 && rows->param == 1)
-    return rings64_sweeps(a, l, rin, xin, L.x.p, L.r.p, nrhs, sweeps, 1, s);
+    return rings64_sweeps(a, l, rin, xin, L.x.p, L.r.p, a->w.p, nrhs, sweeps, 1, s);
   if (zero) {
     size_t vb = prec_bytes(prec) * (size_t)L.n * 2 * nrhs;
     WL_CUDA(cudaMemsetAsync(L.x.p, 0, vb, s));
@@ -1684,7 +1687,7 @@ static int cycle_sweeps(wl_amg *a, int l, int prec, int nrhs, int sweeps, bool z
   }
   if (sweeps <= 0) return WL_OK;
   if (rows && rows->form == 4) return rows_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, sweeps, rows->param, s);
-  if (rows) return rings64_sweeps(a, l, L.r.p, L.x.p, L.x.p, L.r.p, nrhs, sweeps, rows->param, s);
+  if (rows) return rings64_sweeps(a, l, L.r.p, L.x.p, L.x.p, L.r.p, a->w.p, nrhs, sweeps, rows->param, s);
   return kaczmarz_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, sweeps, s);
 }
 
@@ -1749,7 +1752,7 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
       for (int i = 0; i < n; ++i) cand.push_back(KTune{nrhs, prec, 4, prm[i], 0.f});
     }
     if (rings64_ok(a, l, prec, nrhs)) {
-      rc = rings64_prepare(a, l, nrhs, false, s);
+      rc = rings64_prepare(a, l, false, s);
       if (rc && rc != WL_OOM) break;
       for (int q : {0, 1, 2})
         if (!rc && rings64_form(a, l, q, nrhs)) cand.push_back(KTune{nrhs, prec, 6, q, 0.f});
@@ -1757,7 +1760,7 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
     KTune best = cand[0], rows{nrhs, prec, 4, 0, 1e30f};
     float best_us = 1e30f;
     auto sweep = [&](const KTune &c) -> int {
-      return c.form == 6   ? rings64_sweeps(a, l, L.r.p, L.x.p, L.x.p, L.r.p, nrhs, 1, c.param, s)
+      return c.form == 6   ? rings64_sweeps(a, l, L.r.p, L.x.p, L.x.p, L.r.p, a->w.p, nrhs, 1, c.param, s)
              : c.form == 4 ? rows_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c.param, s)
                            : run_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c, s);
     };
@@ -2067,9 +2070,9 @@ static int kaczmarz_entry(wl_amg *a, int level, void *x, void *r, int nrhs, int 
     WL_TRY(wl::rows_sweeps(a, level, prec, sb.b[0].p, sb.b[1].p, nrhs, sweeps, param, s));
   } else if (rings64) {
     WL_TRY(wl::ensure_workspace(a, nrhs, prec));
-    WL_TRY(wl::rings64_prepare(a, level, nrhs, false, s));
+    WL_TRY(wl::rings64_prepare(a, level, false, s));
     if (sweeps > 0)
-      WL_TRY(wl::rings64_sweeps(a, level, sb.b[1].p, sb.b[0].p, sb.b[0].p, sb.b[1].p, nrhs, sweeps, param, s));
+      WL_TRY(wl::rings64_sweeps(a, level, sb.b[1].p, sb.b[0].p, sb.b[0].p, sb.b[1].p, a->w.p, nrhs, sweeps, param, s));
   } else if (rings) {
     WL_TRY(wl::rings_prepare(a, level, prec, s));
     if (sweeps > 0)

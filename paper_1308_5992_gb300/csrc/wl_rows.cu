@@ -1225,9 +1225,8 @@ bool rings64_ok(const wl_amg *a, int l, int prec, int nrhs) {
          !(a->prm.overlap && nrhs >= 16);
 }
 
-int rings64_prepare(wl_amg *a, int l, int nrhs, bool stale, cudaStream_t s) {
+int rings64_prepare(wl_amg *a, int l, bool stale, cudaStream_t s) {
   Level &L = a->lev[l];
-  WL_TRY(L.nums.alloc(sizeof(zd) * (size_t)(L.n / 2) * std::max(nrhs, a->cap)));
   if (L.op64.rows.p && !stale) return WL_OK;
   WL_TRY(L.op64.rows.alloc(sizeof(zd) * (size_t)L.n * 24));
   k_ring64_pack<<<L.n / 4 / RBP_CELLS, 16 * RBP_CELLS, 0, s>>>(L.geo, L.op64.A.as<zd>(), a->prm.omega,
@@ -1321,8 +1320,8 @@ bool rings64_form(const wl_amg *a, int l, int param, int nrhs) {
 // param 0: two launches a pass; 1: one launch of clusters (32 x 32 and 64 x 64); 2:
 // one launch of clusters a pass.
 // rin, xin as in rings_sweeps (param 0 takes r and x themselves)
-int rings64_sweeps(wl_amg *a, int l, const void *rin, const void *xin, void *x, void *r, int nrhs, int sweeps, int param,
-                   cudaStream_t s) {
+int rings64_sweeps(wl_amg *a, int l, const void *rin, const void *xin, void *x, void *r, void *nums, int nrhs, int sweeps,
+                   int param, cudaStream_t s) {
   Level &L = a->lev[l];
   if (param == 1)
     return L.N == 32 ? launch_cluster<32>(L, rin, xin, x, r, nrhs, sweeps, s)
@@ -1336,7 +1335,7 @@ int rings64_sweeps(wl_amg *a, int l, const void *rin, const void *xin, void *x, 
     return WL_OK;
   }
   const zd *A = L.op64.A.as<zd>(), *T = L.op64.rows.as<zd>();
-  double *num = L.nums.as<double>();
+  double *num = (double *)nums;
   const long items = (long)(L.n / 4) * nrhs;
   // lanes a site: as many as leave at most a warp or so per SM partition (a launch
   // of the dots, one right-hand side: 1.6 us on 64 x 64 with H = 4, 2.0 us on 128 x 128

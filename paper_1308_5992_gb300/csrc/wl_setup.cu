@@ -516,14 +516,15 @@ static int galerkin(Setup &S, int l, const zd *A, zd *Ac) {
 }
 
 // the setup's relaxations: the FP64 row-block sweeps (wl_rows.cu), whose
-// triangular inverses follow the level's operator
+// triangular inverses follow the level's operator; tmp2, which holds nothing
+// across a sweep, takes the inner products
 static int setup_sweeps(Setup &S, int l, zd *V, zd *r, int k, int sweeps) {
   wl_amg *a = S.a;
   if (sweeps <= 0) return WL_OK;
   if (!(a->prm.omega > 0.0) || a->lev[l].N < 16) return wl::kaczmarz_sweeps(a, l, WL_FP64, V, r, k, sweeps, S.s);
-  WL_TRY(wl::rings64_prepare(a, l, k, S.stale[l], S.s));
+  WL_TRY(wl::rings64_prepare(a, l, S.stale[l], S.s));
   S.stale[l] = false;
-  return wl::rings64_sweeps(a, l, r, V, V, r, k, sweeps, a->lev[l].N == 32, S.s);
+  return wl::rings64_sweeps(a, l, r, V, V, r, S.S[l].tmp2.p, k, sweeps, a->lev[l].N == 32, S.s);
 }
 
 // Eq. 3.6: Kaczmarz on A_l v = 0
@@ -779,7 +780,7 @@ static int adaptive_step(Setup &S) {
   if (a->prm.omega > 0.0)
     for (int l = 0; l < a->L - 1 && !rc; ++l) {
       if (a->lev[l].N < 16) continue;
-      rc = wl::rings64_prepare(a, l, 1, S.stale[l], S.s);
+      rc = wl::rings64_prepare(a, l, S.stale[l], S.s);
       S.stale[l] = false;
       a->lev[l].rowtune.push_back(KTune{1, WL_FP64, 6, a->lev[l].N == 32, 1.f});
     }
@@ -874,10 +875,7 @@ extern "C" int amg_setup(wl_op *op, const amg_params *params, wl_amg **out) {
   if (!rc) rc = interp_e(S, 0);
   a->prm.kacz_order = prm.kacz_order;
   cudaStreamSynchronize(S.s);
-  for (int l = 0; l < a->L; ++l) {  // made again on first use, from the final operators
-    a->lev[l].op64.rows.release();
-    a->lev[l].nums.release();
-  }
+  for (int l = 0; l < a->L; ++l) a->lev[l].op64.rows.release();  // made again on first use, from the final operators
   if (!rc) rc = wl::hier_finish(a);
   if (S.cs) cusolverDnDestroy(S.cs);
   cudaStreamSynchronize(S.s);

@@ -1,0 +1,67 @@
+"""The library's host side on a stand-in runtime (tests/fake_cudart.c): which buffers its launches
+and captured graphs point to, and what it does when device memory runs out."""
+import pytest
+
+from fakert import run
+
+
+@pytest.mark.parametrize("side,calls", [
+    # the workspace grows through an FP32 cycle
+    (128, "cycle(9, 0) cycle(16, 1) cycle(9, 0) cycle(5, 0) cycle(9, 0)"),
+    # through a solve in two lanes, which takes other sweeps
+    (128, "cycle(5, 0) solve(32) cycle(5, 0) cycle(12, 0) cycle(5, 0) solve(32)"),
+    # through a server that gets the hierarchy after a solve
+    (512, "cycle(1, 0) serve(3) cycle(1, 0) cycle(3, 0)"),
+])
+def test_graphs_keep_their_buffers(side, calls):
+    """One FP64 hierarchy used at changing widths: no launch and no replayed graph points to
+    memory that was freed."""
+    out = run("""
+F = fake()
+F.fake_times(1e4, -1.0)  # each timed candidate beats those before it: the row-block forms win
+h = Hier([%d, %d, 32, 16], overlap=1, fgmres_m=2)
+for c in %r.replace(") ", ");").split(";"):
+    h.ok(eval("h." + c))
+    assert F.fake_dead() == 0, (c, F.fake_dead_what())
+assert "k_ring" in F.fake_captured().decode()
+print("ok")
+""" % (side, side // 4 if side > 256 else 64, calls))
+    assert "ok" in out
+
+
+def test_form6_entry_keeps_graph_buffers():
+    """amg_kaczmarz_form with the FP64 row-block form between two cycles of one width."""
+    out = run("""
+F = fake()
+F.fake_times(1e4, -1.0)
+h = Hier([128, 64, 32, 16])
+h.ok(h.cycle(9, 0))
+h.ok(h.cycle(16, 1))
+h.ok(h.cycle(9, 0))
+h.ok(h.lib.amg_kaczmarz_form(h.amg, 0, h.v, h.v, 12, 1, 0, 6, 0))
+h.ok(h.cycle(9, 0))
+assert F.fake_dead() == 0, F.fake_dead_what()
+print("ok")
+""")
+    assert "ok" in out
+
+
+def test_no_memory_for_the_row_block_forms():
+    """Device memory that runs out while a wider cycle is prepared: the cycles of the widths known
+    before run on buffers that exist."""
+    out = run("""
+F = fake()
+F.fake_times(1e4, -1.0)
+h = Hier([128, 64, 32, 16])
+h.ok(h.cycle(9, 0))
+h.ok(h.cycle(16, 1))
+n = 16 * (128 * 128 // 2 // 2)
+F.fake_fail(n, n * 16, 0, 1)  # what inner products of the ring passes of 1 to 16 would take on level 0
+rc = h.cycle(12, 0)
+F.fake_fail(1, 0, 0, 0)
+assert rc in (0, h.W.WL_OOM), rc
+h.ok(h.cycle(9, 0))
+assert F.fake_dead() == 0, F.fake_dead_what()
+print("ok")
+""")
+    assert "ok" in out
