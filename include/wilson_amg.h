@@ -89,7 +89,9 @@ typedef struct {
                              sweep is timed on each level and the fastest kept; until
                              then, or for per-step calls, a heuristic), 1 = one launch
                              per colour, 2 = one cooperative launch per level visit.
-                             Every form computes the same numbers in the same order. */
+                             All of these compute the same numbers in the same order;
+                             with 0, small levels take row-block forms, rounded
+                             differently (see amg_sweep_form). */
   int kacz_order;         /* Kaczmarz ordering: 0 = 16 colours (a mod 4, b mod 4) over the
                              whole grid; 1 = tile-coloured: 8x8 tiles in (a, b) with four
                              tile colours, the 16 colours inside each tile (grids with
@@ -393,9 +395,10 @@ int wl_time_kernel(wl_amg *amg, int kind, int level, int nrhs, int prec, int rep
  * sweep in microseconds, 0 when the form was not measured (explicit
  * sweep_kernel, or no cycle of that width yet).  Errors: WL_EINVAL.
  * These forms agree bit for bit.  The sweeps of a cycle without a pinned form take the
- * row-block forms instead (the same sweep, rounded differently): FP32 or BF16 on 32x32 and
- * 16x16 levels, and on tile-ordered ones (FP64: on 16-colour ones) where the autotuner measured
- * them faster. */
+ * row-block forms instead (the same sweep, rounded differently), by fixed rules on the level's
+ * size, nrhs and prec: FP32 or BF16 on 32x32 and 16x16 levels, and on small tile-ordered ones
+ * (FP64: 16-colour ones), so that a solve's bits do not depend on measured times.  Where device
+ * memory has no room for their constants, these forms run. */
 int amg_sweep_form(wl_amg *amg, int level, int nrhs, int prec, int *form, int *param, float *us);
 /* Pin the Kaczmarz launch form of `level` (not the coarsest) for `nrhs`
  * right-hand sides in precision `prec` (form and param as in

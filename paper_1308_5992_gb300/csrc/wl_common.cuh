@@ -269,7 +269,7 @@ struct Level {
   // cycle work vectors, [n][2][nrhs_cap] in the cycle precision
   DBuf x, r, f, t;
   std::vector<KTune> tune;    // autotuned sweep forms per (nrhs, precision)
-  std::vector<KTune> rowtune; // where the row-block sweep measured faster: form 4, param = R | RPT << 8
+  std::vector<KTune> rowtune; // row-block sweeps: form 4 with its measured param = R | RPT << 8, or a form set by us = 0
 };
 
 struct wl_amg {
@@ -352,6 +352,7 @@ int rings_sweeps(wl_amg *a, int l, int prec, const void *rin, const void *xin, v
 bool rings64_ok(const wl_amg *a, int l, int prec, int nrhs);
 int rings64_prepare(wl_amg *a, int l, bool stale, cudaStream_t s);  // stale: the operator changed since
 bool rings64_form(const wl_amg *a, int l, int param, int nrhs);
+int rings64_rule(const wl_amg *a, int l, int nrhs);  // the param a cycle takes, or -1: the other forms are faster
 // num: scratch of n / 2 x nrhs complex doubles for a pass's inner products
 int rings64_sweeps(wl_amg *a, int l, const void *rin, const void *xin, void *x, void *r, void *num, int nrhs, int sweeps,
                    int param, cudaStream_t s);

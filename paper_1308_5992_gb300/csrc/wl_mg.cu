@@ -1652,33 +1652,62 @@ int kaczmarz_sweeps(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int 
   return run_sweeps(a, l, prec, x, r, nrhs, sweeps, sweep_form_of(a, l, prec, nrhs), s);
 }
 
-// The sweeps of a cycle: the row-block forms (wl_rows.cu) on 32 x 32 and
-// 16 x 16 levels, and on larger tile-ordered levels where the autotuner
-// measured them faster, unless the launch form is explicit (sweep_kernel) or
-// pinned; per-step calls (amg_kaczmarz) keep kaczmarz_sweeps, whose forms
-// agree bit for bit.  zero: start from x = 0 and r = f (both written).
-// The inner products of the FP64 ring passes go to a->w, the Krylov solver's Dhat z_j: no
-// caller has anything in it while a cycle runs, and it moves only where ensure_workspace
-// drops the captured graphs.
-static bool form_pinned(const wl_amg *a, int l, int prec, int nrhs) {
-  for (const KTune &k : a->lev[l].tune)
-    if (k.nrhs == nrhs && k.prec == prec && k.us == 0.f) return true;
-  return false;
+// The sweeps of a cycle take the row-block forms (wl_rows.cu) by rules on level, width
+// and precision alone (rings_ok, rows_ok, rings64_rule), unless the launch form is
+// explicit (sweep_kernel) or set: those forms are rounded differently from the others
+// and, in FP64, from one another, and what a solve computes must not hang on a timing.
+// The autotuner chooses among forms that agree bit for bit.  Without memory for their
+// constants (ops.rows) the other forms run.  Per-step calls (amg_kaczmarz) keep
+// kaczmarz_sweeps.
+static const KTune *set_form(const std::vector<KTune> &tv, int prec, int nrhs) {
+  for (const KTune &k : tv)
+    if (k.nrhs == nrhs && k.prec == prec && k.us == 0.f) return &k;
+  return nullptr;
 }
-static bool use_rings(const wl_amg *a, int l, int prec, int nrhs) {
-  const LevelOps &o = ops_of(a->lev[l], prec);
-  return a->prm.sweep_kernel == 0 && rings_ok(a, l, prec) && o.rows.p && !form_pinned(a, l, prec, nrhs);
+// the row-block form the rules give (param of form 4: the tuner's, or 0), form -1: none
+static KTune rowblock_rule(const wl_amg *a, int l, int prec, int nrhs) {
+  KTune t{nrhs, prec, -1, 0, 0.f};
+  if (a->prm.sweep_kernel != 0 || set_form(a->lev[l].tune, prec, nrhs)) return t;
+  if (const KTune *k = set_form(a->lev[l].rowtune, prec, nrhs)) return *k;
+  if (rings_ok(a, l, prec)) {
+    t.form = 5;
+  } else if (rows_ok(a, l, prec, nrhs)) {
+    t.form = 4;
+    for (const KTune &k : a->lev[l].rowtune)
+      if (k.nrhs == nrhs && k.prec == prec) t = k;
+  } else if (rings64_ok(a, l, prec, nrhs)) {
+    t.param = rings64_rule(a, l, nrhs);
+    if (t.param >= 0) t.form = 6;
+  }
+  return t;
 }
+// its constants
+static int rowblock_prepare(wl_amg *a, int l, int prec, int form, cudaStream_t s) {
+  return form == 4 ? rows_prepare(a, l, prec, s)
+         : form == 5 ? rings_prepare(a, l, prec, s)
+         : form == 6 ? rings64_prepare(a, l, false, s) : WL_OK;
+}
+// the form of a cycle's sweeps
+static KTune cycle_form(wl_amg *a, int l, int prec, int nrhs) {
+  KTune t = rowblock_rule(a, l, prec, nrhs);
+  if (t.form < 0 || !ops_of(a->lev[l], prec).rows.p) return sweep_form_of(a, l, prec, nrhs);
+  if (t.form == 4 && !t.param) {  // not tuned
+    int prm[8];
+    rows_candidates(nrhs, prm);
+    t.param = prm[0];
+  }
+  return t;
+}
+
+// zero: start from x = 0 and r = f (both written).  The inner products of the FP64 ring
+// passes go to a->w, the Krylov solver's Dhat z_j: no caller has anything in it while a
+// cycle runs, and it moves only where ensure_workspace drops the captured graphs.
 static int cycle_sweeps(wl_amg *a, int l, int prec, int nrhs, int sweeps, bool zero, cudaStream_t s) {
   Level &L = a->lev[l];
   const void *rin = zero ? L.f.p : L.r.p, *xin = zero ? nullptr : L.x.p;  // for the one-launch forms
-  if (sweeps > 0 && use_rings(a, l, prec, nrhs)) return rings_sweeps(a, l, prec, rin, xin, L.x.p, L.r.p, nrhs, sweeps, s);
-  const KTune *rows = nullptr;  // the row-block choice of a tuned level
-  if (sweeps > 0 && a->prm.sweep_kernel == 0 && !form_pinned(a, l, prec, nrhs) &&
-      (rows_ok(a, l, prec, nrhs) || rings64_ok(a, l, prec, nrhs)))
-    for (const KTune &k : L.rowtune)
-      if (k.nrhs == nrhs && k.prec == prec) rows = &k;
-  if (rows && rows->form == 6 && rows->param == 1)
+  const KTune t = cycle_form(a, l, prec, nrhs);
+  if (sweeps > 0 && t.form == 5) return rings_sweeps(a, l, prec, rin, xin, L.x.p, L.r.p, nrhs, sweeps, s);
+  if (sweeps > 0 && t.form == 6 && t.param == 1)
     return rings64_sweeps(a, l, rin, xin, L.x.p, L.r.p, a->w.p, nrhs, sweeps, 1, s);
   if (zero) {
     size_t vb = prec_bytes(prec) * (size_t)L.n * 2 * nrhs;
@@ -1686,16 +1715,17 @@ static int cycle_sweeps(wl_amg *a, int l, int prec, int nrhs, int sweeps, bool z
     WL_CUDA(cudaMemcpyAsync(L.r.p, L.f.p, vb, cudaMemcpyDeviceToDevice, s));
   }
   if (sweeps <= 0) return WL_OK;
-  if (rows && rows->form == 4) return rows_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, sweeps, rows->param, s);
-  if (rows) return rings64_sweeps(a, l, L.r.p, L.x.p, L.x.p, L.r.p, a->w.p, nrhs, sweeps, rows->param, s);
-  return kaczmarz_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, sweeps, s);
+  if (t.form == 4) return rows_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, sweeps, t.param, s);
+  if (t.form == 6) return rings64_sweeps(a, l, L.r.p, L.x.p, L.x.p, L.r.p, a->w.p, nrhs, sweeps, t.param, s);
+  return run_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, sweeps, t, s);
 }
 
 // Autotuner: time every launch form of one sweep on each level (the level's
 // own cycle buffers, whose contents the next cycle overwrites) and keep the
 // fastest.  Candidates: per-colour launches and the cooperative launch at
 // 1, 1/2 and 1/4 of the resident-block limit (colour order); right-hand-side
-// chunks 8, 16, 32 (tile order).  Runs outside stream capture, once per
+// chunks 8, 16, 32 (tile order), and on levels whose cycles take the row-block
+// form 4 its chunks as well.  Runs outside stream capture, once per
 // (nrhs, precision); sweep_kernel != 0 disables it.
 int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
   if (a->prm.sweep_kernel != 0 || nrhs > a->cap) return WL_OK;
@@ -1743,26 +1773,16 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
           if (!dup) cand.push_back(KTune{nrhs, prec, 1, b, 0.f});
         }
     }
-    // the row-block forms' constants are memory the others do without: where there is
-    // no room for them, those forms are left out
-    if (rows_ok(a, l, prec, nrhs)) {
-      rc = rows_prepare(a, l, prec, s);
-      if (rc && rc != WL_OOM) break;
-      int prm[8], n = rc ? 0 : rows_candidates(nrhs, prm);
+    const KTune row = rowblock_rule(a, l, prec, nrhs);
+    if (row.form == 4 && !row.param && ops_of(L, prec).rows.p) {
+      int prm[8], n = rows_candidates(nrhs, prm);
       for (int i = 0; i < n; ++i) cand.push_back(KTune{nrhs, prec, 4, prm[i], 0.f});
-    }
-    if (rings64_ok(a, l, prec, nrhs)) {
-      rc = rings64_prepare(a, l, false, s);
-      if (rc && rc != WL_OOM) break;
-      for (int q : {0, 1, 2})
-        if (!rc && rings64_form(a, l, q, nrhs)) cand.push_back(KTune{nrhs, prec, 6, q, 0.f});
     }
     KTune best = cand[0], rows{nrhs, prec, 4, 0, 1e30f};
     float best_us = 1e30f;
     auto sweep = [&](const KTune &c) -> int {
-      return c.form == 6   ? rings64_sweeps(a, l, L.r.p, L.x.p, L.x.p, L.r.p, a->w.p, nrhs, 1, c.param, s)
-             : c.form == 4 ? rows_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c.param, s)
-                           : run_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c, s);
+      return c.form == 4 ? rows_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c.param, s)
+                         : run_sweeps(a, l, prec, L.x.p, L.r.p, nrhs, 1, c, s);
     };
     for (KTune &c : cand) {
       rc = sweep(c);  // warm-up
@@ -1777,7 +1797,7 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
         break;
       }
       c.us = ms * 1e3f / 3;
-      if (c.form >= 4) {
+      if (c.form == 4) {
         if (c.us < rows.us) rows = c;
       } else if (c.us < best_us) {
         best_us = c.us;
@@ -1786,7 +1806,7 @@ int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s) {
     }
     if (rc == WL_OK) {
       L.tune.push_back(best);
-      if (rows.us < best_us) L.rowtune.push_back(rows);
+      if (rows.param) L.rowtune.push_back(rows);
     }
   }
   cudaEventDestroy(e0);
@@ -1947,12 +1967,11 @@ int cycle_prepare(wl_amg *a, int nrhs, int prec, cudaStream_t s, const wl_amg::G
       if (out) *out = &g;
       return WL_OK;
     }
+  for (int l = 0; l < a->L - 1; ++l) {
+    int rc = rowblock_prepare(a, l, prec, rowblock_rule(a, l, prec, nrhs).form, s);
+    if (rc && rc != WL_OOM) return rc;  // no room: cycle_form sees no constants
+  }
   WL_TRY(autotune_sweeps(a, nrhs, prec, s));  // measured launch forms, before the capture
-  for (int l = 0; l < a->L - 1; ++l)
-    if (a->prm.sweep_kernel == 0 && rings_ok(a, l, prec)) {
-      int rc = rings_prepare(a, l, prec, s);
-      if (rc && rc != WL_OOM) return rc;  // no room: use_rings sees no constants
-    }
   cudaGraph_t graph;
   long long before = wl_launch_count();
   WL_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));

@@ -1110,20 +1110,23 @@ int rows_candidates(int nrhs, int *out) {
   return n;
 }
 
-// Which sweeps may take the row-block form.  Two concurrent lanes fill the GPU
+// Which sweeps take the row-block form.  Two concurrent lanes fill the GPU
 // between them, so there the work of a sweep counts and not its latency: with
 // the row form (about twice the instructions of k_kacz_tile, a third of its
 // dependent steps) on level 1 the 512x512 step of 64 right-hand sides took
 // 145.0 ms instead of 143.7, although that level's sweep alone takes 21
 // instead of 41.7 us.
 bool rows_ok(const wl_amg *a, int l, int prec, int nrhs) {
-  // A launch relaxes a quarter of the level's tiles for every right-hand side.
-  // Measured per sweep, row form against the best other one: 512x512 (512 tiles
-  // a launch) 16 against 58 us for 1 right-hand side, 34 against 46 us for 4,
-  // 52 against 54 us for 5; 256x256 (128 tiles) 57 against 70 us for 16;
-  // 128x128 (32 tiles) 11 against 41.7 us for 1, 20 against 41.7 us for 32.
+  // A launch relaxes a quarter of the level's tiles for every right-hand side.  The
+  // lines lie where a sweep takes as long as the best tile kernel's.  Tiles x
+  // right-hand sides, us a sweep, row form against tile kernel, FP32 (BF16): up to 4
+  // right-hand sides, 1024x1024 x 1 = 2048: 71 / 139.5 (59 / 148), 512x512 x 4 = 2048:
+  // 35.0 / 46.9 (32.9 / 43.1).  More of them, whose tile kernel has fewer idle lanes:
+  // 128x128 x 32 = 1024: 25.1 / 32.9 (24.7 / 37.0), 256x256 x 9 = 1152: 32.4 / 37.0
+  // (31.3 / 37.0), x 12 = 1536: 32.9 / 32.9 (32.9 / 37.2), 128x128 x 48 = 1536: 37.0 / 32.9
+  // (35.8 / 37.1), 256x256 x 16 = 2048: 37.0 / 32.9 (36.6 / 37.1).
   const Level &L = a->lev[l];
-  if ((long)L.n / 256 * nrhs > 2048) return false;
+  if ((long)L.n / 256 * nrhs > (nrhs <= 4 ? 2048 : prec == WL_FP32_BF16 ? 1536 : 1280)) return false;
   return !a->is_twin && !(a->prm.overlap && nrhs >= 16) && prec != WL_FP64 && a->prm.kacz_order == 1 && l < a->L - 1 && L.N >= 64 && L.N % (4 * RB_KT) == 0 &&
          a->prm.omega > 0.0;
 }
@@ -1315,6 +1318,28 @@ static int launch_ring_pass(const Level &L, int pass, void *x, void *r, int nrhs
 bool rings64_form(const wl_amg *a, int l, int param, int nrhs) {
   const int N = a->lev[l].N;
   return param == 0 || (param == 1 && (N == 32 || N == 64)) || (param == 2 && N >= 32 && N <= 256 && nrhs <= 4);
+}
+
+// The form of a cycle's sweeps, by level and width alone, since the forms round
+// differently.  us a sweep (params 0 / 1 / 2 / the best of the other forms):
+//   32x32:   1: 21.7 / 18.7 / 16.5 / 78, 4: 25.7 / 18.5 / 16.5 / 191, 5: 27.6 / 18.7 / - / 193,
+//            32: 36.0 / 28.9 / - / 193, 48: 48.3 / 59.6 / - / 193
+//   64x64:   1: 21.7 / 26.8 / 16.5 / 78, 4: 27.5 / 27.0 / 18.7 / 211, 6: 34.0 / 27.0 / - / 211,
+//            8: 35.9 / 51.6 / - / 213, 64: 125 / 249 / - / 211
+//   128x128: 1: 25.7 / - / 22.7 / 78, 2: 29.9 / - / 35.1 / 228, 24: 174 / - / - / 211
+//   256x256: 1: 57 / - / 71 / 192, 4: 126 / - / 244 / 216, 5: 189 / - / - / 220
+// and one right-hand side of 512x512 146 / 623, of 1024x1024 492 / 2195.  Param 0 works on
+// chunks of 4; it meets the cooperative launch at 2^18 site-vectors (128x128 x 32: 212 / 212,
+// 256x256 x 8: 213 / 213), and where that launch needs a second block on an SM (152 blocks of
+// 2048 site-vectors) again at 3 * 2^17 (128x128 x 48: 308 / 371, 256x256 x 12: 308 / 374,
+// x 9: 284 / 219, x 16: 401 / 373).
+int rings64_rule(const wl_amg *a, int l, int nrhs) {
+  const int N = a->lev[l].N;
+  const long n = a->lev[l].n, padded = n * ((nrhs + 3) / 4 * 4);
+  if (rings64_form(a, l, 2, nrhs) && (N <= 64 || (N == 128 && nrhs == 1))) return 2;
+  if (rings64_form(a, l, 1, nrhs) && nrhs <= (N == 32 ? 32 : 6)) return 1;
+  if (nrhs == 1 || padded <= 1L << 18 || (n * nrhs > 152L * 2048 && padded <= 3L << 17)) return 0;
+  return -1;
 }
 
 // param 0: two launches a pass; 1: one launch of clusters (32 x 32 and 64 x 64); 2:

@@ -782,7 +782,7 @@ static int adaptive_step(Setup &S) {
       if (a->lev[l].N < 16) continue;
       rc = wl::rings64_prepare(a, l, S.stale[l], S.s);
       S.stale[l] = false;
-      a->lev[l].rowtune.push_back(KTune{1, WL_FP64, 6, a->lev[l].N == 32, 1.f});
+      a->lev[l].rowtune.push_back(KTune{1, WL_FP64, 6, a->lev[l].N == 32, 0.f});
     }
   for (int it = 0; it < 2 && !rc; ++it) {
     k_get_col<<<WL_GRID(n2, 256), 256, 0, S.s>>>(Vb, S.S[0].tmp2.as<zd>(), n2, kb, qb, 1.0);

@@ -45,3 +45,31 @@ def test_cycles_at_changing_widths(c2):
         x = cycle(amg, f[:nrhs].contiguous(), prec)
         assert torch.equal(x, first.setdefault((nrhs, prec), x)), (nrhs, prec)
     amg.close()
+
+
+@pytest.mark.parametrize("prec", [W.WL_FP32, W.WL_FP32_BF16])
+@pytest.mark.parametrize("nrhs", [1, 3, 11])
+def test_row_block_chunks_agree_bitwise(c2, prec, nrhs):
+    """The tuner may choose any chunk of the row-block form: a right-hand side's numbers do not
+    depend on it."""
+    amg = setup(c2, kacz_order=1, precision=prec)
+    n = amg.n(0)
+    x0, r0 = (np.stack([cgauss(s, r, n) for r in range(nrhs)]).astype(np.complex64).astype(complex) for s in (710, 720))
+    outs = []
+    for param in (1 | 1 << 8, 2 | 1 << 8, 4 | 1 << 8, 8 | 1 << 8, 8 | 2 << 8):
+        x, r = T(x0), T(r0)
+        W.amg_kaczmarz_form(amg, 0, x, r, nrhs, 2, prec, 4, param)
+        outs.append((x, r))
+        assert torch.equal(x, outs[0][0]) and torch.equal(r, outs[0][1]), param
+    amg.close()
+
+
+@pytest.mark.parametrize("prec,order", [(W.WL_FP64, 0), (W.WL_FP64, 1), (W.WL_FP32, 1), (W.WL_FP32_BF16, 1)])
+def test_two_hierarchies_agree_bitwise(c2, prec, order):
+    """The same cycle of two hierarchies, each tuned on its own, gives the same bits."""
+    a, b = (setup(c2, kacz_order=order, precision=prec) for _ in range(2))
+    f = T(np.stack([cgauss(730, r, a.n(0)) for r in range(6)]))
+    for nrhs in (1, 2, 6):
+        assert torch.equal(cycle(a, f[:nrhs].contiguous(), prec), cycle(b, f[:nrhs].contiguous(), prec)), nrhs
+    a.close()
+    b.close()

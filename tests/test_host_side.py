@@ -65,3 +65,30 @@ assert F.fake_dead() == 0, F.fake_dead_what()
 print("ok")
 """)
     assert "ok" in out
+
+
+@pytest.mark.parametrize("order,prec,sides", [
+    (0, 0, [256, 128, 64, 32, 16]), (0, 1, [128, 64, 32, 16, 8]), (1, 0, [128, 64, 32, 16]),
+    (1, 1, [256, 128, 64, 32, 16]), (1, 2, [128, 64, 32, 16])])
+def test_what_a_cycle_computes_does_not_hang_on_timings(order, prec, sides):
+    """Whatever the tuner measures, the kernels that a cycle captures are the same but for those
+    that agree bit for bit: one family of forms 0 to 3, and k_kacz_rows with any chunks."""
+    out = run("""
+F = fake()
+def captured(start, step, nrhs):
+    F.fake_times(start, step)
+    h = Hier(%r, kacz_order=%d, precision=%d, fgmres_m=1)
+    h.ok(h.cycle(nrhs, %d))
+    out = []
+    for n in F.fake_captured().decode().split():
+        old = "k_kacz" in n and "k_kacz_r" not in n
+        k = "old" if old else "k_kacz_rows" if "k_kacz_rows" in n else n
+        if k != "old" or not out or out[-1] != k:  # a sweep of forms 0 to 3 is one to 64 launches
+            out.append(k)
+    return out
+for nrhs in (1, 2, 5, 9, 16, 30):
+    a, b = captured(1.0, 1.0, nrhs), captured(1e4, -1.0, nrhs)
+    assert a == b, (nrhs, set(a) ^ set(b))
+print("ok")
+""" % (sides, order, prec, prec))
+    assert "ok" in out
