@@ -541,7 +541,7 @@ def run_gb300(args, rank, world, local_rank):
         "plain_fp64_single_rhs": {"value": round(1e3 / (sorted(p64)[1]), 3), "unit": "solves/s",
                                   "ms": sorted(p64)[1], "iters": inf64[0]["iters"]},
         "e2e": e2e, "gpu_launches": int(launches), "roofline": roof, "roofline_more": roof_more, "clocks": clk,
-        "sweep_forms": [list(W.amg_sweep_form(amg, l, lane, prec)) for l in range(len(w["blocks"]))],
+        "sweep_forms": [list(W.amg_cycle_form(amg, l, lane, prec)) for l in range(len(w["blocks"]))],
     }
     # The other single-configuration workloads, beside the headline: C3 (this lattice, one
     # right-hand side, the same FP32 cycle on the same hierarchy) and C2 (128x128, the plain

@@ -382,8 +382,8 @@ enum {
  * hierarchy's own work buffers (their contents are not preserved).
  * Errors: WL_EINVAL. */
 int wl_time_kernel(wl_amg *amg, int kind, int level, int nrhs, int prec, int reps, double *avg_ms);
-/* Kaczmarz launch form used on `level` (not the coarsest) for `nrhs`
- * right-hand sides in precision `prec`: form 0 = one launch per colour,
+/* Kaczmarz launch form of per-step sweeps (amg_kaczmarz) on `level` (not the coarsest) for `nrhs`
+ * right-hand sides in precision `prec`, and of a cycle's where amg_cycle_form says so: form 0 = one launch per colour,
  * 1 = cooperative launch with *param blocks, 2 = tile-coloured kernel with
  * right-hand-side chunk (*param & 255) and right-hand sides per thread
  * ((*param >> 8) & 15: 1 or 2; 8 = one per thread with paired FP32 FMAs);
@@ -400,22 +400,27 @@ int wl_time_kernel(wl_amg *amg, int kind, int level, int nrhs, int prec, int rep
  * (FP64: 16-colour ones), so that a solve's bits do not depend on measured times.  Where device
  * memory has no room for their constants, these forms run. */
 int amg_sweep_form(wl_amg *amg, int level, int nrhs, int prec, int *form, int *param, float *us);
+/* The form that the sweeps of a cycle take on `level` once a cycle of that width has run: as
+ * amg_sweep_form, or a row-block form, 4 to 6 as in amg_kaczmarz_form (*us = 0 for 5 and 6,
+ * which follow from a rule).  Errors: WL_EINVAL. */
+int amg_cycle_form(wl_amg *amg, int level, int nrhs, int prec, int *form, int *param, float *us);
 /* Pin the Kaczmarz launch form of `level` (not the coarsest) for `nrhs`
  * right-hand sides in precision `prec` (form and param as in
- * amg_sweep_form; the form must belong to the hierarchy's ordering on that
+ * amg_sweep_form or amg_cycle_form; the form must belong to the hierarchy's ordering on that
  * level).  The autotuner then keeps it, so a cycle of that width captured
  * afterwards uses it; graphs captured earlier are not changed.  For
  * reproducible measurements (a profiler slows every launch, so the tuner's
  * timings under it do not hold).  Ignored while sweep_kernel != 0.  Not
- * thread-safe against solves on the same hierarchy.  Errors: WL_EINVAL. */
+ * thread-safe against solves on the same hierarchy.  Errors: WL_EINVAL; WL_OOM (no memory for a
+ * row-block form's constants). */
 int amg_pin_sweep_form(wl_amg *amg, int level, int nrhs, int prec, int form, int param);
 /* amg_kaczmarz with an explicit launch form (form and param as reported by
  * amg_sweep_form; the form must belong to the hierarchy's ordering on that
- * level), for tests and measurements: every form of one ordering computes
- * the same numbers.  Form 4 (tile ordering, FP32 or BF16, param = R | RPT << 8: right-hand
- * sides per block and per warp, one of (1, 1), (2, 1), (4, 1), (8, 1), (8, 2)) is the
- * row-block form of the cycle; form 5 (32x32 and 16x16 levels, FP32 or BF16, param 0) its
- * one-launch form there; form 6 (16-colour ordering, FP64) those of FP64 cycles: param 0 two
+ * level), for tests and measurements: forms 0 to 3 of one ordering compute
+ * the same numbers.  The row-block forms of a cycle's sweeps round differently.  Form 4 (tile ordering, FP32 or BF16, param = R | RPT << 8: right-hand
+ * sides per block and per warp, one of (1, 1), (2, 1), (4, 1), (8, 1), (8, 2), which agree bit
+ * for bit) is that of tile-ordered levels; form 5 (32x32 and 16x16 levels, FP32 or BF16, param 0)
+ * one launch for all sweeps; form 6 (16-colour ordering, FP64) those of FP64 cycles: param 0 two
  * launches a pass, 1 (32x32 and 64x64 levels) one launch of clusters, 2 (levels 32 to 256, up
  * to 4 right-hand sides) one launch a pass.  Errors: WL_EINVAL (no such form). */
 int amg_kaczmarz_form(wl_amg *amg, int level, void *x, void *r, int nrhs, int sweeps, int prec, int form, int param);

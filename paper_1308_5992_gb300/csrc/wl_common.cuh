@@ -357,6 +357,7 @@ int rings64_rule(const wl_amg *a, int l, int nrhs);  // the param a cycle takes,
 int rings64_sweeps(wl_amg *a, int l, const void *rin, const void *xin, void *x, void *r, void *num, int nrhs, int sweeps,
                    int param, cudaStream_t s);
 KTune sweep_form_of(wl_amg *a, int l, int prec, int nrhs);
+void unset_forms(Level &L, int prec, int nrhs);  // those pinned (us = 0)
 int restrict_op(wl_amg *a, int l, int prec, const void *r, void *fc, int nrhs, cudaStream_t s);
 int prolong_op(wl_amg *a, int l, int prec, const void *e, void *x, int nrhs, cudaStream_t s);
 int coarsest_apply(wl_amg *a, int prec, const void *f, void *x, int nrhs, cudaStream_t s);

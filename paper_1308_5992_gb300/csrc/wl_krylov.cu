@@ -1222,6 +1222,9 @@ static int run_two_lanes(wl_amg *a, int nb, wl_info *info, Lane lane) {
   if (!t_has_graph)
     for (int l = 0; l < a->L; ++l) {
       std::vector<KTune> &tv = t->lev[l].tune;
+      wl::unset_forms(t->lev[l], prec, h1);
+      for (const KTune &k : a->lev[l].rowtune)
+        if (k.nrhs == h1 && k.prec == prec && k.us == 0.f) t->lev[l].rowtune.push_back(k);
       for (const KTune &k : a->lev[l].tune) {
         if (k.nrhs != h1 || k.prec != prec) continue;
         bool set = false;

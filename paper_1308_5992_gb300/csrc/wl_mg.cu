@@ -1664,6 +1664,13 @@ static const KTune *set_form(const std::vector<KTune> &tv, int prec, int nrhs) {
     if (k.nrhs == nrhs && k.prec == prec && k.us == 0.f) return &k;
   return nullptr;
 }
+// drop the forms set for (nrhs, prec): the tuner and the rules choose again
+void unset_forms(Level &L, int prec, int nrhs) {
+  for (std::vector<KTune> *tv : {&L.tune, &L.rowtune})
+    tv->erase(std::remove_if(tv->begin(), tv->end(),
+                             [=](const KTune &k) { return k.nrhs == nrhs && k.prec == prec && k.us == 0.f; }),
+              tv->end());
+}
 // the row-block form the rules give (param of form 4: the tuner's, or 0), form -1: none
 static KTune rowblock_rule(const wl_amg *a, int l, int prec, int nrhs) {
   KTune t{nrhs, prec, -1, 0, 0.f};
@@ -2058,6 +2065,13 @@ static bool form_exists(const wl_amg *a, int level, int nrhs, int prec, int form
                  (form == 3 && nrhs > 1 && wl::block_fits(L, param, prec)));
 }
 
+// the same for the row-block forms
+static bool rowblock_exists(const wl_amg *a, int level, int nrhs, int prec, int form, int param) {
+  return form == 4   ? wl::rows_form_exists(a, level, prec, param)
+         : form == 5 ? param == 0 && wl::rings_ok(a, level, prec)
+                     : form == 6 && wl::rings64_ok(a, level, prec, 1) && wl::rings64_form(a, level, param, nrhs);
+}
+
 // form < 0: the solver's own choice; else an explicit launch form (KTune)
 static int kaczmarz_entry(wl_amg *a, int level, void *x, void *r, int nrhs, int sweeps, int prec, int form,
                           int param, const char *who) {
@@ -2066,10 +2080,8 @@ static int kaczmarz_entry(wl_amg *a, int level, void *x, void *r, int nrhs, int 
     wl_set_error("%s: invalid argument (the coarsest level is not relaxed)", who);
     return WL_EINVAL;
   }
-  const bool rings = form == 5 && param == 0 && wl::rings_ok(a, level, prec);
-  const bool rings64 = form == 6 && wl::rings64_ok(a, level, prec, 1) && wl::rings64_form(a, level, param, nrhs);
-  const bool rows = form == 4 && level < a->L - 1 && wl::rows_form_exists(a, level, prec, param);
-  if (form >= 0 && !rows && !rings && !rings64 && !form_exists(a, level, nrhs, prec, form, param)) {
+  const bool row = rowblock_exists(a, level, nrhs, prec, form, param);
+  if (form >= 0 && !row && !form_exists(a, level, nrhs, prec, form, param)) {
     wl_set_error("%s: launch form %d / %d does not exist for this level and ordering", who, form, param);
     return WL_EINVAL;
   }
@@ -2084,18 +2096,14 @@ static int kaczmarz_entry(wl_amg *a, int level, void *x, void *r, int nrhs, int 
   WL_TRY(wl::to_internal((const zd *)r, sb.b[1].p, n2, nrhs, pin, s));
   if (form < 0) {
     WL_TRY(wl::kaczmarz_sweeps(a, level, prec, sb.b[0].p, sb.b[1].p, nrhs, sweeps, s));
-  } else if (rows) {
-    WL_TRY(wl::rows_prepare(a, level, prec, s));
-    WL_TRY(wl::rows_sweeps(a, level, prec, sb.b[0].p, sb.b[1].p, nrhs, sweeps, param, s));
-  } else if (rings64) {
-    WL_TRY(wl::ensure_workspace(a, nrhs, prec));
-    WL_TRY(wl::rings64_prepare(a, level, false, s));
+  } else if (row) {
+    if (form == 6) WL_TRY(wl::ensure_workspace(a, nrhs, prec));  // a->w
+    WL_TRY(wl::rowblock_prepare(a, level, prec, form, s));
+    void *xi = sb.b[0].p, *ri = sb.b[1].p;
     if (sweeps > 0)
-      WL_TRY(wl::rings64_sweeps(a, level, sb.b[1].p, sb.b[0].p, sb.b[0].p, sb.b[1].p, a->w.p, nrhs, sweeps, param, s));
-  } else if (rings) {
-    WL_TRY(wl::rings_prepare(a, level, prec, s));
-    if (sweeps > 0)
-      WL_TRY(wl::rings_sweeps(a, level, prec, sb.b[1].p, sb.b[0].p, sb.b[0].p, sb.b[1].p, nrhs, sweeps, s));
+      WL_TRY(form == 4   ? wl::rows_sweeps(a, level, prec, xi, ri, nrhs, sweeps, param, s)
+             : form == 5 ? wl::rings_sweeps(a, level, prec, ri, xi, xi, ri, nrhs, sweeps, s)
+                         : wl::rings64_sweeps(a, level, ri, xi, xi, ri, a->w.p, nrhs, sweeps, param, s));
   } else if (sweeps > 0) {
     KTune t{nrhs, prec, form, param, 0.f};
     WL_TRY(wl::run_sweeps(a, level, prec, sb.b[0].p, sb.b[1].p, nrhs, sweeps, t, s));
@@ -2185,11 +2193,15 @@ extern "C" int amg_cycle(wl_amg *a, const void *f, void *x, int nrhs, int prec) 
 
 extern "C" int amg_pin_sweep_form(wl_amg *a, int level, int nrhs, int prec, int form, int param) {
   WL_TRY(check_amg(a, level, nrhs, prec, "amg_pin_sweep_form"));
-  if (level == a->L - 1 || !form_exists(a, level, nrhs, prec, form, param)) {
+  const bool row = rowblock_exists(a, level, nrhs, prec, form, param);
+  if (level == a->L - 1 || (!row && !form_exists(a, level, nrhs, prec, form, param))) {
     wl_set_error("amg_pin_sweep_form: launch form %d / %d does not exist for this level and ordering", form, param);
     return WL_EINVAL;
   }
-  std::vector<KTune> &tv = a->lev[level].tune;
+  if (row) WL_TRY(wl::rowblock_prepare(a, level, prec, form, a->op->stream));
+  Level &L = a->lev[level];
+  wl::unset_forms(L, prec, nrhs);
+  std::vector<KTune> &tv = row ? L.rowtune : L.tune;
   for (KTune &k : tv)
     if (k.nrhs == nrhs && k.prec == prec) {
       k = KTune{nrhs, prec, form, param, 0.f};
@@ -2199,15 +2211,24 @@ extern "C" int amg_pin_sweep_form(wl_amg *a, int level, int nrhs, int prec, int 
   return WL_OK;
 }
 
-extern "C" int amg_sweep_form(wl_amg *a, int level, int nrhs, int prec, int *form, int *param, float *us) {
+static int form_query(wl_amg *a, int level, int nrhs, int prec, int *form, int *param, float *us, bool cycle,
+                      const char *who) {
   if (!a || !form || !param || !us || level < 0 || level >= a->L - 1 || nrhs < 1 ||
       (prec != WL_FP64 && prec != WL_FP32 && prec != WL_FP32_BF16)) {
-    wl_set_error("amg_sweep_form: invalid argument");
+    wl_set_error("%s: invalid argument", who);
     return WL_EINVAL;
   }
-  KTune t = wl::sweep_form_of(a, level, prec, nrhs);
+  KTune t = cycle ? wl::cycle_form(a, level, prec, nrhs) : wl::sweep_form_of(a, level, prec, nrhs);
   *form = t.form;
   *param = t.param;
   *us = t.us;
   return WL_OK;
+}
+
+extern "C" int amg_sweep_form(wl_amg *a, int level, int nrhs, int prec, int *form, int *param, float *us) {
+  return form_query(a, level, nrhs, prec, form, param, us, false, "amg_sweep_form");
+}
+
+extern "C" int amg_cycle_form(wl_amg *a, int level, int nrhs, int prec, int *form, int *param, float *us) {
+  return form_query(a, level, nrhs, prec, form, param, us, true, "amg_cycle_form");
 }

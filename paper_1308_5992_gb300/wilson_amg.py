@@ -91,6 +91,7 @@ def lib():
             "amg_fgmres": (i, [P, P, P, i, d, C.POINTER(wl_info)]),
             "amg_rho": (i, [P, P, P, i, d, i, P, P, P]),
             "amg_sweep_form": (i, [P, i, i, i, P, P, P]),
+            "amg_cycle_form": (i, [P, i, i, i, P, P, P]),
             "amg_pin_sweep_form": (i, [P, i, i, i, i, i]),
             "amg_kaczmarz_form": (i, [P, i, P, P, i, i, i, i, i]),
             "wl_last_error": (C.c_char_p, []),
@@ -393,13 +394,23 @@ def amg_pin_sweep_form(amg, level, nrhs, prec, form, param):
 
 
 def amg_sweep_form(amg, level, nrhs, prec):
-    """(form, param, us) of the Kaczmarz sweep on `level`: form 0 per-colour
+    """(form, param, us) of per-step sweeps (amg_kaczmarz) on `level`: form 0 per-colour
     launches, 1 cooperative (param blocks), 2 tile kernel (param = RHS chunk | RHS per thread << 8,
     8 meaning one RHS per thread with paired FP32 FMAs), 3 block-resident (param RHS per block);
     us = measured time of one sweep (0 if not measured)."""
     f, p, u = C.c_int(), C.c_int(), C.c_float()
     _chk(lib().amg_sweep_form(amg.handle, level, nrhs, prec, C.byref(f), C.byref(p), C.byref(u)),
          "amg_sweep_form")
+    return f.value, p.value, u.value
+
+
+def amg_cycle_form(amg, level, nrhs, prec):
+    """(form, param, us) of a cycle's sweeps on `level`, once a cycle of that width has run: as
+    amg_sweep_form, or a row-block form: 4 (param = RHS per block | RHS per warp << 8), 5, or 6
+    (param 0 two launches a pass, 1 one launch of clusters, 2 one launch a pass)."""
+    f, p, u = C.c_int(), C.c_int(), C.c_float()
+    _chk(lib().amg_cycle_form(amg.handle, level, nrhs, prec, C.byref(f), C.byref(p), C.byref(u)),
+         "amg_cycle_form")
     return f.value, p.value, u.value
 
 

@@ -73,3 +73,24 @@ def test_two_hierarchies_agree_bitwise(c2, prec, order):
         assert torch.equal(cycle(a, f[:nrhs].contiguous(), prec), cycle(b, f[:nrhs].contiguous(), prec)), nrhs
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("prec,order", [(W.WL_FP64, 0), (W.WL_FP32, 1)])
+def test_pinned_cycle_forms_give_the_same_bits(c2, prec, order):
+    """The forms that amg_cycle_form reports, pinned on another hierarchy, give the same bits; in
+    FP64 every row-block form gives the cycle to rounding (1e-12, as the other cycles)."""
+    a, b = (setup(c2, kacz_order=order, precision=prec) for _ in range(2))
+    f = T(np.stack([cgauss(740, r, a.n(0)) for r in range(2)]))
+    x = cycle(a, f, prec)
+    L = len(c2[0]["blocks"])
+    for l in range(L):
+        W.amg_pin_sweep_form(b, l, 2, prec, *W.amg_cycle_form(a, l, 2, prec)[:2])
+    assert torch.equal(cycle(b, f, prec), x)
+    b.close()
+    if prec == W.WL_FP64:
+        for param in (0, 2):
+            c = setup(c2)
+            W.amg_pin_sweep_form(c, 0, 2, prec, 6, param)
+            assert float((cycle(c, f, prec) - x).abs().max() / x.abs().max()) <= 1e-12, param
+            c.close()
+    a.close()

@@ -92,3 +92,66 @@ for nrhs in (1, 2, 5, 9, 16, 30):
 print("ok")
 """ % (sides, order, prec, prec))
     assert "ok" in out
+
+
+@pytest.mark.parametrize("order,prec,sides", [(0, 0, [256, 128, 64, 32, 16]), (1, 1, [256, 128, 64, 32, 16, 8]),
+                                              (0, 2, [64, 32, 16])])
+def test_cycle_forms_are_reported_and_pinned(order, prec, sides):
+    """amg_cycle_form names what the cycle's graph holds; those forms, pinned on a second hierarchy
+    whose tuner would choose otherwise, give the same kernels; a pinned form of the other kind
+    takes their place."""
+    out = run("""
+F = fake()
+sides, prec = %r, %d
+def hier():
+    return Hier(sides, kacz_order=%d, precision=prec, fgmres_m=1)
+def form(h, l, nrhs):
+    f, p, u = C.c_int(), C.c_int(), C.c_float()
+    h.ok(h.lib.amg_cycle_form(h.amg, l, nrhs, prec, C.byref(f), C.byref(p), C.byref(u)))
+    return f.value, p.value
+def captured(h, nrhs):
+    h.ok(h.cycle(nrhs, prec))
+    return F.fake_captured().decode().split()
+KERNEL = {0: "k_kacz", 1: "k_kacz_coop", 2: "k_kacz_tile", 3: "k_kacz_block", 4: "k_kacz_rows", 5: "k_kacz_rings"}
+for nrhs in (1, 3, 9, 12):
+    F.fake_times(1.0, 1.0)
+    a = hier()
+    names = captured(a, nrhs)
+    forms = [form(a, l, nrhs) for l in range(len(sides) - 1)]
+    for l, (f, p) in enumerate(forms):
+        k = KERNEL[f] if f < 6 else ("k_ring_dots", "k_ring64_cluster", "k_ring_pass")[p]
+        assert any(k in n for n in names), (l, f, p, names)
+    assert ("k_ring_" in " ".join(names)) == any(f == 6 and p != 1 for f, p in forms)
+    F.fake_times(1e4, -1.0)  # the last candidate wins
+    b = hier()
+    for l, (f, p) in enumerate(forms):
+        b.ok(b.lib.amg_pin_sweep_form(b.amg, l, nrhs, prec, f, p))
+    assert captured(b, nrhs) == names and [form(b, l, nrhs) for l in range(len(sides) - 1)] == forms
+    c = hier()  # a row-block form pinned, then an old one: the old one runs
+    for l, (f, p) in enumerate(forms):
+        if f >= 4:
+            old = (2, 8) if f == 4 else (0, 0)
+            c.ok(c.lib.amg_pin_sweep_form(c.amg, l, nrhs, prec, f, p))
+            c.ok(c.lib.amg_pin_sweep_form(c.amg, l, nrhs, prec, *old))
+    assert not any("k_ring" in n or "k_kacz_r" in n for n in captured(c, nrhs))
+    for f, p in ((4, 3 | 1 << 8), (5, 1), (6, 3), (7, 0), (6 if prec else 5, 0)):
+        assert c.lib.amg_pin_sweep_form(c.amg, 0, nrhs, prec, f, p) == c.W.WL_EINVAL, (f, p)
+print("ok")
+""" % (sides, prec, order))
+    assert "ok" in out
+
+
+def test_two_lanes_take_a_pinned_row_block_form():
+    """A form pinned for the lanes' width is the second lane's too, with constants of its own."""
+    out = run("""
+F = fake()
+h = Hier([128, 64, 32, 16], overlap=1, fgmres_m=1)
+h.ok(h.lib.amg_pin_sweep_form(h.amg, 0, 16, 0, 6, 0))
+h.ok(h.solve(32))
+assert "k_ring_dots" in F.fake_captured().decode()  # the second lane's graph is captured last
+h.ok(h.lib.amg_pin_sweep_form(h.amg, 0, 17, 0, 0, 0))
+h.ok(h.solve(34))
+assert "k_ring_dots" not in F.fake_captured().decode() and F.fake_dead() == 0
+print("ok")
+""")
+    assert "ok" in out
