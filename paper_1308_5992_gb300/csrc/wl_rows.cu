@@ -1315,9 +1315,53 @@ static int launch_ring_pass(const Level &L, int pass, void *x, void *r, int nrhs
   return WL_OK;
 }
 
+// Does the current device (a partition of one, perhaps) hold a cluster of this kernel?
+// Asked once per device; raises the kernel's limits on the way.
+static bool cluster_fits(const void *fn, int blocks, int nt, size_t smem, std::atomic<unsigned long long> *known) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (!(known[0].load(std::memory_order_acquire) & bit)) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(nt);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = blocks;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if ((!smem || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) &&
+        (blocks <= 8 || cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+        cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n > 0)
+      known[1].fetch_or(bit, std::memory_order_acq_rel);
+    else
+      cudaGetLastError();
+    known[0].fetch_or(bit, std::memory_order_acq_rel);
+  }
+  return (known[1].load(std::memory_order_acquire) & bit) != 0;
+}
+template <int N>
+static bool ring_cluster_fits() {
+  static std::atomic<unsigned long long> known[2];
+  return cluster_fits((const void *)k_ring64_cluster<N>, 16, RingCluster<N>::NT, sizeof(RingCluster<N>), known);
+}
+template <int W, int BLOCKS>
+static bool ring_pass_fits() {
+  static std::atomic<unsigned long long> known[2];
+  return cluster_fits((const void *)k_ring_pass<W>, BLOCKS, RingPass<W>::NT, 0, known);
+}
+
 bool rings64_form(const wl_amg *a, int l, int param, int nrhs) {
   const int N = a->lev[l].N;
-  return param == 0 || (param == 1 && (N == 32 || N == 64)) || (param == 2 && N >= 32 && N <= 256 && nrhs <= 4);
+  if (param == 1) return N == 32 ? ring_cluster_fits<32>() : N == 64 && ring_cluster_fits<64>();
+  if (param == 2 && nrhs <= 4)
+    return N == 32 ? ring_pass_fits<8, 4>() : N == 64 ? ring_pass_fits<8, 8>()
+         : N == 128 ? ring_pass_fits<8, 16>() : N == 256 && ring_pass_fits<16, 16>();
+  return param == 0;
 }
 
 // The form of a cycle's sweeps, by level and width alone, since the forms round

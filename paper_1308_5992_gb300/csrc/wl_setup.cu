@@ -515,6 +515,9 @@ static int galerkin(Setup &S, int l, const zd *A, zd *Ac) {
   return WL_OK;
 }
 
+// one launch of clusters on 32 x 32, where the device has room for one; else two launches a pass
+static int setup_param(const wl_amg *a, int l) { return a->lev[l].N == 32 && wl::rings64_form(a, l, 1, 1); }
+
 // the setup's relaxations: the FP64 row-block sweeps (wl_rows.cu), whose
 // triangular inverses follow the level's operator; tmp2, which holds nothing
 // across a sweep, takes the inner products
@@ -524,7 +527,7 @@ static int setup_sweeps(Setup &S, int l, zd *V, zd *r, int k, int sweeps) {
   if (!(a->prm.omega > 0.0) || a->lev[l].N < 16) return wl::kaczmarz_sweeps(a, l, WL_FP64, V, r, k, sweeps, S.s);
   WL_TRY(wl::rings64_prepare(a, l, S.stale[l], S.s));
   S.stale[l] = false;
-  return wl::rings64_sweeps(a, l, r, V, V, r, S.S[l].tmp2.p, k, sweeps, a->lev[l].N == 32, S.s);
+  return wl::rings64_sweeps(a, l, r, V, V, r, S.S[l].tmp2.p, k, sweeps, setup_param(a, l), S.s);
 }
 
 // Eq. 3.6: Kaczmarz on A_l v = 0
@@ -782,7 +785,7 @@ static int adaptive_step(Setup &S) {
       if (a->lev[l].N < 16) continue;
       rc = wl::rings64_prepare(a, l, S.stale[l], S.s);
       S.stale[l] = false;
-      a->lev[l].rowtune.push_back(KTune{1, WL_FP64, 6, a->lev[l].N == 32, 0.f});
+      a->lev[l].rowtune.push_back(KTune{1, WL_FP64, 6, setup_param(a, l), 0.f});
     }
   for (int it = 0; it < 2 && !rc; ++it) {
     k_get_col<<<WL_GRID(n2, 256), 256, 0, S.s>>>(Vb, S.S[0].tmp2.as<zd>(), n2, kb, qb, 1.0);

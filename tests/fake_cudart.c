@@ -2,6 +2,7 @@
 // side runs without a GPU: device memory is host memory, launches are logged and compute
 // nothing, copies and fills happen at once.  Memory that was freed is kept aside, so a launch
 // or a captured graph that still points into it is seen (fake_dead), as is a NULL argument.
+// The eigensolver's entries (cuSOLVER) compute nothing either.
 // Allocations of a range of sizes can be made to fail, clusters can be made impossible, and
 // every timed interval is what the test says.
 #include <cuda_runtime_api.h>
@@ -241,4 +242,20 @@ cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *f, const cudaLaun
   (void)f, (void)c;
   *n = clusters;
   return cudaSuccess;
+}
+
+int cusolverDnCreate(void **h) { *h = get(1); return 0; }
+int cusolverDnDestroy(void *h) { (void)h; return 0; }
+int cusolverDnSetStream(void *h, cudaStream_t s) { (void)h, (void)s; return 0; }
+int cusolverDnZhegvd_bufferSize(void *h, int t, int z, int u, int n, const void *A, int la, const void *B, int lb,
+                                const double *W, int *lwork) {
+  (void)h, (void)t, (void)z, (void)u, (void)n, (void)A, (void)la, (void)B, (void)lb, (void)W;
+  *lwork = 1;
+  return 0;
+}
+int cusolverDnZhegvd(void *h, int t, int z, int u, int n, void *A, int la, void *B, int lb, double *W, void *work, int lwork,
+                     int *info) {
+  (void)h, (void)t, (void)z, (void)u, (void)n, (void)A, (void)la, (void)B, (void)lb, (void)W, (void)work, (void)lwork;
+  *info = 0;
+  return 0;
 }

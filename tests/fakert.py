@@ -58,9 +58,18 @@ class Hier:
                   [np.zeros((n * n // 2, 2, 4)) for n in Nl[:-1]], [np.zeros((n * n // 2, 9, 2, 2)) for n in Nl[1:]])
         self.op, self.amg = C.c_void_p(), C.c_void_p()
         self.ok(self.lib.wilson_create(C.c_void_p(U.ctypes.data), Nl[0], 0.1, None, C.byref(self.op)))
-        self.prm = W.amg_params_default(zero_guess=1, **params)
+        self.prm = W.amg_params_default(zero_guess=1, levels=len(Nl), block=[a // b for a, b in zip(Nl, Nl[1:])],
+                                        **params)
         self.ok(self.lib.amg_import(self.op, path.encode(), C.byref(self.prm), C.byref(self.amg)))
         self.buf = np.zeros(64 * 2 * Nl[0] * Nl[0], np.complex128)
+
+    def setup(self):
+        """amg_setup on the same operator (its hierarchy is given back at once)"""
+        out = C.c_void_p()
+        rc = self.lib.amg_setup(self.op, C.byref(self.prm), C.byref(out))
+        if rc == 0:
+            self.lib.amg_destroy(out)
+        return rc
 
     def ok(self, rc):
         assert rc == 0, (rc, self.lib.wl_last_error())

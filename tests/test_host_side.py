@@ -155,3 +155,28 @@ assert "k_ring_dots" not in F.fake_captured().decode() and F.fake_dead() == 0
 print("ok")
 """)
     assert "ok" in out
+
+
+@pytest.mark.parametrize("clusters", [4, 0])
+def test_clusters_are_used_where_the_device_holds_them(clusters):
+    """A device that cannot hold the kernels' clusters (a partition, say) gets the two-launch form,
+    in cycles, in the setup and where a form is named."""
+    out = run("""
+F = fake()
+F.fake_clusters(%d)
+F.fake_times(1e4, -1.0)
+h = Hier([128, 64, 32, 16], fgmres_m=1)
+for nrhs in (1, 3, 5, 9):
+    h.ok(h.cycle(nrhs, 0))
+    names = F.fake_captured().decode()
+    assert ("k_ring64_cluster" in names or "k_ring_pass" in names) == (%d > 0), names
+    for l, param in ((1, 1), (2, 1), (0, 2)):
+        rc = h.lib.amg_kaczmarz_form(h.amg, l, h.v, h.v, 1, 1, 0, 6, param)
+        assert rc == (0 if %d else h.W.WL_EINVAL), (rc, l, param)
+F.fake_clear()
+h.ok(h.setup())
+names = F.fake_launched().decode()
+assert ("k_ring64_cluster" in names) == (%d > 0) and "k_ring_dots" in names
+print("ok")
+""" % ((clusters,) * 4))
+    assert "ok" in out
