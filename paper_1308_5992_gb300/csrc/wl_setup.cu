@@ -518,15 +518,24 @@ static int galerkin(Setup &S, int l, const zd *A, zd *Ac) {
 // one launch of clusters on 32 x 32, where the device has room for one; else two launches a pass
 static int setup_param(const wl_amg *a, int l) { return a->lev[l].N == 32 && wl::rings64_form(a, l, 1, 1); }
 
+// the triangular inverses of a level's row-block sweeps; *ok = false: no memory for
+// them, so the other sweeps run, as in a solve
+static int setup_rows(Setup &S, int l, bool *ok) {
+  int rc = wl::rings64_prepare(S.a, l, S.stale[l], S.s);
+  *ok = rc == WL_OK;
+  if (*ok) S.stale[l] = false;
+  return rc == WL_OOM ? WL_OK : rc;
+}
+
 // the setup's relaxations: the FP64 row-block sweeps (wl_rows.cu), whose
 // triangular inverses follow the level's operator; tmp2, which holds nothing
 // across a sweep, takes the inner products
 static int setup_sweeps(Setup &S, int l, zd *V, zd *r, int k, int sweeps) {
   wl_amg *a = S.a;
   if (sweeps <= 0) return WL_OK;
-  if (!(a->prm.omega > 0.0) || a->lev[l].N < 16) return wl::kaczmarz_sweeps(a, l, WL_FP64, V, r, k, sweeps, S.s);
-  WL_TRY(wl::rings64_prepare(a, l, S.stale[l], S.s));
-  S.stale[l] = false;
+  bool rows = a->prm.omega > 0.0 && a->lev[l].N >= 16;
+  if (rows) WL_TRY(setup_rows(S, l, &rows));
+  if (!rows) return wl::kaczmarz_sweeps(a, l, WL_FP64, V, r, k, sweeps, S.s);
   return wl::rings64_sweeps(a, l, r, V, V, r, S.S[l].tmp2.p, k, sweeps, setup_param(a, l), S.s);
 }
 
@@ -783,9 +792,9 @@ static int adaptive_step(Setup &S) {
   if (a->prm.omega > 0.0)
     for (int l = 0; l < a->L - 1 && !rc; ++l) {
       if (a->lev[l].N < 16) continue;
-      rc = wl::rings64_prepare(a, l, S.stale[l], S.s);
-      S.stale[l] = false;
-      a->lev[l].rowtune.push_back(KTune{1, WL_FP64, 6, setup_param(a, l), 0.f});
+      bool rows;
+      rc = setup_rows(S, l, &rows);
+      if (rows) a->lev[l].rowtune.push_back(KTune{1, WL_FP64, 6, setup_param(a, l), 0.f});
     }
   for (int it = 0; it < 2 && !rc; ++it) {
     k_get_col<<<WL_GRID(n2, 256), 256, 0, S.s>>>(Vb, S.S[0].tmp2.as<zd>(), n2, kb, qb, 1.0);

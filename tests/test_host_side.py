@@ -180,3 +180,20 @@ assert ("k_ring64_cluster" in names) == (%d > 0) and "k_ring_dots" in names
 print("ok")
 """ % ((clusters,) * 4))
     assert "ok" in out
+
+
+@pytest.mark.parametrize("level,coarsest", [(0, 8), (1, 16), (2, 16)])  # no other buffer of that size
+def test_setup_without_memory_for_the_row_block_forms(level, coarsest):
+    """amg_setup does with the other sweeps on a level whose triangular inverses find no memory."""
+    out = run("""
+F = fake()
+h = Hier([128, 64, 32, %d], fgmres_m=1)
+n = h.Nl[%d] ** 2 // 2
+F.fake_fail(n * 384, n * 384, 0, 1000)
+F.fake_clear()
+h.ok(h.setup())
+names = F.fake_launched().decode()
+assert "k_ring" in names and "k_kacz" in names and F.fake_dead() == 0, F.fake_dead_what()
+print("ok")
+""" % (coarsest, level))
+    assert "ok" in out
