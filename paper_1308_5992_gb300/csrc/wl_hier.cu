@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <string>
 #include <vector>
 
 #include "wl_common.cuh"
@@ -275,12 +276,18 @@ static void release_graphs(wl_amg *a) {
   a->graphs.clear();
 }
 
-int ensure_workspace(wl_amg *a, int nrhs, int prec) {
-  (void)prec;
-  if (nrhs <= a->cap) return WL_OK;
-  cudaStreamSynchronize(a->op->stream);
-  release_graphs(a);
-  int cap = std::max(nrhs, a->cap);
+static void release_workspace(wl_amg *a) {
+  for (int l = 0; l < a->L; ++l) {
+    Level &L = a->lev[l];
+    for (DBuf *b : {&L.x, &L.r, &L.f, &L.t}) b->release();
+  }
+  for (DBuf *b : {&a->V, &a->Z, &a->w, &a->bh, &a->xh, &a->rr, &a->red, &a->small}) b->release();
+  if (a->h_small) cudaFreeHost(a->h_small);
+  a->h_small = nullptr;
+  a->cap = 0;
+}
+
+static int alloc_workspace(wl_amg *a, int cap) {
   for (int l = 0; l < a->L; ++l) {
     Level &L = a->lev[l];
     size_t vb = sizeof(zd) * (size_t)L.n * 2 * cap;
@@ -310,6 +317,23 @@ int ensure_workspace(wl_amg *a, int nrhs, int prec) {
   WL_CUDA(cudaMallocHost(&a->h_small, a->slots_at + sizeof(int) * 4 * 32));
   a->cap = cap;
   return WL_OK;
+}
+
+int ensure_workspace(wl_amg *a, int nrhs, int prec) {
+  (void)prec;
+  if (nrhs <= a->cap) return WL_OK;
+  cudaStreamSynchronize(a->op->stream);
+  release_graphs(a);
+  const int old = a->cap;
+  a->cap = 0;  // until every buffer is there
+  int rc = alloc_workspace(a, nrhs);
+  if (rc) {  // back to the width that fitted: the calls (and the server) of that width go on
+    const std::string err = wl_last_error();
+    release_workspace(a);
+    if (old && alloc_workspace(a, old)) release_workspace(a);
+    wl_set_error("%s", err.c_str());
+  }
+  return rc;
 }
 
 // allocate the level structures for sizes Nl and copy P / coarse stencils
@@ -409,24 +433,12 @@ void amg_free(wl_amg *a) {
       o->P.release();
       o->rows.release();
     }
-    L.x.release();
-    L.r.release();
-    L.f.release();
-    L.t.release();
   }
+  release_workspace(a);
   a->Ainv.release();
   a->Ainv32.release();
-  a->V.release();
-  a->Z.release();
-  a->w.release();
-  a->bh.release();
-  a->xh.release();
-  a->rr.release();
   a->sb.release();
   a->sx.release();
-  a->red.release();
-  a->small.release();
-  if (a->h_small) cudaFreeHost(a->h_small);
   for (cudaEvent_t ev : a->lag_ev)
     if (ev) cudaEventDestroy(ev);
   wl_op *op = a->op;

@@ -197,3 +197,30 @@ assert "k_ring" in names and "k_kacz" in names and F.fake_dead() == 0, F.fake_de
 print("ok")
 """ % (coarsest, level))
     assert "ok" in out
+
+
+@pytest.mark.parametrize("at", [0, 3, 8, 17])
+def test_no_memory_for_a_wider_batch(at):
+    """A batch whose workspace does not fit is refused with WL_OOM at whichever buffer; the widths
+    before it, and a server that holds the hierarchy, go on."""
+    out = run("""
+F = fake()
+h = Hier([128, 64, 32, 16], fgmres_m=1)
+h.ok(h.cycle(9, 0))
+for prec in (0, 1):
+    F.fake_fail(40 * 16 * 2, 1 << 40, %d, 1)  # one of the buffers that grow
+    assert h.cycle(40, prec) == h.W.WL_OOM
+    assert b"failed" in h.lib.wl_last_error()
+    F.fake_fail(1, 0, 0, 0)
+    h.ok(h.cycle(9, prec))
+    h.ok(h.cycle(4, prec))
+    assert F.fake_dead() == 0, F.fake_dead_what()
+h.ok(h.cycle(40, 0))
+F.fake_fail(1, 1 << 40, 0, 1 << 30)  # no memory at all: refused until there is some
+assert h.cycle(50, 0) == h.W.WL_OOM and h.cycle(9, 0) == h.W.WL_OOM
+F.fake_fail(1, 0, 0, 0)
+h.ok(h.cycle(9, 0))
+assert F.fake_dead() == 0, F.fake_dead_what()
+print("ok")
+""" % at)
+    assert "ok" in out
