@@ -404,6 +404,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mb, uint32_t parity, unsigned
   }
 }
 
+// for one thread of a block whose wait ran out: another bounded wait (one second each) for
+// the copies that complete on phase `parity` of n mbarriers, so that none lands in shared
+// memory that the block has given back.  Not inlined: in k_kacz_rows it took 0.7 % of a
+// 512x512 solve with one right-hand side by its mere presence
+static __device__ __noinline__ void mbar_drain(const uint64_t *mbar, int n, uint32_t parity) {
+  for (int i = 0; i < n; ++i) mbar_wait(smem_u32(mbar + i), parity, 1000000000ull);
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t mb, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mb), "r"(count) : "memory");
 }

@@ -352,7 +352,10 @@ __global__ void __launch_bounds__(256) k_kacz_block(Geo g, int sweeps, int RC, c
   }
   if constexpr (STAGE) {
     if (!__syncthreads_and(mbar_wait(smem_u32(mbar), 0, 1000000000ull))) {
-      if (tid == 0) atomicExch(&g_tile_timeout, 1);
+      if (tid == 0) {
+        mbar_drain(mbar, 1, 0);
+        atomicExch(&g_tile_timeout, 1);
+      }
       return;
     }
   }
@@ -889,7 +892,10 @@ __global__ void __launch_bounds__(4 * R / RPT) k_kacz_tile_p(Geo g, int tc, cons
     }
     __syncthreads();
     if (!__syncthreads_and(mbar_wait(smem_u32(&mbar[b]), (uint32_t)((i >> 1) & 1), 1000000000ull))) {
-      if (tid == 0) atomicExch(&g_tile_timeout, 1);
+      if (tid == 0) {
+        mbar_drain(&mbar[b], 1, (uint32_t)((i >> 1) & 1));
+        atomicExch(&g_tile_timeout, 1);
+      }
       break;
     }
     if (w + (int)gridDim.x < nitems) fetch(w + gridDim.x, b ^ 1);  // that buffer was freed after item i - 1

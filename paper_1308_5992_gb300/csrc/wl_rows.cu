@@ -179,7 +179,7 @@ __device__ __forceinline__ float2 rb_shfl_xor1(float2 v) {
 // FMAs on (re, im) pairs as they lie in memory: sum (a.re x.re, a.im x.im) and
 // sum (a.re x.im, a.im x.re), combined once per sum.  The tile's packed rows
 // arrive as one bulk copy per row step, all four issued at the start (bounded
-// waits; on a timeout *timeout gets 1 and nothing is written).  x and r are not
+// waits; on a timeout *timeout gets 1, r is not written and x may be partly). x and r are not
 // declared restrict: their loads have to stay after griddepcontrol.wait.
 template <typename S, int R, int RPT>
 __global__ void __launch_bounds__(32 * R / RPT, RPT == 1 ? 16 / R : 0) k_kacz_rows(Geo g, int tc, const unsigned char *__restrict__ pk,
@@ -339,7 +339,10 @@ __global__ void __launch_bounds__(32 * R / RPT, RPT == 1 ? 16 / R : 0) k_kacz_ro
     __syncwarp();
   }
   if (!__syncthreads_and(ok)) {
-    if (tid == 0) atomicExch(timeout, 1);
+    if (tid == 0) {
+      mbar_drain(mbar, 4, 0);
+      atomicExch(timeout, 1);
+    }
     return;
   }
 #pragma unroll
@@ -596,7 +599,10 @@ __global__ void __launch_bounds__(N *N / 8) k_kacz_rings(Geo g, int sweeps, cons
     }
   }
   if (!__syncthreads_and(ok)) {
-    if (tid == 0) atomicExch(timeout, 1);
+    if (tid == 0) {
+      mbar_drain(mbar, 4, 0);
+      atomicExch(timeout, 1);
+    }
     return;
   }
   float2 *ro = (float2 *)r, *xo = (float2 *)x;
