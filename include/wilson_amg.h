@@ -229,7 +229,7 @@ int amg_prolong(wl_amg *amg, int level, const void *e, void *x, int nrhs, int pr
 /* x = A_L^{-1} f on the coarsest level (FP64 inverse). */
 int amg_coarsest(wl_amg *amg, const void *f, void *x, int nrhs);
 /* One preconditioning cycle x = M(f) on level 0 from x = 0 (the
- * configured V or W cycle, nu_pre / nu_post sweeps). */
+ * configured V or W cycle, nu_pre / nu_post sweeps).  WL_TIMEOUT: x is not valid. */
 int amg_cycle(wl_amg *amg, const void *f, void *x, int nrhs, int prec);
 /* FGMRES on Dhat x = bhat (level-0 vectors, x = initial guess); info host
  * array [nrhs].  Return values and per-right-hand-side status as for
@@ -247,7 +247,7 @@ int amg_fgmres(wl_amg *amg, const void *bhat, void *x, int nrhs, double tol, wl_
  * iteration.  A right-hand side whose error norm overflows (a divergent
  * cycle) stops there, keeping the ratio of its last two finite norms.
  * Returns WL_OK if every right-hand side met tol, WL_NOT_CONVERGED
- * otherwise; WL_EINVAL for nrhs outside 1..256, tol < 0 or maxit < 1. */
+ * otherwise; WL_EINVAL for nrhs outside 1..256, tol < 0 or maxit < 1; WL_TIMEOUT as amg_solve. */
 int amg_rho(wl_amg *amg, const void *x0, void *x, int nrhs, double tol, int maxit, double *rho, int *iters,
             double *hist);
 

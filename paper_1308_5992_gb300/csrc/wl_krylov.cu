@@ -1150,6 +1150,7 @@ extern "C" int amg_rho(wl_amg *a, const void *x0, void *x, int nrhs, double tol,
   }
   WL_TRY(wl::from_internal(e, (zd *)x, n2, nrhs, WL_FP64, s));
   WL_CUDA(cudaStreamSynchronize(s));
+  if (wl::tile_timeout_take(s)) return WL_TIMEOUT;
   return (left || diverged) ? WL_NOT_CONVERGED : WL_OK;
 }
 

@@ -2194,6 +2194,7 @@ extern "C" int amg_cycle(wl_amg *a, const void *f, void *x, int nrhs, int prec) 
   WL_TRY(wl::cycle_run(a, nrhs, prec, s));
   WL_TRY(wl::from_internal(a->lev[0].x.p, (zd *)x, n2, nrhs, pin, s));
   WL_CUDA(cudaStreamSynchronize(s));
+  if (wl::tile_timeout_take(s)) return WL_TIMEOUT;
   return WL_OK;
 }
 

@@ -5,13 +5,20 @@
 // The eigensolver's entries (cuSOLVER) compute nothing either.
 // Allocations of a range of sizes can be made to fail, clusters can be made impossible, and
 // every timed interval is what the test says.
+#define _GNU_SOURCE
 #include <cuda_runtime_api.h>
+#include <pthread.h>
 #include <stdint.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
 
 typedef struct { char *p; size_t n; int live; } Block;
+// two solve lanes launch from two threads
+static pthread_mutex_t mu = PTHREAD_RECURSIVE_MUTEX_INITIALIZER_NP;
+#define LOCK pthread_mutex_lock(&mu)
+#define UNLOCK pthread_mutex_unlock(&mu)
+
 static Block *blocks;
 static int nblocks, capblocks;
 
@@ -31,16 +38,22 @@ int fake_dead(void) { return dead; }
 const char *fake_dead_what(void) { return dead_what; }
 
 static void *get(size_t n) {
+  LOCK;
   if (nblocks == capblocks) blocks = realloc(blocks, sizeof(Block) * (capblocks = capblocks ? 2 * capblocks : 256));
   blocks[nblocks].p = calloc(1, n + 256);
   blocks[nblocks].n = n;
   blocks[nblocks].live = 1;
-  return blocks[nblocks++].p;
+  void *p = blocks[nblocks++].p;
+  UNLOCK;
+  return p;
 }
 static int state(const void *p) {  // 1 live, 0 freed, -1 not one of ours
+  int s = -1;
+  LOCK;
   for (int i = 0; i < nblocks; ++i)
-    if ((char *)p >= blocks[i].p && (char *)p < blocks[i].p + blocks[i].n) return blocks[i].live;
-  return -1;
+    if ((char *)p >= blocks[i].p && (char *)p < blocks[i].p + blocks[i].n) s = blocks[i].live;
+  UNLOCK;
+  return s;
 }
 
 cudaError_t cudaMalloc(void **p, size_t n) {
@@ -53,8 +66,10 @@ cudaError_t cudaMalloc(void **p, size_t n) {
   return cudaSuccess;
 }
 cudaError_t cudaFree(void *p) {
+  LOCK;
   for (int i = 0; i < nblocks; ++i)
     if (blocks[i].p == p) blocks[i].live = 0;
+  UNLOCK;
   return cudaSuccess;
 }
 cudaError_t cudaMallocHost(void **p, size_t n) { *p = calloc(1, n); return cudaSuccess; }
@@ -79,15 +94,19 @@ static Graph *capturing, last;
 static Graph log_;
 
 static void check(const Node *n) {
+  LOCK;
   for (int i = 0; i < n->np; ++i)
     if (n->p[i] == NULL || state(n->p[i]) == 0) {
       ++dead;
       snprintf(dead_what, sizeof dead_what, "%.200s, pointer %d: %s", n->name, i, n->p[i] ? "freed" : "NULL");
     }
+  UNLOCK;
 }
 static void add(Graph *g, const Node *n) {
+  LOCK;
   if (g->count == g->cap) g->n = realloc(g->n, sizeof(Node) * (g->cap = g->cap ? 2 * g->cap : 64));
   g->n[g->count++] = *n;
+  UNLOCK;
 }
 static cudaError_t launch(const void *fn, void **args, int cluster) {
   Node n;
@@ -136,8 +155,8 @@ void __cudaRegisterFunction(void **h, const char *host, char *dev, const char *n
 void __cudaRegisterVar(void **h, char *host, char *dev, const char *name, int ext, size_t n, int c, int g) {
   (void)h, (void)host, (void)dev, (void)name, (void)ext, (void)n, (void)c, (void)g;
 }
-static struct { dim3 g, b; size_t sm; void *s; } conf[8];
-static int nconf;
+static __thread struct { dim3 g, b; size_t sm; void *s; } conf[8];
+static __thread int nconf;
 unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t sm, void *s) {
   conf[nconf].g = g, conf[nconf].b = b, conf[nconf].sm = sm, conf[nconf++].s = s;
   return 0;

@@ -224,3 +224,19 @@ assert F.fake_dead() == 0, F.fake_dead_what()
 print("ok")
 """ % at)
     assert "ok" in out
+
+
+def test_a_wait_that_ran_out_is_reported():
+    """A cycle whose sweeps gave up on a bounded wait (the flag that their kernels set) is not passed
+    off as valid, by amg_cycle or amg_rho, and the next one is."""
+    out = run("""
+F = fake()
+h = Hier([64, 32, 16], fgmres_m=1, precision=1)
+rho, it = C.c_double(), C.c_int()
+for call in (lambda: h.cycle(1, 1), lambda: h.lib.amg_rho(h.amg, h.v, h.v, 1, 0.5, 1, C.byref(rho), C.byref(it), None)):
+    F.fake_symbol(1)
+    assert call() == h.W.WL_TIMEOUT
+    assert call() in (h.W.WL_OK, h.W.WL_NOT_CONVERGED)
+print("ok")
+""")
+    assert "ok" in out
