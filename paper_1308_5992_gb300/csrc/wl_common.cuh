@@ -335,6 +335,8 @@ int kaczmarz_colour(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int 
 int kaczmarz_tile(wl_amg *a, int l, int prec, void *x, void *r, int nrhs, int tc, cudaStream_t s, int R = 0, int pdl = 0);
 int autotune_sweeps(wl_amg *a, int nrhs, int prec, cudaStream_t s);  // every level but the coarsest
 int tile_timeout_take(cudaStream_t s);  // 1 if a tile launch's bounded wait ran out (flag cleared)
+size_t fg_scalar_bytes(int m, int nrhs);   // wl_amg::small of FGMRES(m) on nrhs right-hand sides
+size_t fg_partial_bytes(int m, int nrhs);  // wl_amg::red
 int *tile_timeout_flag();               // device address of that flag on the current device
 // row-block form of the tile-coloured sweep (wl_rows.cu): FP32 and BF16 cycles
 bool rows_ok(const wl_amg *a, int l, int prec, int nrhs);

@@ -309,8 +309,8 @@ static int alloc_workspace(wl_amg *a, int cap) {
   WL_CUDA(cudaMemsetAsync(a->V.p, 0, vb0 * (m + 1), a->op->stream));
   WL_CUDA(cudaMemsetAsync(a->Z.p, 0, vb0 * m, a->op->stream));
   WL_CUDA(cudaMemsetAsync(a->w.p, 0, vb0, a->op->stream));
-  WL_TRY(a->red.alloc(sizeof(zd) * 1024 * (m + 2) * (size_t)cap));
-  WL_TRY(a->small.alloc(sizeof(zd) * (size_t)cap * 8 * (m + 2) * (m + 2)));
+  WL_TRY(a->red.alloc(fg_partial_bytes(m, cap)));
+  WL_TRY(a->small.alloc(fg_scalar_bytes(m, cap)));
   if (a->h_small) cudaFreeHost(a->h_small);
   a->h_small = nullptr;
   a->slots_at = sizeof(double) * (size_t)cap * 16 + 64;

@@ -45,7 +45,7 @@ struct KS {
   float2 *invdf; // [nrhs] inv as a double-float (hi, lo)
 };
 
-static KS ks_layout(void *base, int m, int nrhs) {
+static KS ks_layout(void *base, int m, int nrhs, size_t *bytes = nullptr) {
   KS k;
   k.m = m;
   k.nrhs = nrhs;
@@ -75,6 +75,7 @@ static KS ks_layout(void *base, int m, int nrhs) {
   k.running = (int *)take(sizeof(int) * 4);
   k.hpd = (float4 *)take(sizeof(float4) * 2 * nrhs * (m + 1));
   k.invdf = (float2 *)take(sizeof(float2) * nrhs);
+  if (bytes) *bytes = (size_t)(p - (char *)base);
   return k;
 }
 
@@ -746,6 +747,7 @@ namespace wl {
 struct RedCfg {
   int R, nt, nblk;
 };
+static constexpr long RED_BLOCKS = 608;  // 4 blocks per SM on 152 SMs
 static RedCfg red_cfg(long E, int R) {
   RedCfg c;
   c.R = R;
@@ -753,8 +755,18 @@ static RedCfg red_cfg(long E, int R) {
   while (R * G * 2 <= 256) G *= 2;
   c.nt = R * G;
   long want = (E + c.nt - 1) / c.nt;
-  c.nblk = (int)std::max(1L, std::min(want, 608L));  // 4 blocks per SM on 152 SMs
+  c.nblk = (int)std::max(1L, std::min(want, RED_BLOCKS));
   return c;
+}
+
+size_t fg_scalar_bytes(int m, int nrhs) {
+  size_t bytes;
+  ks_layout(nullptr, m, nrhs, &bytes);
+  return bytes;
+}
+// a launch's dots: at most KCH complex doubles, or KCH_DF sums of 32 bytes
+size_t fg_partial_bytes(int m, int nrhs) {
+  return RED_BLOCKS * std::max(sizeof(zd) * std::min(m + 1, KCH), 2 * sizeof(float4) * std::min(m + 1, KCH_DF)) * nrhs;
 }
 
 // out[r][k0+k] (=|+=) V_k^H w for k < kc, chunks of KCH

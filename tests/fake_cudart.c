@@ -1,7 +1,8 @@
 // A stand-in for the CUDA runtime (preloaded by tests/fakert.py), so that the library's host
 // side runs without a GPU: device memory is host memory, launches are logged and compute
 // nothing, copies and fills happen at once.  Memory that was freed is kept aside, so a launch
-// or a captured graph that still points into it is seen (fake_dead), as is a NULL argument.
+// or a captured graph that still points into it is seen (fake_dead), as is a NULL argument, a
+// copy or fill beyond an allocation, and a sum's partials for which there is no room.
 // The eigensolver's entries (cuSOLVER) compute nothing either.
 // Allocations of a range of sizes can be made to fail, clusters can be made impossible, and
 // every timed interval is what the test says.
@@ -13,6 +14,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#define GUARD 65536
 typedef struct { char *p; size_t n; int live; } Block;
 // two solve lanes launch from two threads
 static pthread_mutex_t mu = PTHREAD_RECURSIVE_MUTEX_INITIALIZER_NP;
@@ -40,7 +42,7 @@ const char *fake_dead_what(void) { return dead_what; }
 static void *get(size_t n) {
   LOCK;
   if (nblocks == capblocks) blocks = realloc(blocks, sizeof(Block) * (capblocks = capblocks ? 2 * capblocks : 256));
-  blocks[nblocks].p = calloc(1, n + 256);
+  blocks[nblocks].p = calloc(1, n + GUARD);
   blocks[nblocks].n = n;
   blocks[nblocks].live = 1;
   void *p = blocks[nblocks++].p;
@@ -54,6 +56,21 @@ static int state(const void *p) {  // 1 live, 0 freed, -1 not one of ours
     if ((char *)p >= blocks[i].p && (char *)p < blocks[i].p + blocks[i].n) s = blocks[i].live;
   UNLOCK;
   return s;
+}
+
+static size_t room(const void *p) {  // bytes from p to its allocation's end; a host pointer: any
+  size_t r = (size_t)1 << 62;
+  LOCK;
+  for (int i = 0; i < nblocks; ++i)
+    if ((char *)p >= blocks[i].p && (char *)p < blocks[i].p + blocks[i].n + GUARD)
+      r = (char *)p < blocks[i].p + blocks[i].n && blocks[i].live ? blocks[i].p + blocks[i].n - (char *)p : 0;
+  UNLOCK;
+  return r;
+}
+static void need(const void *p, size_t n, const char *what) {
+  if (room(p) >= n) return;
+  ++dead;
+  snprintf(dead_what, sizeof dead_what, "%.200s: %zu bytes, room for %zu", what, n, room(p));
 }
 
 cudaError_t cudaMalloc(void **p, size_t n) {
@@ -108,7 +125,7 @@ static void add(Graph *g, const Node *n) {
   g->n[g->count++] = *n;
   UNLOCK;
 }
-static cudaError_t launch(const void *fn, void **args, int cluster) {
+static cudaError_t launch(const void *fn, void **args, int cluster, unsigned grid) {
   Node n;
   memset(&n, 0, sizeof n);
   n.cluster = cluster;
@@ -119,6 +136,9 @@ static cudaError_t launch(const void *fn, void **args, int cluster) {
       for (int k = 0; w->arg[k] >= 0; ++k) n.p[n.np++] = *(void **)args[w->arg[k]];
       break;
     }
+  const char *t = strstr(n.name, "9k_mdot_dfILi"), *u = strstr(n.name, "6k_mdotI");
+  if (t) need(*(void **)args[5], 32ul * atoi(t + 13) * grid * *(int *)args[4], "k_mdot_df");
+  if (u) need(*(void **)args[5], 16ul * atoi(strstr(u, "Li") + 2) * grid * *(int *)args[4], "k_mdot");
   if (cluster && !clusters) return cudaErrorLaunchOutOfResources;
   if (capturing) {
     add(capturing, &n);
@@ -168,13 +188,13 @@ cudaError_t __cudaPopCallConfiguration(dim3 *g, dim3 *b, size_t *sm, void *s) {
 }
 cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *fn) { *k = (cudaKernel_t)fn; return cudaSuccess; }
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void **args, size_t sm, cudaStream_t s) {
-  (void)g, (void)b, (void)sm, (void)s;
-  return launch((const void *)k, args, 0);
+  (void)b, (void)sm, (void)s;
+  return launch((const void *)k, args, 0, g.x);
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *fn, void **args) {
   int cl = 0;
   for (unsigned i = 0; i < c->numAttrs; ++i) cl |= c->attrs[i].id == cudaLaunchAttributeClusterDimension;
-  return launch(fn, args, cl);
+  return launch(fn, args, cl, c->gridDim.x);
 }
 
 // ------------------------------------------------------- graphs and streams
@@ -218,13 +238,19 @@ cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t a, cudaEvent_t b) {
 }
 
 // ------------------------------------------------------------------- copies
-cudaError_t cudaMemcpy(void *d, const void *s, size_t n, enum cudaMemcpyKind k) { (void)k; memmove(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemcpy(void *d, const void *s, size_t n, enum cudaMemcpyKind k) {
+  (void)k;
+  need(d, n, "copy to"), need(s, n, "copy from");
+  memmove(d, s, n);
+  return cudaSuccess;
+}
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, enum cudaMemcpyKind k, cudaStream_t st) {
   (void)st;
   return capturing ? cudaSuccess : cudaMemcpy(d, s, n, k);
 }
 cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t s) {
   (void)s;
+  need(d, n, "fill");
   if (!capturing) memset(d, v, n);
   return cudaSuccess;
 }

@@ -71,6 +71,10 @@ class Hier:
             self.lib.amg_destroy(out)
         return rc
 
+    def close(self):
+        self.lib.amg_destroy(self.amg)
+        self.lib.wl_destroy(self.op)
+
     def ok(self, rc):
         assert rc == 0, (rc, self.lib.wl_last_error())
 

@@ -240,3 +240,23 @@ for call in (lambda: h.cycle(1, 1), lambda: h.lib.amg_rho(h.amg, h.v, h.v, 1, 0.
 print("ok")
 """)
     assert "ok" in out
+
+
+@pytest.mark.parametrize("m", [1, 2, 4, 5, 6, 7, 8, 11, 12, 32])
+def test_krylov_workspace_holds_every_restart_length(m):
+    """FGMRES(m) with few right-hand sides: the solver's scalars and the partial sums of its dot
+    products (FP64 and double-float) lie within their buffers."""
+    out = run("""
+F = fake()
+for Nl, params, prec in (([16, 8], {}, 0), ([512, 128, 32, 16], {}, 0),
+                         ([512, 128, 32, 16], dict(precision=1, arnoldi_matvec=1, gs_arith=1), 1)):
+    ms = C.c_double()
+    for nrhs in (1, 7):
+        h = Hier(Nl, fgmres_m=%d, max_restarts=1, **params)
+        assert h.lib.amg_fgmres(h.amg, h.v, h.v, nrhs, 1e-3, None) in (0, 1)
+        h.ok(h.lib.wl_time_kernel(h.amg, h.W.WL_K_GS_DOT, 0, nrhs, prec, 1, C.byref(ms)))
+        assert F.fake_dead() == 0, (Nl, nrhs, F.fake_dead_what())
+        h.close()
+print("ok")
+""" % m)
+    assert "ok" in out
