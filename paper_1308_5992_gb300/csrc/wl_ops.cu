@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(128) k_hop_lanes(Geo g, const zd *__restrict__
                                                    double *__restrict__ out, int nrhs) {
   const long tid = (long)blockIdx.x * 128 + threadIdx.x, it = tid >> 1;
   const int c = (int)tid & 1, N = g.N;
-  if (it >= (long)g.nsites() * nrhs) return;
+  if (it >= (long)g.nsites() * nrhs) return;  // whole warps: a lattice has a multiple of 128 even sites
   const int h = (int)(it / nrhs), r = (int)(it - (long)h * nrhs);
   const int y = h >> (g.lg - 1), x = ((h & (g.half() - 1)) << 1) | ((y + par_out) & 1);
   zd link[4], v0[4], v1[4];
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(128) k_hop_lanes(Geo g, const zd *__restrict__
     if (mu == 0) {
       o1 = fwd ? o1 - p : o1 + p;
     } else {  // -+ i (l w): its component c is +- the other component of l w
-      const double q = __shfl_xor_sync(__activemask(), p, 1);
+      const double q = __shfl_xor_sync(0xffffffffu, p, 1);
       o1 += flip64(q, (c == 0) != fwd);
     }
   }

@@ -94,3 +94,19 @@ def test_pinned_cycle_forms_give_the_same_bits(c2, prec, order):
             assert float((cycle(c, f, prec) - x).abs().max() / x.abs().max()) <= 1e-12, param
             c.close()
     a.close()
+
+
+@pytest.mark.parametrize("N,nrhs", [(16, 1), (16, 3), (32, 5)])
+def test_residual_of_small_lattices(O, N, nrhs):
+    """The FP64 residual of few site-vectors (a hop on two lanes each) on the smallest lattices
+    against the oracle's operator; relative to 1e-12 (sums of 10 terms of order one, 1e-15 each)."""
+    U = np.exp(2j * np.pi * np.random.default_rng(5).random((2, N, N)))
+    op = W.wilson_create(T(U), N, 0.3)
+    amg = W.amg_setup(op, W.amg_params_default(zero_guess=1, block=[2], levels=2, k_r=4, k_e=4, max_restarts=1, fgmres_m=1))
+    bh = np.stack([cgauss(750, r, N * N) for r in range(nrhs)])
+    x = torch.zeros_like(T(bh))
+    _, info = W.amg_fgmres(amg, T(bh), x, nrhs, 1e-14)
+    for r in range(nrhs):
+        res = np.linalg.norm(bh[r] - O.dhat_apply(N, U, 0.3, x[r].cpu().numpy())) / np.linalg.norm(bh[r])
+        assert abs(info[r]["true_relres"] - res) <= 1e-12 * res, (r, info[r], res)
+    amg.close()
