@@ -397,8 +397,9 @@ int wl_time_kernel(wl_amg *amg, int kind, int level, int nrhs, int prec, int rep
  * These forms agree bit for bit.  The sweeps of a cycle without a pinned form take the
  * row-block forms instead (the same sweep, rounded differently), by fixed rules on the level's
  * size, nrhs and prec: FP32 or BF16 on 32x32 and 16x16 levels, and on small tile-ordered ones
- * (FP64: 16-colour ones), so that a solve's bits do not depend on measured times.  Where device
- * memory has no room for their constants, these forms run. */
+ * (FP64: 16-colour ones), so that a solve's bits do not depend on measured times.  Their constants
+ * are made on first use and kept: up to 480 bytes a site of such a level in FP32, 336 with BF16
+ * storage, 384 in FP64.  Where device memory has no room for them, forms 0 to 3 run. */
 int amg_sweep_form(wl_amg *amg, int level, int nrhs, int prec, int *form, int *param, float *us);
 /* The form that the sweeps of a cycle take on `level` once a cycle of that width has run: as
  * amg_sweep_form, or a row-block form, 4 to 6 as in amg_kaczmarz_form (*us = 0 for 5 and 6,

@@ -256,7 +256,8 @@ struct LevelOps {
 // (measured) or by the heuristic: form 0 = one launch per colour, 1 = one
 // cooperative launch for all colours (param = blocks), 2 = tile-coloured
 // kernel (param = right-hand-side chunk R | right-hand sides per thread << 8),
-// 3 = block-resident sweeps of a small level (param = right-hand sides per block)
+// 3 = block-resident sweeps of a small level (param = right-hand sides per block),
+// 4 to 6 = the row-block forms of cycles (wl_rows.cu)
 struct KTune {
   int nrhs, prec, form, param;
   float us;  // measured time of one sweep (0 if not measured)

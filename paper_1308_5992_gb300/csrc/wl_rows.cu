@@ -432,8 +432,8 @@ __device__ __forceinline__ float4 rb_cat(float2 a, float2 b) { return make_float
 // written.  Bounded waits as in k_kacz_rows.
 //
 // Bound by shared-memory bandwidth (a pass reads 61 KB) and the chain of a pass.
-// Four sweeps of the 32 x 32 level: 5 right-hand sides with BF16-stored stencil
-// 17.9 us (k_kacz_block 61.7), one FP32 right-hand side 17 us (k_kacz_coop 160).
+// Four sweeps of the 32 x 32 level, back to back: 5 right-hand sides with BF16-stored
+// stencil 20.6 us (k_kacz_block 61.7), one FP32 right-hand side 16.5 us (k_kacz_coop 160).
 template <typename S, int N>
 __global__ void __launch_bounds__(N *N / 8) k_kacz_rings(Geo g, int sweeps, const unsigned char *__restrict__ pk,
                                                          const zf *rin, const zf *xin, zf *x, zf *r, int nrhs,
@@ -666,7 +666,7 @@ __global__ void __launch_bounds__(16 * RBP_CELLS) k_ring64_pack(Geo g, const zd 
 
 // v with its sign flipped where `neg` (on the integer pipe: a negation that is
 // not known at compile time costs an instruction of the FP64 unit, and the
-// update of a pass took 2860 instead of 1580 cycles with them)
+// update of a pass took 2860 instead of 1306 cycles with them)
 __device__ __forceinline__ double rb_flip(double v, bool neg) {
   return __hiloint2double(__double2hiint(v) ^ (neg ? (int)0x80000000 : 0), __double2loint(v));
 }
@@ -823,7 +823,7 @@ __global__ void __launch_bounds__(W *C * 12 / NI) k_ring_update(Geo g, int pass,
 // neighbour's halo holds are stored there as well (distributed shared memory), so
 // that every load is the block's own; a cluster barrier (390 cycles) follows the
 // inner products and another one the update.  16 passes (four sweeps) of the
-// 32 x 32 level with 12 right-hand sides: 60 us, two launches a pass 104 us.
+// 32 x 32 level with 12 right-hand sides: 56 us, two launches a pass 104 us.
 template <int N>
 struct RingCluster {
   static constexpr int NG = N / 8, SEG = 16 / NG, W = N / SEG, H = N == 32 ? 4 : 2;
@@ -1121,7 +1121,8 @@ int rows_candidates(int nrhs, int *out) {
 // the row form (about twice the instructions of k_kacz_tile, a third of its
 // dependent steps) on level 1 the 512x512 step of 64 right-hand sides took
 // 145.0 ms instead of 143.7, although that level's sweep alone takes 21
-// instead of 41.7 us.
+// instead of 41.7 us.  (A batch of 16 to 31 with overlap = 1 is one lane, but of the
+// width that a lane of a split batch has.  FP64 lanes were not measured.)
 bool rows_ok(const wl_amg *a, int l, int prec, int nrhs) {
   // A launch relaxes a quarter of the level's tiles for every right-hand side.  The
   // lines lie where a sweep takes as long as the best tile kernel's.  Tiles x
@@ -1378,7 +1379,8 @@ bool rings64_form(const wl_amg *a, int l, int param, int nrhs) {
 //            8: 35.9 / 51.6 / - / 213, 64: 125 / 249 / - / 211
 //   128x128: 1: 25.7 / - / 22.7 / 78, 2: 29.9 / - / 35.1 / 228, 24: 174 / - / - / 211
 //   256x256: 1: 57 / - / 71 / 192, 4: 126 / - / 244 / 216, 5: 189 / - / - / 220
-// and one right-hand side of 512x512 146 / 623, of 1024x1024 492 / 2195.  Param 0 works on
+// (over four sweeps, 32x32, one right-hand side: 79 / 47 / 58) and one right-hand side of
+// 512x512 146 / 623, of 1024x1024 492 / 2195.  Param 0 works on
 // chunks of 4; it meets the cooperative launch at 2^18 site-vectors (128x128 x 32: 212 / 212,
 // 256x256 x 8: 213 / 213), and where that launch needs a second block on an SM (152 blocks of
 // 2048 site-vectors) again at 3 * 2^17 (128x128 x 48: 308 / 371, 256x256 x 12: 308 / 374,
